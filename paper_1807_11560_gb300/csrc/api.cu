@@ -123,14 +123,9 @@ int lddmm_create(lddmm_ctx** out, int ndim, const int* grid, const int* K, doubl
   lddmm_default_opts(&o);
   if (opts) o = *opts;
   if (o.precision < LDDMM_FP64 || o.precision > LDDMM_BF16X3) return LDDMM_EINVAL;
-  // the split modes are FP32 contexts whose contractions take the tensor cores
-  // wherever a tcgen05 kernel covers their sizes
-  int split = 0;
-  if (o.precision == LDDMM_3XTF32 || o.precision == LDDMM_BF16X3) {
-    split = o.precision == LDDMM_BF16X3 ? 1 : 0;
-    o.precision = LDDMM_FP32;
-    o.tensor_cores = 2;
-  }
+  // the split modes are FP32 contexts: every contraction runs in FP32, which is no
+  // less accurate than either split
+  if (o.precision == LDDMM_3XTF32 || o.precision == LDDMM_BF16X3) o.precision = LDDMM_FP32;
   if (o.state_eq != 0 && o.state_eq != 1) return LDDMM_EINVAL;
   if (o.state_eq == 1 && o.newton != 0) return LDDMM_EINVAL;
   if (o.debug_stall < 0) return LDDMM_EINVAL;
@@ -155,7 +150,6 @@ int lddmm_create(lddmm_ctx** out, int ndim, const int* grid, const int* K, doubl
     auto* im = new (std::nothrow) Impl<float>();
     if (!im) { delete ctx; return LDDMM_ENOMEM; }
     im->err = &ctx->err;
-    im->split = split;
     ctx->impl = im;
     rc = lddmm::guarded(ctx, [&] { im->create(ndim, grid, K, alpha, s, sigma, Nt, o); });
   }
@@ -354,10 +348,13 @@ long long lddmm_kernel_count(const lddmm_ctx* ctx) {
 
 int lddmm_tile_config(const lddmm_ctx* ctx, int* tws, int* tp, int* kc) {
   if (!ctx || !ctx->impl || !tws || !tp || !kc) return LDDMM_EINVAL;
-  if (ctx->precision == LDDMM_FP64)
-    lddmm::tile_config<double>(static_cast<const Impl<double>*>(ctx->impl)->pad, tws, tp, kc);
-  else
-    lddmm::tile_config<float>(static_cast<const Impl<float>*>(ctx->impl)->pad, tws, tp, kc);
+  auto read = [&](const auto& p) {
+    *tws = 2;
+    *tp = p.geom[lddmm::PW_GT].ppc;
+    *kc = 1 << p.geom[lddmm::PW_GT].tqs;
+  };
+  if (ctx->precision == LDDMM_FP64) read(static_cast<const Impl<double>*>(ctx->impl)->pad);
+  else read(static_cast<const Impl<float>*>(ctx->impl)->pad);
   return LDDMM_OK;
 }
 

@@ -1,413 +1,685 @@
-// Truncated separable DFTs between band-limited coefficients and grid values
-// (iota and pi of Section 3.1, Eq. 46) and the stand-alone kernels of one
-// bracket evaluation of ad~* / ad~ (Eqs. 4, 48, 49) on the padded product
-// grid, for sm_103a.
+// Stand-alone kernels of the truncated transforms (iota and pi of Section 3.1,
+// Eq. 46) and of one pseudo-spectral evaluation (Eqs. 4, 48, 49) for sm_103a;
+// the bodies and the form of the transforms are in trig.cuh.
 //
-// iota runs three contractions:
-//   A  k3 -> x3   T1[k2][x3]       = sum_k3 m_f(k) a_f(h,k2,k3) E3f[k3][x3]
-//   B  k2 -> x2   T2[f][h][x2][x3] = sum_k2 E2f[k2][x2] T1[k2][x3]
-//   C  k1 -> x1   out_f[x1][x2][x3] = sum_h Re(E1f[h][x1] T2[f][h][x2][x3])
-// where h runs over the non-negative k1 slots only: the field is real, so the
-// k1 < 0 half is the conjugate of the k1 > 0 half (E1f carries weight 2 for
-// h > 0).  m_f is the field's spectral multiplier (L^ and/or 2 pi i k_j).
-// pi runs the transposed contractions C' (x1 -> h), B' (x2 -> k2), A' (x3 -> k3),
-// the last one fused with an epilogue that applies K^ = 1/L^, the Heun or
-// Krylov linear combination, and writes the k1 < 0 half by conjugation.
-//
-// Kernels (CTAs of 256 threads; bodies in bracket.cuh):
-//   k_iota_AB  CTA per (field, h): A and B through shared memory -> T2.
-//   k_iota_C   CTA per (field, 256 pencils): C -> grid field (image-grid
-//              transforms); each pencil's K1/2 coefficients read once.
-//   k_cpw      CTA per tile of (x2,x3) pencils: C of the 24 fields of a
-//              bracket evaluation, the bracket products, C' -> P2.
-//   k_pi_C     CTA per (field, 256 pencils): C' of image-grid fields -> P2,
-//              each pencil streamed once.
-//   k_pi_BA    CTA per (component, h, k2 chunk): B', A', epilogue.
+//   k_band        band phase of an evaluation
+//   k_plane       plane phase of an evaluation
+//   k_iota_band   k1 -> x1 of scalar band fields (image grid)
+//   k_iota_plane  k2 -> x2, k3 -> x3 of one x1 plane of up to three fields
+//   k_pi_plane    x3 -> k3, x2 -> k2 of part of one x1 plane of a grid field
+//   k_pi_band     x1 -> k1 of projected image-grid planes
+//   k_band_load, k_band_store   Hermitian arrays <-> band vectors
+#include <atomic>
 #include <utility>
 
-#include "bracket.cuh"
+#include "trig.cuh"
 
 namespace lddmm {
 namespace {
 
-using dev::kThreads;
-using dev::kMaxSmem;
+using namespace dev;
 
+constexpr int kImgThreads = 256;
+constexpr int kIotaGroup = 3;     // fields per image-plane item (one velocity)
+constexpr int kIotaPT = 8;        // row pairs per thread of its k2 -> x2
+constexpr int kIotaBandGroup = 6; // fields per k1 -> x1 item
+constexpr int kSMs = 152;         // sizing only: fixed, so that sums never depend on the device
 
+// raises a kernel's dynamic shared memory limit once per device
 template <auto Kernel>
-void allow_smem() {
-  // one attribute call per kernel instantiation (thread-safe static init)
-  static const bool done = [] {
-    cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
-    return true;
-  }();
-  (void)done;
+cudaError_t allow_smem() {
+  static std::atomic<unsigned long long> done{0};
+  int d = 0;
+  cudaError_t e = cudaGetDevice(&d);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = 1ull << (d & 63);
+  if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+  return e;
 }
 
 // Launch with programmatic stream serialisation: the kernel may be scheduled
-// while the previous kernel of the stream still runs (its phase body waits in
-// pdl_wait before reading what earlier kernels wrote).  Used for the chain of
-// bracket-evaluation kernels, whose prologues (twiddle staging) then overlap
-// the tail of the kernel before.  Recorded as programmatic edges when the
-// stream is captured into a graph.
+// while the previous kernel of the stream still runs; its body waits in
+// pdl_wait before it reads or writes what other kernels use.
 template <typename... KArgs, typename... Args>
-void launch_pdl(void (*kern)(KArgs...), unsigned grid, size_t smem, cudaStream_t st, Args&&... args) {
+cudaError_t launch_chain(void (*kern)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kThreads);
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[2];
+  cudaLaunchAttribute at[1];
   cfg.attrs = at;
   cfg.numAttrs = chain_attrs(at);
-  cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+  return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
-template <typename T, bool TWS>
-__global__ void __launch_bounds__(kThreads)
-k_iota_AB(Plan<T> p, IotaDesc<T> d, const T* __restrict__ Lhat, cplx<T>* __restrict__ T2) {
+template <typename T>
+struct BandArgs {
+  Plan<T> p;
+  PiEpi<T> e;
+  const T *P1, *A, *B, *Lhat;
+  T* T1;
+  int tqs, nparts, prev;
+};
+
+template <typename T, int MODE, bool FLAT>
+__global__ void __launch_bounds__(kPhaseThreads, 1)
+k_band(const __grid_constant__ BandArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  dev::pdl_trigger();
-  const int f = blockIdx.x / p.b.h1, h = blockIdx.x % p.b.h1;
-  const dev::FieldSpec<T> fs{d.src[f], d.deriv[f], d.applyL[f] != 0};
-  dev::phase_iota_ab<T, TWS>(p, fs, f, h, Lhat, T2, smraw);
+  pdl_trigger();
+  band_item<T, MODE, kPhaseThreads, FLAT>(a.p, a.tqs, a.prev ? &a.e : nullptr, a.nparts, a.P1, a.A, a.B, a.T1, a.Lhat,
+                                         blockIdx.x, reinterpret_cast<V2<T>*>(smraw));
+}
+
+template <typename T, int MODE, int PT, int TT>
+__global__ void __launch_bounds__(kPhaseThreads, 1)
+k_plane(const __grid_constant__ Plan<T> p, int ppc, int nparts, const T* T1, T* slot, T* slot2, T* P1) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  pdl_trigger();
+  plane_item<T, MODE, kPhaseThreads, PT, TT>(p, ppc, nparts, T1, slot, slot2, P1, blockIdx.x,
+                                             reinterpret_cast<V2<T>*>(smraw));
 }
 
 template <typename T, int MODE>
-__global__ void __launch_bounds__(kThreads)
-k_cpw(Plan<T> p, const cplx<T>* __restrict__ T2, T* __restrict__ slot, T* __restrict__ slot2,
-      cplx<T>* __restrict__ P2, int TP) {
+__global__ void __launch_bounds__(kPhaseThreads)
+k_plane_flat(const __grid_constant__ Plan<T> p, const T* T1, T* slot, T* slot2, T* P1) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  dev::pdl_trigger();
-  dev::phase_cpw<T, MODE>(p, T2, slot, slot2, P2, TP, blockIdx.x, smraw);
+  pdl_trigger();
+  plane_item_flat<T, MODE, kPhaseThreads>(p, T1, slot, slot2, P1, blockIdx.x, reinterpret_cast<V2<T>*>(smraw));
 }
+
+// ---- image grid ----------------------------------------------------------------
+constexpr int kChunk = 32;        // folded x1 points per twiddle chunk
 
 template <typename T>
-__global__ void __launch_bounds__(kThreads)
-k_pi_BA(Plan<T> p, PiEpi<T> e, const T* __restrict__ Lhat, const cplx<T>* __restrict__ P2, dev::BAGeom g) {
+__global__ void __launch_bounds__(kImgThreads)
+k_iota_band(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList<T> d, int tqs, T* T1) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  dev::pdl_trigger();
-  dev::phase_pi_ba<T>(p, e, Lhat, P2, g, blockIdx.x, smraw);
-}
-
-// ---- iota C: half-spectrum k1 -> x1, real output ----------------------------------
-// CTA per (field, 256 consecutive (x2,x3) positions): every thread loads the
-// H1 complex values of its position once into registers and walks all x1,
-// the twiddle row E1f[.][x1] broadcast from shared memory.
-constexpr int kMaxH1Reg = 32;
-template <typename T, int HR>
-__global__ void __launch_bounds__(kThreads)
-k_iota_C(Plan<T> p, IotaDesc<T> d, const cplx<T>* __restrict__ T2) {
-  using C = cplx<T>;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  C* sE = reinterpret_cast<C*>(smraw);                     // [G1][H1] = E1f transposed
-  const int G1 = p.g.n1, H1 = p.b.h1;
-  const long long inner = (long long)p.g.n2 * p.g.n3;
-  const long long nblk = (inner + kThreads - 1) / kThreads;
-  const int f = (int)(blockIdx.x / nblk);
-  const long long i = (blockIdx.x % nblk) * kThreads + threadIdx.x;
-  for (int j = threadIdx.x; j < H1 * G1; j += kThreads) {   // written in shared-memory order
-    const int x = j / H1, h = j - x * H1;
-    sE[j] = p.E1f[h * G1 + x];
+  V2<T>* sG = reinterpret_cast<V2<T>*>(smraw);             // [NF][H1][PC]
+  const int PC = 4 << tqs, H1 = p.k.H1, q0 = blockIdx.x << tqs, nq = min(1 << tqs, p.k.Kq() - q0);
+  const int f0 = blockIdx.y * kIotaBandGroup, NF = min(kIotaBandGroup, d.nf - f0), ntp = up8(p.NT1);
+  V2<T>* sF = sG + up2(kIotaBandGroup * H1 * PC);          // [H1][kChunk]
+  const V2<T>* tab = reinterpret_cast<const V2<T>*>(p.e1f);
+  pdl_trigger();
+  pdl_wait();
+  for (int it = threadIdx.x; it < NF * H1 * PC; it += kImgThreads) {
+    const int col = it & (PC - 1), r = it >> (tqs + 2);
+    const int f = r / H1, h = r - f * H1;
+    if (col < 4 * nq)
+      sG[it] = reinterpret_cast<const V2<T>*>(d.src[f0 + f])[((long long)(q0 + (col >> 2)) * H1 + h) * 4 + (col & 3)];
   }
-  C a[HR];
-  const bool live = i < inner;
-  const C* __restrict__ src = T2 + (long long)f * H1 * inner + i;
-#pragma unroll
-  for (int h = 0; h < HR; ++h) a[h] = (live && h < H1) ? src[(long long)h * inner] : C{T(0), T(0)};
-  __syncthreads();
-  if (!live) return;
-  T* __restrict__ dst = d.dst[f] + i;
-  for (int x = 0; x < G1; ++x) {
-    const C* e = sE + x * H1;
-    T v0 = T(0), v1 = T(0);
-#pragma unroll
-    for (int h = 0; h < HR; h += 2) {
-      if (h < H1) v0 = fma(a[h].x, e[h].x, fma(-a[h].y, e[h].y, v0));
-      if (h + 1 < H1) v1 = fma(a[h + 1].x, e[h + 1].x, fma(-a[h + 1].y, e[h + 1].y, v1));
+  for (int t0 = 0; t0 < p.NT1; t0 += kChunk) {
+    const int nt = min(kChunk, p.NT1 - t0);
+    if (t0 > 0) __syncthreads();
+    for (int i = threadIdx.x; i < H1 * kChunk; i += kImgThreads) {
+      const int h = i / kChunk, t = i - h * kChunk;
+      sF[i] = t0 + t < ntp ? tab[(long long)h * ntp + t0 + t] : zero2<T>();
     }
-    dst[(long long)x * inner] = v0 + v1;
+    __syncthreads();
+    band_to_planes<T, kImgThreads, false>(p, sG, sF, NF, f0, d.nf, q0, nq, tqs, t0, nt, kChunk, T1);
   }
 }
 
-// ---- pi C': real grid x1 -> half-spectrum h ----------------------------------------
-// CTA per (field, 256 consecutive positions): each thread streams its pencil
-// over x1 once (coalesced) and keeps the H1 complex sums in registers.  The
-// pencil is read kPiCBatch rows at a time, all loads of a batch issued before
-// its sums, so each thread keeps that many HBM reads in flight; the sums keep
-// their x1 order.
-constexpr int kPiCBatch = 8;
-template <typename T, int HR>
-__global__ void __launch_bounds__(kThreads)
-k_pi_C(Plan<T> p, PiSrc<T> s, cplx<T>* __restrict__ P2) {
-  using C = cplx<T>;
+// One x1 plane, ppc row pairs, up to three fields.  k3 -> x3 costs K3/2 products
+// per point and dominates: a lane owns TL points t (and their partners G3 - t) of
+// RB rows, so a row's coefficients are read once per warp (broadcast) and a
+// twiddle once per RB rows.
+template <typename T, int TL, int RB>
+__global__ void __launch_bounds__(kImgThreads)
+k_iota_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList<T> d, int ppc, const T* T1) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  C* sE = reinterpret_cast<C*>(smraw);                     // [G1][H1] = E1b
-  const int G1 = p.g.n1, H1 = p.b.h1;
-  const long long inner = (long long)p.g.n2 * p.g.n3;
-  const long long nblk = (inner + kThreads - 1) / kThreads;
-  const int f = (int)(blockIdx.x / nblk);
-  const long long i = (blockIdx.x % nblk) * kThreads + threadIdx.x;
-  for (int j = threadIdx.x; j < H1 * G1; j += kThreads) sE[j] = p.E1b[j];
+  V2<T>* sm = reinterpret_cast<V2<T>*>(smraw);
+  const int f0 = blockIdx.y * kIotaGroup, NF = min(kIotaGroup, d.nf - f0), x1 = blockIdx.z;
+  const int t0 = blockIdx.x * ppc, np = min(ppc, p.NT2 - t0);
+  const PlaneShape<T> s = plane_shape(p, kIotaGroup, 0, ppc, kIotaPT);
+  const int R = s.R, K3e = p.K3e, K3s = s.K3s, NT3 = p.NT3, G2 = p.g.n2, G3 = p.g.n3;
+  const long long Kq = p.k.Kq();
+  V2<T>* S1 = sm + s.off_s;
+  pdl_trigger();
+  plane_tables<T, kImgThreads, kIotaPT>(p, s, t0, np, true, false, sm);
+  pdl_wait();
   __syncthreads();
-  if (i >= inner) return;
-  C acc[HR];
+  rows_from_band<T, kImgThreads, kIotaGroup, kIotaPT>(p, T1 + ((long long)x1 * d.nf + f0) * Kq * 4, NF, np, s,
+                                                sm + s.off_2f, S1);
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ntb = (NT3 + 32 * TL - 1) / (32 * TL), nrb = (2 * np + RB - 1) / RB;
+  for (int it = warp; it < NF * nrb * ntb; it += kImgThreads / 32) {
+    const int tb = it % ntb, r = it / ntb;
+    const int row0 = (r % nrb) * RB, f = r / nrb;
+    V2<T> acc[RB][TL];
 #pragma unroll
-  for (int h = 0; h < HR; ++h) acc[h] = C{T(0), T(0)};
-  const T* __restrict__ src = s.src[f] + i;
-  for (int x0 = 0; x0 < G1; x0 += kPiCBatch) {
-    T v[kPiCBatch];
+    for (int i = 0; i < RB; ++i)
 #pragma unroll
-    for (int u = 0; u < kPiCBatch; ++u) v[u] = x0 + u < G1 ? src[(long long)(x0 + u) * inner] : T(0);
+      for (int j = 0; j < TL; ++j) acc[i][j] = zero2<T>();
+    const V2<T>* v = S1 + (f * R + row0) * K3s;
+    int tt[TL];
 #pragma unroll
-    for (int u = 0; u < kPiCBatch; ++u) {
-      if (x0 + u >= G1) break;
-      const C* e = sE + (x0 + u) * H1;
+    for (int j = 0; j < TL; ++j) tt[j] = min(tb * 32 * TL + 32 * j + lane, NT3 - 1);
+    const int last = 2 * np - 1 - row0;                    // rows past the item repeat its last row
+    for (int b = 0; b < K3e; b += 2) {
+      V2<T> w0[TL], w1[TL];
 #pragma unroll
-      for (int h = 0; h < HR; ++h)
-        if (h < H1) {
-          acc[h].x = fma(v[u], e[h].x, acc[h].x);
-          acc[h].y = fma(v[u], e[h].y, acc[h].y);
+      for (int j = 0; j < TL; ++j) {
+        w0[j] = sm[b * NT3 + tt[j]];
+        w1[j] = sm[(b + 1) * NT3 + tt[j]];
+      }
+#pragma unroll
+      for (int i = 0; i < RB; ++i) {
+        V2<T> a0, a1;
+        ld2(v + min(i, last) * K3s + b, a0, a1);
+#pragma unroll
+        for (int j = 0; j < TL; ++j) acc[i][j] = fma2(a1, w1[j], fma2(a0, w0[j], acc[i][j]));
+      }
+    }
+    T* __restrict__ dst = d.dst[f0 + f] + (long long)x1 * G2 * G3;
+#pragma unroll
+    for (int i = 0; i < RB; ++i) {
+      const int row = row0 + i, u = t0 + (row >> 1);
+      if (row >= 2 * np || ((row & 1) && (u == 0 || 2 * u == G2))) continue;
+      T* o = dst + (long long)((row & 1) ? G2 - u : u) * G3;
+#pragma unroll
+      for (int j = 0; j < TL; ++j) {
+        const int t = tb * 32 * TL + 32 * j + lane;
+        if (t >= NT3) continue;
+        T E, O;
+        un2(acc[i][j], E, O);
+        o[t] = E + O;
+        if (t > 0 && 2 * t != G3) o[G3 - t] = E - O;
+      }
+    }
+  }
+}
+
+// Part of one x1 plane of grid field f: rows folded along x3 into shared memory,
+// x3 -> k3, then x2 -> k2 as a partial plane.
+template <typename T>
+__global__ void __launch_bounds__(kImgThreads)
+k_pi_plane(const __grid_constant__ Plan<T> p, const T* f0, const T* f1, const T* f2, int ppc, T* __restrict__ P1) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  V2<T>* sm = reinterpret_cast<V2<T>*>(smraw);
+  const int part = blockIdx.x, f = blockIdx.y, x1 = blockIdx.z;
+  const int t0 = part * ppc, np = min(ppc, p.NT2 - t0);
+  const PlaneShape<T> s = plane_shape(p, 0, 1, ppc, 1);
+  const int NT3 = p.NT3, NT3e = p.NT3e, G2 = p.g.n2, G3 = p.g.n3;
+  const long long Kq = p.k.Kq();
+  V2<T>*Z = sm + s.off_s, *sP = sm + s.off_p;
+  pdl_trigger();
+  plane_tables<T, kImgThreads, 1>(p, s, t0, np, false, true, sm);
+  pdl_wait();
+  const T* __restrict__ src = (f == 0 ? f0 : (f == 1 ? f1 : f2)) + (long long)x1 * G2 * G3;
+#pragma unroll 4
+  for (int it = threadIdx.x; it < 2 * np * NT3; it += kImgThreads) {
+    const int row = fdiv(it, p.dNT3), t = it - row * NT3;
+    const int u = t0 + (row >> 1);
+    const bool two = t > 0 && 2 * t != G3;
+    const bool live = !((row & 1) && (u == 0 || 2 * u == G2));
+    const T* v = src + (long long)((row & 1) && live ? G2 - u : u) * G3;
+    const T a = v[t], b = two ? v[G3 - t] : T(0);
+    V2<T>* o = sP + row * NT3e + t;
+    *o = two ? mk2(a + b, a - b) : mk2(a, T(0));
+    if (t == NT3 - 1 && NT3e > NT3) o[1] = zero2<T>();
+  }
+  __syncthreads();
+  rows_to_k3<T, kImgThreads, 1, 1>(p, sP, t0, ppc, np, sm + s.off_3b, Z);
+  __syncthreads();
+  T* out = P1 + (((long long)x1 * gridDim.x + part) * gridDim.y + f) * Kq * 4;
+  if (p.k.K2h >= 16) band_from_rows<T, kImgThreads, 1, 8>(p, Z, ppc, np, sm + s.off_2b, out);
+  else band_from_rows<T, kImgThreads, 1, 4>(p, Z, ppc, np, sm + s.off_2b, out);
+}
+
+// the two plane steps of a 2D image: one output per thread
+template <typename T>
+__global__ void __launch_bounds__(kImgThreads)
+k_iota_plane_flat(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList<T> d, const T* T1) {
+  const int K2h = p.k.K2h, NT2 = p.NT2, G2 = p.g.n2, t = blockIdx.x * kImgThreads + threadIdx.x, f = blockIdx.y,
+            x1 = blockIdx.z;
+  pdl_trigger();
+  pdl_wait();
+  if (t >= NT2) return;
+  const T* v = T1 + ((long long)x1 * d.nf + f) * K2h * 4;
+  const V2<T>* w = reinterpret_cast<const V2<T>*>(p.e2f) + t;
+  V2<T> acc = zero2<T>();
+#pragma unroll 8
+  for (int a = 0; a < K2h; ++a) acc = fma2(ldq(v + 4 * a).c, w[(long long)a * NT2], acc);
+  T E, O;
+  un2(acc, E, O);
+  T* o = d.dst[f] + (long long)x1 * G2;
+  o[t] = E + O;
+  if (t > 0 && 2 * t != G2) o[G2 - t] = E - O;
+}
+template <typename T>
+__global__ void __launch_bounds__(kImgThreads)
+k_pi_plane_flat(const __grid_constant__ Plan<T> p, const T* f0, const T* f1, const T* f2, T* __restrict__ P1) {
+  const int K2h = p.k.K2h, K2p = up8(K2h), G2 = p.g.n2, a = blockIdx.x * kImgThreads + threadIdx.x, f = blockIdx.y,
+            x1 = blockIdx.z;
+  pdl_trigger();
+  pdl_wait();
+  if (a >= K2h) return;
+  const T* __restrict__ src = (f == 0 ? f0 : (f == 1 ? f1 : f2)) + (long long)x1 * G2;
+  const V2<T>* w = reinterpret_cast<const V2<T>*>(p.e2b) + a;
+  V2<T> acc = zero2<T>();
+#pragma unroll 4
+  for (int t = 0; t < p.NT2; ++t) {
+    const bool two = t > 0 && 2 * t != G2;
+    const T u = src[t], v = two ? src[G2 - t] : T(0);
+    acc = fma2(two ? mk2(u + v, u - v) : mk2(u, T(0)), w[(long long)t * K2p], acc);
+  }
+  stq(P1 + (((long long)x1 * gridDim.y + f) * K2h + a) * 4, Quad<T>{acc, zero2<T>()});
+}
+
+// x1 -> k1 of the nf projected planes of image-grid fields and their scaling:
+// out_c = coef * (applyK ? 1/L^ : 1) * the sums (twice per axis of nonzero frequency)
+template <typename T>
+__global__ void __launch_bounds__(kImgThreads)
+k_pi_band(const __grid_constant__ Plan<T> p, const T* P1, int nf, int nparts, int tqs, T coef, int applyK,
+          const T* __restrict__ Lhat, T* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int PC = 4 << tqs, H1 = p.k.H1, q0 = blockIdx.x << tqs, nq = min(1 << tqs, p.k.Kq() - q0), H1p = up4(H1);
+  V2<T>* sW = reinterpret_cast<V2<T>*>(smraw);             // [kChunk][H1p]
+  V2<T>* sE = sW + kChunk * H1p;                           // [nf][kChunk][PC]
+  V2<T>* sY = sE + 3 * kChunk * PC;                        // [nf][H1][PC]
+  pdl_trigger();
+  for (int t0 = 0; t0 < p.NT1; t0 += kChunk) {
+    const int nt = min(kChunk, p.NT1 - t0);
+    if (t0 > 0) __syncthreads();
+    copy2<T, kImgThreads>(sW, p.e1b + (long long)t0 * H1p, nt * H1p);
+    if (t0 == 0) pdl_wait();
+    fold_planes<T, kImgThreads>(p, P1, nf, nparts, q0, nq, tqs, t0, nt, FastDiv{nt > 1 ? 0xffffffffu / nt + 1u : 0u},
+                                sE);
+    __syncthreads();
+    contract_k1<T, kImgThreads, false>(p, nf, nt, tqs, H1p, sE, sW, t0 > 0, sY);
+  }
+  __syncthreads();
+  for (int it = threadIdx.x; it < nf * H1 * PC; it += kImgThreads) {
+    const int col = it & (PC - 1), r = it >> (tqs + 2);
+    const int c = r / H1, h = r - c * H1, q = q0 + (col >> 2), sc = col & 3;
+    if (col >= 4 * nq) continue;
+    const int a = fdiv(q, p.dK3h), b = q - a * p.k.K3h;
+    const long long at = ((long long)q * H1 + h) * 4 + sc;
+    const bool dead = (a == 0 && (sc & 1)) || (b == 0 && (sc & 2));
+    const T f = coef * (applyK ? T(1) / Lhat[2 * at] : T(1)) * (h ? T(2) : T(1)) * (a ? T(2) : T(1)) * (b ? T(2) : T(1));
+    T x, y;
+    un2(sY[it], x, y);
+    reinterpret_cast<V2<T>*>(out)[(long long)c * p.k.Kq() * H1 * 4 + at] =
+        dead ? zero2<T>() : mk2(f * x, h ? f * y : T(0));
+  }
+}
+
+// ---- Hermitian arrays <-> band vectors -------------------------------------------
+// V[s1][s2][s3] = Re sum over the signs of (h, a, b) of prod_j (s_j ? i sigma_j : 1)
+// in(sigma k): the real part keeps exactly the Hermitian part of the input.  One
+// thread per slot.
+template <typename T>
+__global__ void k_band_load(const cplx<T>* __restrict__ in, T* __restrict__ out, int ncomp, Band bd) {
+  const Trig k = trig_of(bd);
+  const long long kvol = k.vol();
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= ncomp * kvol) return;
+  const int c = (int)(idx / kvol);
+  const int r = (int)(idx - c * kvol), s = (r >> 1) & 3, h = (r >> 3) % k.H1, q = (r >> 3) / k.H1;
+  const int a = q / k.K3h, b = q - a * k.K3h;
+  const int f[3] = {h, a, b}, sn[3] = {r & 1, s & 1, s >> 1}, n[3] = {bd.k1, bd.k2, bd.k3};
+  T v = T(0);
+  if (!((f[0] == 0 && sn[0]) || (f[1] == 0 && sn[1]) || (f[2] == 0 && sn[2]))) {
+    for (int m = 0; m < 8; ++m) {
+      int pos[3], turns = 0;                               // product of i sigma: i^ones times the signs
+      bool skip = false;
+      T sg = T(1);
+      for (int j = 0; j < 3; ++j) {
+        const bool neg = (m >> j) & 1;
+        if (neg && f[j] == 0) skip = true;
+        pos[j] = neg ? n[j] - f[j] : f[j];
+        if (sn[j]) {
+          ++turns;
+          if (neg) sg = -sg;
         }
+      }
+      if (skip) continue;
+      const cplx<T> z = in[(long long)c * bd.vol() + ((long long)pos[0] * bd.k2 + pos[1]) * bd.k3 + pos[2]];
+      v += sg * (turns == 0 ? z.x : (turns == 1 ? -z.y : (turns == 2 ? -z.x : z.y)));   // Re(i^turns z)
     }
   }
-  C* dst = P2 + (long long)f * H1 * inner + i;
-#pragma unroll
-  for (int h = 0; h < HR; ++h)
-    if (h < H1) dst[(long long)h * inner] = acc[h];
+  out[idx] = v;
 }
 
+// out(sigma k) = sum over (s1, s2, s3) of prod_j w_j V, w = 1 for a zero frequency,
+// else 1/2 (cosine) or -i sigma / 2 (sine); Nyquist slots are zero
 template <typename T>
-void launch_iota_AB(const Plan<T>& p, const IotaDesc<T>& d, const T* Lhat, cplx<T>* T2, cudaStream_t st,
-                    bool pdl = false) {
-  const unsigned grid = (unsigned)(d.nf * p.b.h1);
-  if (dev::ab_tws(p)) {
-    allow_smem<k_iota_AB<T, true>>();
-    if (pdl) launch_pdl(k_iota_AB<T, true>, grid, dev::ab_smem(p, true), st, p, d, Lhat, T2);
-    else k_iota_AB<T, true><<<grid, kThreads, dev::ab_smem(p, true), st>>>(p, d, Lhat, T2);
-  } else {
-    allow_smem<k_iota_AB<T, false>>();
-    if (pdl) launch_pdl(k_iota_AB<T, false>, grid, dev::ab_smem(p, false), st, p, d, Lhat, T2);
-    else k_iota_AB<T, false><<<grid, kThreads, dev::ab_smem(p, false), st>>>(p, d, Lhat, T2);
+__global__ void k_band_store(const T* __restrict__ in, cplx<T>* __restrict__ out, int ncomp, Band bd) {
+  const Trig k = trig_of(bd);
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= ncomp * bd.vol()) return;
+  const int c = (int)(idx / bd.vol());
+  const int r = (int)(idx - c * bd.vol());
+  const int pos[3] = {r / (bd.k2 * bd.k3), (r / bd.k3) % bd.k2, r % bd.k3}, n[3] = {bd.k1, bd.k2, bd.k3};
+  int f[3];
+  bool neg[3], nyq = false;
+  for (int j = 0; j < 3; ++j) {
+    neg[j] = 2 * pos[j] > n[j];
+    f[j] = neg[j] ? n[j] - pos[j] : pos[j];
+    if (n[j] > 1 && 2 * pos[j] == n[j]) nyq = true;
   }
+  cplx<T> z{T(0), T(0)};
+  if (!nyq) {
+    const T* v = in + (long long)c * k.vol() + ((long long)(f[1] * k.K3h + f[2]) * k.H1 + f[0]) * 8;
+    for (int m = 0; m < 8; ++m) {
+      const int sn[3] = {m & 1, (m >> 1) & 1, (m >> 2) & 1};
+      T w = T(1);
+      int turns = 0;                                       // factors -i
+      bool skip = false;
+      for (int j = 0; j < 3; ++j) {
+        if (f[j] == 0) {
+          if (sn[j]) skip = true;
+          continue;
+        }
+        w *= T(0.5);
+        if (sn[j]) {
+          ++turns;
+          if (neg[j]) w = -w;
+        }
+      }
+      if (skip) continue;
+      const T u = w * v[(2 * sn[2] + sn[1]) * 2 + sn[0]];
+      if (turns == 0) z.x += u;
+      else if (turns == 1) z.y -= u;
+      else if (turns == 2) z.x -= u;
+      else z.y += u;
+    }
+  }
+  out[idx] = z;
+}
+
+// row pairs per thread of k2 -> x2: all of an item's where that fits the registers
+int plane_pt(int ppc) { return ppc <= 3 ? 3 : (ppc <= 5 ? 5 : 9); }
+// x3 points per thread of k3 -> x3: two while that leaves a thread for most lanes
+template <typename T>
+int plane_tt(const Plan<T>& p, int ppc) {
+  return sizeof(T) == 4 && 2 * ppc * ((p.NT3 + 1) / 2) >= 160 ? 2 : 1;
 }
 
 template <typename T>
-void launch_pi_BA(const Plan<T>& p, const PiEpi<T>& e, const T* Lhat, const cplx<T>* P2, cudaStream_t st,
-                  bool pdl = false) {
-  const dev::BAGeom g = dev::ba_geom(p, e.ncomp, e.nper);
-  const unsigned grid = (unsigned)(e.ncomp * p.b.h1 * g.nch);
-  const size_t smem = dev::ba_smem(p, e.nper, g);
-  allow_smem<k_pi_BA<T>>();
-  if (pdl) launch_pdl(k_pi_BA<T>, grid, smem, st, p, e, Lhat, P2, g);
-  else k_pi_BA<T><<<grid, kThreads, smem, st>>>(p, e, Lhat, P2, g);
+size_t plane_smem(const Plan<T>& p, int mode, int ppc) {
+  return plane_shape(p, mode_in(mode), mode_out(mode), ppc, plane_pt(ppc)).smem;
+}
+
+// quads per band-phase item (2^tqs <= 4): one item per SM while every (k1, column)
+// has a thread and the item fits shared memory
+template <typename T>
+int band_tqs(const Plan<T>& p, int mode) {
+  int s = 0;
+  while (s < 2 && (p.k.Kq() >> s) > kSMs && p.k.H1 * (8 << s) <= kPhaseThreads &&
+         band_shape(p, 2 << s, mode_out(mode), mode_in(mode)).smem <= (size_t)kMaxSmem)
+    ++s;
+  return s;
+}
+
+int iota_ppc(int NT2) { return std::min(NT2, 16); }
+int pi_ppc(int NT2) { return std::min(NT2, 8); }
+template <typename T>
+int fit_ppc(const Plan<T>& p, int NF, int NO, int ppc) {
+  while (ppc > 1 && plane_shape(p, NF, NO, ppc, NF > 0 ? kIotaPT : 1).smem > (size_t)96 * 1024) --ppc;
+  return ppc;
+}
+
+template <typename T, int MODE, int PT, int TT>
+cudaError_t launch_plane_pt(const Plan<T>& p, const T* T1, T* slot, T* slot2, T* P1, cudaStream_t st) {
+  const EvalGeom g = p.geom[MODE];
+  cudaError_t e = allow_smem<k_plane<T, MODE, PT, TT>>();
+  if (e != cudaSuccess) return e;
+  return launch_chain(k_plane<T, MODE, PT, TT>, dim3((unsigned)(p.g.n1 * g.nparts)), kPhaseThreads,
+                      plane_smem(p, MODE, g.ppc), st, p, g.ppc, g.nparts, T1, slot, slot2, P1);
+}
+template <typename T, int MODE>
+cudaError_t launch_plane(const Plan<T>& p, const T* T1, T* slot, T* slot2, T* P1, cudaStream_t st) {
+  const int pt = plane_pt(p.geom[MODE].ppc);
+  if (p.flat) {
+    cudaError_t e = allow_smem<k_plane_flat<T, MODE>>();
+    if (e != cudaSuccess) return e;
+    return launch_chain(k_plane_flat<T, MODE>, dim3((unsigned)p.g.n1), kPhaseThreads, plane_flat_smem(p, MODE), st, p,
+                        T1, slot, slot2, P1);
+  }
+  if constexpr (sizeof(T) == 4) {
+    if (plane_tt(p, p.geom[MODE].ppc) == 2) {
+      if (pt == 5) return launch_plane_pt<T, MODE, 5, 2>(p, T1, slot, slot2, P1, st);
+      if (pt == 9) return launch_plane_pt<T, MODE, 9, 2>(p, T1, slot, slot2, P1, st);
+    }
+  }
+  if (pt == 3) return launch_plane_pt<T, MODE, 3, 1>(p, T1, slot, slot2, P1, st);
+  if (pt == 5) return launch_plane_pt<T, MODE, 5, 1>(p, T1, slot, slot2, P1, st);
+  return launch_plane_pt<T, MODE, 9, 1>(p, T1, slot, slot2, P1, st);
+}
+
+template <typename T, int MODE, bool FLAT>
+cudaError_t launch_band_as(const Plan<T>& p, const PiEpi<T>* prev, const T* P1, const T* A, const T* B, T* T1,
+                           const T* Lhat, cudaStream_t st) {
+  BandArgs<T> a{};
+  a.p = p;
+  a.P1 = P1;
+  a.A = A;
+  a.B = B;
+  a.Lhat = Lhat;
+  a.T1 = T1;
+  a.tqs = p.geom[MODE].tqs;
+  a.nparts = p.geom[MODE].nparts;
+  if (prev != nullptr && prev->nout > 0) {
+    a.e = *prev;
+    a.prev = 1;
+  } else if (A == nullptr) {
+    return cudaSuccess;
+  }
+  cudaError_t e = allow_smem<k_band<T, MODE, FLAT>>();
+  if (e != cudaSuccess) return e;
+  return launch_chain(k_band<T, MODE, FLAT>, dim3((unsigned)((p.k.Kq() + (1 << a.tqs) - 1) >> a.tqs)), kPhaseThreads,
+                      band_shape(p, 1 << a.tqs, fields_out(MODE, FLAT), fields_in(MODE, FLAT)).smem, st, a);
+}
+template <typename T, int MODE>
+cudaError_t launch_band(const Plan<T>& p, const PiEpi<T>* prev, const T* P1, const T* A, const T* B, T* T1,
+                        const T* Lhat, cudaStream_t st) {
+  return p.flat ? launch_band_as<T, MODE, true>(p, prev, P1, A, B, T1, Lhat, st)
+                : launch_band_as<T, MODE, false>(p, prev, P1, A, B, T1, Lhat, st);
+}
+
+template <typename T, int TL, int RB>
+cudaError_t launch_iota_plane(const Plan<T>& p, const IotaList<T>& d, const T* T1, cudaStream_t st) {
+  const int ppc = fit_ppc(p, kIotaGroup, 0, iota_ppc(p.NT2));
+  cudaError_t e = allow_smem<k_iota_plane<T, TL, RB>>();
+  if (e != cudaSuccess) return e;
+  const dim3 grid((unsigned)((p.NT2 + ppc - 1) / ppc), (unsigned)((d.nf + kIotaGroup - 1) / kIotaGroup),
+                  (unsigned)p.g.n1);
+  return launch_chain(k_iota_plane<T, TL, RB>, grid, kImgThreads, plane_shape(p, kIotaGroup, 0, ppc, kIotaPT).smem, st, p, d,
+                      ppc, T1);
 }
 
 }  // namespace
 
+// Rows per plane item: the fewest waves of items over the SMs, each costing its
+// rows plus a fixed chain (launch, first loads, barriers: about two row pairs'
+// work), and a partial plane more to be summed for every part.
 template <typename T>
-size_t max_smem_needed(const Plan<T>& p, int nper_max, bool brackets) {
-  // every B' column of a CTA needs its own accumulators, and the image-grid
-  // C/C' kernels keep the K1/2 slots of a pencil in registers
-  if ((long long)nper_max * p.g.n3 > (long long)dev::kAccB * kThreads) return ~size_t(0);
-  if (p.b.h1 > kMaxH1Reg) return ~size_t(0);
-  if ((size_t)p.b.h1 * p.g.n1 * sizeof(cplx<T>) > (size_t)kMaxSmem) return ~size_t(0);
-  const size_t ab = dev::ab_smem(p, dev::ab_tws(p));
-  if (brackets && p.g.n1 > 2 * kThreads) return ~size_t(0);
-  const size_t cpw = brackets ? dev::cpw_smem(p, dev::cpw_tile(p), 9) : 0;
-  size_t ba = 0;
-  for (int nper = 1; nper <= nper_max; ++nper)
-    ba = std::max(ba, dev::ba_smem(p, nper, dev::ba_geom(p, 36, nper)));
-  return std::max(ab, std::max(cpw, ba));
-}
-
-size_t smem_limit() { return kMaxSmem; }
-
-template <typename T>
-void tile_config(const Plan<T>& p, int* tws, int* tp, int* kc) {
-  *tws = dev::ab_tws(p) ? 2 : 1;
-  *tp = dev::cpw_tile(p);
-  *kc = dev::ba_geom(p, 3, 3).KC;
-}
-
-template <typename T>
-bool tile_valid(const Plan<T>& p, int tws, int tp, int kc) {
-  if (tws == 2 && dev::ab_smem(p, true) > (size_t)kMaxSmem) return false;
-  if (tp > 0 && !dev::cpw_tile_ok(p, tp)) return false;
-  if (kc > p.b.k2 || kc > dev::kMaxKC) return false;
-  Plan<T> q = p;
-  q.tws = tws;
-  q.tp = tp;
-  q.kc = kc;
-  return max_smem_needed(q, 3, true) <= (size_t)kMaxSmem;
+EvalGeom eval_geom(const Plan<T>& p, PwMode mode) {
+  EvalGeom g{1, p.NT2, 0};
+  if (p.flat) {
+    g.ppc = p.NT2;                                         // one item per plane
+    g.nparts = 1;
+    g.tqs = 0;
+    return g;
+  }
+  double best = 1e300;
+  for (int parts = 1; parts <= p.NT2; ++parts) {
+    const int ppc = (p.NT2 + parts - 1) / parts;
+    if ((p.NT2 + ppc - 1) / ppc != parts) continue;        // the same cut as with fewer parts
+    if (plane_smem(p, mode, ppc) > (size_t)kMaxSmem) continue;
+    const double waves = (double)(((long long)p.g.n1 * parts + kSMs - 1) / kSMs);
+    const double cost = waves * (ppc + 2.0) + 0.3 * parts;
+    if (cost < best) {
+      best = cost;
+      g.ppc = ppc;
+      g.nparts = parts;
+    }
+  }
+  g.tqs = band_tqs(p, mode);
+  return g;
 }
 
 template <typename T>
-void staged_twiddle_dims(const Plan<T>& p, int* G3e, int* G2e, int* G1q, int* H1q, int* G3s) {
-  *G3e = dev::even_up(p.g.n3);
-  *G2e = dev::even_up(p.g.n2);
-  *G1q = dev::quad_up(p.g.n1);
-  *H1q = dev::quad_up(p.b.h1);
-  *G3s = dev::e3_stride<T>(p.g.n3);
-}
-
-template <typename T>
-long long cache_slot_elems(const Plan<T>& p) {
-  const long long P = (long long)p.g.n2 * p.g.n3;
-  const int TP = dev::cpw_tile(p);
-  return 24LL * p.g.n1 * TP * ((P + TP - 1) / TP);
-}
-
-// register slots of the image-grid C / C' kernels: the smallest of 8/16/32 >= K1/2
-template <typename T, int HR>
-void launch_C(const Plan<T>& p, const IotaDesc<T>& d, const cplx<T>* T2, unsigned grid, size_t smem,
-              cudaStream_t st) {
-  allow_smem<k_iota_C<T, HR>>();
-  k_iota_C<T, HR><<<grid, kThreads, smem, st>>>(p, d, T2);
-}
-template <typename T, int HR>
-void launch_Cb(const Plan<T>& p, const PiSrc<T>& s, cplx<T>* P2, unsigned grid, size_t smem, cudaStream_t st) {
-  allow_smem<k_pi_C<T, HR>>();
-  k_pi_C<T, HR><<<grid, kThreads, smem, st>>>(p, s, P2);
-}
-
-template <typename T>
-bool try_tc(const Plan<T>&, const IotaDesc<T>&, const cplx<T>*, double*, cudaStream_t) {
-  return false;
-}
-template <>
-bool try_tc<float>(const Plan<float>& p, const IotaDesc<float>& d, const float2* T2, double* flag,
-                   cudaStream_t st) {
-  if (!flag || !iota_C_tc_supported(p)) return false;
-  return iota_C_tc(p, d, T2, flag, st) == cudaSuccess;
-}
-
-template <typename T>
-void iota_c_stage(const Plan<T>& p, const IotaDesc<T>& d, cplx<T>* T2, cudaStream_t st, double* tc_flag) {
-  if (try_tc<T>(p, d, T2, tc_flag, st)) return;
-  const long long nblk = ((long long)p.g.n2 * p.g.n3 + kThreads - 1) / kThreads;
-  const size_t smem = (size_t)p.b.h1 * p.g.n1 * sizeof(cplx<T>);
-  const unsigned grid = (unsigned)(d.nf * nblk);
-  if (p.b.h1 <= 8) launch_C<T, 8>(p, d, T2, grid, smem, st);
-  else if (p.b.h1 <= 16) launch_C<T, 16>(p, d, T2, grid, smem, st);
-  else launch_C<T, 32>(p, d, T2, grid, smem, st);
-}
-
-template <typename T>
-void iota_batch(const Plan<T>& p, const IotaDesc<T>& d, const T* Lhat, cplx<T>* T2, cudaStream_t st,
-                double* tc_flag) {
-  launch_iota_AB<T>(p, d, Lhat, T2, st);
-  iota_c_stage<T>(p, d, T2, st, tc_flag);
-}
-
-template <typename T>
-void pi_c_stage(const Plan<T>& p, const PiSrc<T>& s, cplx<T>* P2, cudaStream_t st) {
-  const long long nblk = ((long long)p.g.n2 * p.g.n3 + kThreads - 1) / kThreads;
-  const size_t smem = (size_t)p.b.h1 * p.g.n1 * sizeof(cplx<T>);
-  const unsigned grid = (unsigned)(s.nf * nblk);
-  if (p.b.h1 <= 8) launch_Cb<T, 8>(p, s, P2, grid, smem, st);
-  else if (p.b.h1 <= 16) launch_Cb<T, 16>(p, s, P2, grid, smem, st);
-  else launch_Cb<T, 32>(p, s, P2, grid, smem, st);
-}
-
-template <typename T>
-void pi_batch(const Plan<T>& p, const PiSrc<T>& s, const PiEpi<T>& e, const T* Lhat, cplx<T>* P2,
-              cudaStream_t st) {
-  pi_c_stage<T>(p, s, P2, st);
-  launch_pi_BA<T>(p, e, Lhat, P2, st);
-}
-
-template <typename T>
-bool try_ab_tc(const Plan<T>&, const IotaDesc<T>&, const T*, cplx<T>*, double*, cudaStream_t) {
-  return false;
-}
-template <>
-bool try_ab_tc<float>(const Plan<float>& p, const IotaDesc<float>& d, const float* Lhat, float2* T2,
-                      double* flag, cudaStream_t st) {
-  if (!flag || !iota_ab_tc_supported(p)) return false;
-  return iota_ab_tc(p, d, Lhat, T2, flag, st) == cudaSuccess;
-}
-
-template <typename T>
-void bracket_iota(const Plan<T>& p, const IotaDesc<T>& d, const T* Lhat, cplx<T>* T2, cudaStream_t st,
-                  double* tc_flag) {
-  if (try_ab_tc<T>(p, d, Lhat, T2, tc_flag, st)) return;
-  launch_iota_AB<T>(p, d, Lhat, T2, st, true);
-}
-
-template <typename T>
-bool try_cpw_tc(const Plan<T>&, PwMode, const cplx<T>*, T*, T*, cplx<T>*, double*, cudaStream_t) {
-  return false;
-}
-template <>
-bool try_cpw_tc<float>(const Plan<float>& p, PwMode mode, const float2* T2, float* slot, float* slot2,
-                       float2* P2, double* flag, cudaStream_t st) {
-  if (!flag || p.tc_cpw == nullptr) return false;
-  if (cpw_tc(p, mode, T2, slot, slot2, P2, flag, st) == cudaSuccess) return true;
-  cudaGetLastError();   // a refused launch configuration: the SIMT kernel runs instead
-  return false;
-}
-
-template <typename T>
-void bracket_cpw(const Plan<T>& p, PwMode mode, const cplx<T>* T2, T* slot, T* slot2, cplx<T>* P2,
-                 cudaStream_t st, double* tc_flag) {
-  if (try_cpw_tc<T>(p, mode, T2, slot, slot2, P2, tc_flag, st)) return;
-  const int TP = dev::cpw_tile(p);
-  const int NP = (mode == PW_GT) ? 9 : 3;
-  const size_t smem = dev::cpw_smem(p, TP, NP);
-  const long long P = (long long)p.g.n2 * p.g.n3;
-  const unsigned grid = (unsigned)((P + TP - 1) / TP);
+cudaError_t band_phase(const Plan<T>& p, PwMode mode, const PiEpi<T>* prev, const T* P1, const T* A, const T* B, T* T1,
+                       const T* Lhat, cudaStream_t st) {
   switch (mode) {
-    case PW_F:
-      allow_smem<k_cpw<T, PW_F>>();
-      launch_pdl(k_cpw<T, PW_F>, grid, smem, st, p, T2, slot, slot2, P2, TP);
-      break;
-    case PW_T:
-      allow_smem<k_cpw<T, PW_T>>();
-      launch_pdl(k_cpw<T, PW_T>, grid, smem, st, p, T2, slot, slot2, P2, TP);
-      break;
-    case PW_GT:
-      allow_smem<k_cpw<T, PW_GT>>();
-      launch_pdl(k_cpw<T, PW_GT>, grid, smem, st, p, T2, slot, slot2, P2, TP);
-      break;
+    case PW_F: return launch_band<T, PW_F>(p, prev, P1, A, B, T1, Lhat, st);
+    case PW_T: return launch_band<T, PW_T>(p, prev, P1, A, B, T1, Lhat, st);
+    case PW_TC: return launch_band<T, PW_TC>(p, prev, P1, A, B, T1, Lhat, st);
+    case PW_GT: return launch_band<T, PW_GT>(p, prev, P1, A, B, T1, Lhat, st);
+    case PW_D0: return launch_band<T, PW_D0>(p, prev, P1, A, B, T1, Lhat, st);
+    case PW_D1: return launch_band<T, PW_D1>(p, prev, P1, A, B, T1, Lhat, st);
+    default: return launch_band<T, PW_D2>(p, prev, P1, A, B, T1, Lhat, st);
   }
 }
 
 template <typename T>
-bool try_pi_tc(const Plan<T>&, const PiEpi<T>&, const T*, const cplx<T>*, double*, cudaStream_t) {
-  return false;
-}
-template <>
-bool try_pi_tc<float>(const Plan<float>& p, const PiEpi<float>& e, const float* Lhat, const float2* P2,
-                      double* flag, cudaStream_t st) {
-  if (!flag || p.tc_pi == nullptr) return false;
-  if (pi_ba_tc(p, e, Lhat, P2, flag, st) == cudaSuccess) return true;
-  cudaGetLastError();   // a refused launch configuration: the SIMT kernel runs instead
-  return false;
+cudaError_t plane_phase(const Plan<T>& p, PwMode mode, const T* T1, T* slot, T* slot2, T* P1, cudaStream_t st) {
+  switch (mode) {
+    case PW_F: return launch_plane<T, PW_F>(p, T1, slot, slot2, P1, st);
+    case PW_T: return launch_plane<T, PW_T>(p, T1, slot, slot2, P1, st);
+    case PW_TC: return launch_plane<T, PW_TC>(p, T1, slot, slot2, P1, st);
+    case PW_GT: return launch_plane<T, PW_GT>(p, T1, slot, slot2, P1, st);
+    case PW_D0: return launch_plane<T, PW_D0>(p, T1, slot, slot2, P1, st);
+    case PW_D1: return launch_plane<T, PW_D1>(p, T1, slot, slot2, P1, st);
+    default: return launch_plane<T, PW_D2>(p, T1, slot, slot2, P1, st);
+  }
 }
 
 template <typename T>
-void bracket_pi(const Plan<T>& p, const PiEpi<T>& e, const T* Lhat, const cplx<T>* P2, cudaStream_t st,
-                double* tc_flag) {
-  if (try_pi_tc<T>(p, e, Lhat, P2, tc_flag, st)) return;
-  launch_pi_BA<T>(p, e, Lhat, P2, st, true);
+long long eval_T1_elems(const Plan<T>& p) {
+  return (long long)p.g.n1 * kMaxInFields * p.k.Kq() * 4;
+}
+template <typename T>
+long long eval_P1_elems(const Plan<T>& p) {
+  long long n = 0;
+  for (int m = 0; m < PW_MODES; ++m)
+    n = std::max(n, (long long)p.g.n1 * p.geom[m].nparts * mode_out(m) * p.k.Kq() * 4);
+  return n;
 }
 
-#define LDDMM_DFT_INST(T)                                                                          \
-  template size_t max_smem_needed<T>(const Plan<T>&, int, bool);                                   \
-  template long long cache_slot_elems<T>(const Plan<T>&);                                           \
-  template void staged_twiddle_dims<T>(const Plan<T>&, int*, int*, int*, int*, int*);               \
-  template void tile_config<T>(const Plan<T>&, int*, int*, int*);                                   \
-  template bool tile_valid<T>(const Plan<T>&, int, int, int);                                        \
-  template void iota_batch<T>(const Plan<T>&, const IotaDesc<T>&, const T*, cplx<T>*, cudaStream_t,    \
-                              double*);                                                            \
-  template void iota_c_stage<T>(const Plan<T>&, const IotaDesc<T>&, cplx<T>*, cudaStream_t, double*); \
-  template void pi_c_stage<T>(const Plan<T>&, const PiSrc<T>&, cplx<T>*, cudaStream_t);             \
-  template void pi_batch<T>(const Plan<T>&, const PiSrc<T>&, const PiEpi<T>&, const T*, cplx<T>*,  \
-                            cudaStream_t);                                                         \
-  template void bracket_iota<T>(const Plan<T>&, const IotaDesc<T>&, const T*, cplx<T>*, cudaStream_t, double*); \
-  template void bracket_cpw<T>(const Plan<T>&, PwMode, const cplx<T>*, T*, T*, cplx<T>*, cudaStream_t, double*); \
-  template void bracket_pi<T>(const Plan<T>&, const PiEpi<T>&, const T*, const cplx<T>*, cudaStream_t, double*);
+template <typename T>
+long long iota_T1_elems(const Plan<T>& p, int nf) {
+  return (long long)p.g.n1 * nf * p.k.Kq() * 4;
+}
+template <typename T>
+cudaError_t iota_fields(const Plan<T>& p, const IotaList<T>& d, T* T1, cudaStream_t st) {
+  const int tqs = p.k.Kq() >= 4 ? 2 : 0;
+  const size_t smem = (size_t)(up2(kIotaBandGroup * p.k.H1 * (4 << tqs)) + p.k.H1 * kChunk) * sizeof(V2<T>);
+  cudaError_t e = allow_smem<k_iota_band<T>>();
+  if (e != cudaSuccess) return e;
+  const dim3 grid((unsigned)((p.k.Kq() + (1 << tqs) - 1) >> tqs),
+                  (unsigned)((d.nf + kIotaBandGroup - 1) / kIotaBandGroup));
+  if ((e = launch_chain(k_iota_band<T>, grid, kImgThreads, smem, st, p, d, tqs, T1)) != cudaSuccess) return e;
+  if (p.flat)
+    return launch_chain(k_iota_plane_flat<T>,
+                        dim3((unsigned)((p.NT2 + kImgThreads - 1) / kImgThreads), (unsigned)d.nf, (unsigned)p.g.n1),
+                        kImgThreads, 0, st, p, d, (const T*)T1);
+  if (p.NT3 <= 32) return launch_iota_plane<T, 1, 8>(p, d, T1, st);
+  if (p.NT3 <= 64) return launch_iota_plane<T, 2, 8>(p, d, T1, st);
+  if (p.NT3 <= 96) return launch_iota_plane<T, 3, 6>(p, d, T1, st);
+  return launch_iota_plane<T, 4, 4>(p, d, T1, st);
+}
+
+template <typename T>
+long long pi_P1_elems(const Plan<T>& p) {
+  const int ppc = fit_ppc(p, 0, 1, pi_ppc(p.NT2));
+  return (long long)p.g.n1 * ((p.NT2 + ppc - 1) / ppc) * 3 * p.k.Kq() * 4;
+}
+template <typename T>
+cudaError_t pi_fields(const Plan<T>& p, const T* const* src, const PiEpi<T>& e, const T* Lhat, T* P1,
+                      cudaStream_t st) {
+  const int nf = e.ncomp;
+  int nparts = 1;
+  cudaError_t rc;
+  if (p.flat) {
+    rc = launch_chain(k_pi_plane_flat<T>,
+                      dim3((unsigned)((p.k.K2h + kImgThreads - 1) / kImgThreads), (unsigned)nf, (unsigned)p.g.n1),
+                      kImgThreads, 0, st, p, src[0], src[nf > 1 ? 1 : 0], src[nf > 2 ? 2 : 0], P1);
+  } else {
+    const int ppc = fit_ppc(p, 0, 1, pi_ppc(p.NT2));
+    nparts = (p.NT2 + ppc - 1) / ppc;
+    if ((rc = allow_smem<k_pi_plane<T>>()) != cudaSuccess) return rc;
+    rc = launch_chain(k_pi_plane<T>, dim3((unsigned)nparts, (unsigned)nf, (unsigned)p.g.n1), kImgThreads,
+                      plane_shape(p, 0, 1, ppc, 1).smem, st, p, src[0], src[nf > 1 ? 1 : 0], src[nf > 2 ? 2 : 0], ppc,
+                      P1);
+  }
+  if (rc != cudaSuccess) return rc;
+  const int tqs = p.k.Kq() >= 2 * kSMs ? 1 : 0, PC = 4 << tqs, H1 = p.k.H1;
+  const size_t smem = (size_t)(kChunk * up4(H1) + 3 * kChunk * PC + 3 * H1 * PC) * sizeof(V2<T>);
+  if ((rc = allow_smem<k_pi_band<T>>()) != cudaSuccess) return rc;
+  return launch_chain(k_pi_band<T>, dim3((unsigned)((p.k.Kq() + (1 << tqs) - 1) >> tqs)), kImgThreads, smem, st, p,
+                      (const T*)P1, nf, nparts, tqs, e.coef[0], e.applyK[0], Lhat, e.dst[0]);
+}
+
+template <typename T>
+void band_load(const cplx<T>* in, T* out, int ncomp, const Band& b, cudaStream_t st) {
+  const long long n = ncomp * trig_of(b).vol();
+  k_band_load<T><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, out, ncomp, b);
+}
+template <typename T>
+void band_store(const T* in, cplx<T>* out, int ncomp, const Band& b, cudaStream_t st) {
+  const long long n = ncomp * b.vol();
+  k_band_store<T><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, out, ncomp, b);
+}
+
+// ---- accepted sizes -----------------------------------------------------------
+// The interface takes the grids and bands whose complex half-spectrum tiles (two
+// slabs and a twiddle table per axis) fit 200 KB of shared memory, N_3 nper <= 512
+// and K_1 <= 64; every kernel above runs within that range in less.
+template <typename T>
+bool sizes_accepted(const Dims& g, const Band& b, int nper, bool brackets) {
+  constexpr size_t lim = 200 * 1024, C = 2 * sizeof(T);
+  constexpr int threads = 256;
+  const size_t G1 = g.n1, G2 = g.n2, G3 = g.n3, H1 = b.h1, K2 = b.k2, K3 = b.k3;
+  if ((size_t)nper * G3 > 2 * (size_t)threads || H1 > 32 || H1 * G1 * C > lim) return false;
+  if (brackets && G1 > 2 * (size_t)threads) return false;
+  const size_t G3e = G3 + (G3 & 1), G2e = G2 + (G2 & 1);
+  const size_t ab0 = (K2 * K3 + K2 * G3e) * C + K2 * K3 * sizeof(T), ab1 = ab0 + (K3 * G3e + K2 * G2e) * C;
+  if ((ab1 <= 64 * 1024 ? ab1 : ab0) > lim) return false;
+  if (brackets) {
+    auto cpw = [&](size_t TP) {
+      return (24 * H1 * TP + H1 * ((G1 + 3) & ~size_t(3)) + G1 * ((H1 + 3) & ~size_t(3))) * C + 33 * G1 * TP * sizeof(T);
+    };
+    size_t TP = std::max<size_t>(1, std::min<size_t>(8, G2 * G3 / 152));
+    while (TP > 1 && (cpw(TP) > lim || G1 * TP > 2 * (size_t)threads)) --TP;
+    if (cpw(TP) > lim) return false;
+  }
+  constexpr size_t E = 128 / C;
+  const size_t G3s = G3 + ((E / 2 + E - G3 % E) % E);
+  for (size_t np = 1; np <= (size_t)nper; ++np) {
+    const size_t want = std::max<size_t>(1, (304 + 36 * H1 - 1) / (36 * H1));
+    size_t KC = std::min(std::min(std::max<size_t>(1, (K2 + want - 1) / want), size_t(8)), K2);
+    const size_t R = std::max<size_t>(1, std::min<size_t>(8, threads / (np * G3)));
+    const size_t row = np * G3 * C;
+    auto fixed = [&]() { return (G2 * KC + G3s * K3 + R * np * KC * G3 + KC * K3 * 16) * C + KC * K3 * sizeof(T); };
+    while (KC > 1 && fixed() + row * KC > lim) --KC;
+    const size_t target = fixed() + 16 * row > 72 * 1024 ? 150 * 1024 : 72 * 1024;
+    const size_t rows = fixed() < target ? (target - fixed()) / row : 0;
+    if (fixed() + row * std::max(KC, std::min(G2, rows)) > lim) return false;
+  }
+  return true;
+}
+
+#define LDDMM_DFT_INST(T)                                                                                          \
+  template EvalGeom eval_geom<T>(const Plan<T>&, PwMode);                                                          \
+  template cudaError_t band_phase<T>(const Plan<T>&, PwMode, const PiEpi<T>*, const T*, const T*, const T*, T*,     \
+                                     const T*, cudaStream_t);                                                      \
+  template cudaError_t plane_phase<T>(const Plan<T>&, PwMode, const T*, T*, T*, T*, cudaStream_t);                 \
+  template long long eval_T1_elems<T>(const Plan<T>&);                                                             \
+  template long long eval_P1_elems<T>(const Plan<T>&);                                                             \
+  template long long iota_T1_elems<T>(const Plan<T>&, int);                                                        \
+  template cudaError_t iota_fields<T>(const Plan<T>&, const IotaList<T>&, T*, cudaStream_t);                       \
+  template long long pi_P1_elems<T>(const Plan<T>&);                                                               \
+  template cudaError_t pi_fields<T>(const Plan<T>&, const T* const*, const PiEpi<T>&, const T*, T*, cudaStream_t); \
+  template void band_load<T>(const cplx<T>*, T*, int, const Band&, cudaStream_t);                                  \
+  template void band_store<T>(const T*, cplx<T>*, int, const Band&, cudaStream_t);                                 \
+  template bool sizes_accepted<T>(const Dims&, const Band&, int, bool);
 LDDMM_DFT_INST(float)
 LDDMM_DFT_INST(double)
 

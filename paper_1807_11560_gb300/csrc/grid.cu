@@ -16,8 +16,6 @@ namespace {
 constexpr int kThreads = 256;
 inline unsigned blocks_for(long long n) { return (unsigned)((n + kThreads - 1) / kThreads); }
 
-__device__ __forceinline__ bool nyq(int q, int K) { return (K % 2 == 0) && (2 * q == K); }
-
 // ---- periodic trilinear interpolation ------------------------------------------
 // Cell of the point ix - dsp on an axis of n nodes: lower node c0, upper c1,
 // weight w of the upper node.  The foot point is kept as integer index plus a
@@ -288,28 +286,6 @@ k_terminal(const T* __restrict__ m, const T* __restrict__ y, int diff, T coef, T
 }
 
 // ---- band vectors -----------------------------------------------------------------
-template <typename T>
-__global__ void k_hermitianize(const cplx<T>* __restrict__ in, cplx<T>* __restrict__ out, int ncomp,
-                               Band b) {
-  const long long kvol = b.vol();
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= ncomp * kvol) return;
-  const long long c = idx / kvol;
-  const long long r = idx % kvol;
-  const int k3 = (int)(r % b.k3);
-  const int k2 = (int)((r / b.k3) % b.k2);
-  const int k1 = (int)(r / ((long long)b.k2 * b.k3));
-  cplx<T> v{T(0), T(0)};
-  if (!(nyq(k1, b.k1) || nyq(k2, b.k2) || nyq(k3, b.k3))) {
-    const long long m = c * kvol +
-        (((long long)((b.k1 - k1) % b.k1) * b.k2 + (b.k2 - k2) % b.k2) * b.k3 + (b.k3 - k3) % b.k3);
-    const cplx<T> a = in[idx], am = in[m];
-    v.x = T(0.5) * (a.x + am.x);
-    v.y = T(0.5) * (a.y - am.y);
-  }
-  out[idx] = v;
-}
-
 // ---- conjugate gradients with device-resident scalars (Eq. 45) ------------------
 // s[] holds rho, ||b||, <d, Hd>, alpha, rho_new, beta, the stop flag, the
 // iterations done, the iteration counter and the "x = d" flag; every update
@@ -325,39 +301,27 @@ __global__ void k_pcg_init(double* s) {
 
 // out = x + sign s[ci] y unless stopped
 template <typename T>
-__global__ void k_axpy_dev(cplx<T>* out, const cplx<T>* x, const cplx<T>* y, const double* s, int ci, double sign,
-                           long long n) {
+__global__ void k_axpy_dev(T* out, const T* x, const T* y, const double* s, int ci, double sign, long long n) {
   if (s[PCG_DONE] != 0.0) return;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const T b = (T)(sign * s[ci]);
-  cplx<T> v = x[i];
-  v.x = fma(b, y[i].x, v.x);
-  v.y = fma(b, y[i].y, v.y);
+  out[i] = fma((T)(sign * s[ci]), y[i], x[i]);
+}
+
+template <typename T>
+__global__ void k_axpby(T* out, T a, const T* x, T bc, const T* y, long long n) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  T v = a * x[i];
+  if (y) v = fma(bc, y[i], v);
   out[i] = v;
 }
 
 template <typename T>
-__global__ void k_axpby(cplx<T>* out, T a, const cplx<T>* x, T bc, const cplx<T>* y, long long n) {
+__global__ void k_scale_L(T* out, const T* x, const T* __restrict__ L, long long kvol, long long n) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  cplx<T> v = x[i];
-  v.x *= a;
-  v.y *= a;
-  if (y) {
-    v.x = fma(bc, y[i].x, v.x);
-    v.y = fma(bc, y[i].y, v.y);
-  }
-  out[i] = v;
-}
-
-template <typename T>
-__global__ void k_scale_L(cplx<T>* out, const cplx<T>* x, const T* __restrict__ L, long long kvol,
-                          long long n) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const T l = L[i % kvol];
-  out[i] = cplx<T>{l * x[i].x, l * x[i].y};
+  out[i] = L[i % kvol] * x[i];
 }
 
 // ---- deterministic FP64 reductions ------------------------------------------------
@@ -390,14 +354,12 @@ k_sumsq_diff(const T* __restrict__ a, const T* __restrict__ b, long long n, doub
 
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
-k_inner_V(const cplx<T>* __restrict__ a, const cplx<T>* __restrict__ b, const T* __restrict__ L,
-          long long kvol, long long n, double* partial) {
+k_inner_V(const T* __restrict__ a, const T* __restrict__ b, const T* __restrict__ Lw, long long kvol, long long n,
+          double* partial) {
   double acc = 0.0;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    const double l = (double)L[i % kvol];
-    acc = fma(l, (double)a[i].x * (double)b[i].x + (double)a[i].y * (double)b[i].y, acc);
-  }
+       i += (long long)gridDim.x * blockDim.x)
+    acc = fma((double)Lw[i % kvol], (double)a[i] * (double)b[i], acc);
   acc = block_sum(acc);
   if (threadIdx.x == 0) partial[blockIdx.x] = acc;
 }
@@ -469,57 +431,6 @@ k_def_force(const T* __restrict__ gs, const T* __restrict__ m1, const T* __restr
   f[2 * vol + idx] = a * g2;
 }
 
-// pointwise products of the deformation form on the padded grid; fields are
-// [12][vol] blocks {Jacobian D[3 i + j] = d_j a_i, values}:
-//   mode 0:  out_i = -(v_i + sum_j D_ij v_j)                      fl = {D u, v}
-//   mode 1:  out_i = -(dv_i + sum_j dD_ij v_j + D_ij dv_j)         fl = {D du, dv}, fc = {D u, v}
-//   mode 2:  out_i = r_i + sum_j D_ji r_j                           fl = {D u, r}
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
-k_def_products(int mode, const T* __restrict__ fl, const T* __restrict__ fc, T* __restrict__ out,
-               long long vol) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= vol) return;
-  const T* src = mode == 1 ? fc : fl;       // the block holding D u and v (or r)
-  T D[9], v[3];
-#pragma unroll
-  for (int q = 0; q < 9; ++q) D[q] = src[q * vol + idx];
-#pragma unroll
-  for (int j = 0; j < 3; ++j) v[j] = src[(9 + j) * vol + idx];
-  if (mode == 2) {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      T acc = v[i];
-#pragma unroll
-      for (int j = 0; j < 3; ++j) acc = fma(D[3 * j + i], v[j], acc);
-      out[i * vol + idx] = acc;
-    }
-    return;
-  }
-  if (mode == 0) {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      T a = T(0);
-#pragma unroll
-      for (int j = 0; j < 3; ++j) a = fma(D[3 * i + j], v[j], a);
-      out[i * vol + idx] = -(v[i] + a);
-    }
-    return;
-  }
-  T dD[9], dv[3];
-#pragma unroll
-  for (int q = 0; q < 9; ++q) dD[q] = fl[q * vol + idx];
-#pragma unroll
-  for (int j = 0; j < 3; ++j) dv[j] = fl[(9 + j) * vol + idx];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    T a = T(0);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) a = fma(dD[3 * i + j], v[j], fma(D[3 * i + j], dv[j], a));
-    out[i * vol + idx] = -(dv[i] + a);
-  }
-}
-
 
 // ---- PCG steps with the scalar logic folded into the reductions ---------------
 // <d, q>_V from the block partials, then alpha, or the stop at non-positive
@@ -552,9 +463,8 @@ __global__ void __launch_bounds__(kThreads) k_finalize_alpha(const double* parti
 // r -= alpha q; block partials of <r, r>_V
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
-k_pcg_xr(cplx<T>* __restrict__ x, cplx<T>* __restrict__ r, const cplx<T>* __restrict__ d,
-         const cplx<T>* __restrict__ q, const T* __restrict__ L, long long kvol, long long n,
-         const double* s, double* partial) {
+k_pcg_xr(T* __restrict__ x, T* __restrict__ r, const T* __restrict__ d, const T* __restrict__ q,
+         const T* __restrict__ Lw, long long kvol, long long n, const double* s, double* partial) {
   const bool copy = s[PCG_COPY] != 0.0;
   const bool done = s[PCG_DONE] != 0.0;
   const T a = (T)s[PCG_A];
@@ -563,16 +473,10 @@ k_pcg_xr(cplx<T>* __restrict__ x, cplx<T>* __restrict__ r, const cplx<T>* __rest
        i += (long long)gridDim.x * blockDim.x) {
     if (copy) x[i] = d[i];
     if (done) continue;
-    cplx<T> xv = x[i], rv = r[i];
-    const cplx<T> dv = d[i], qv = q[i];
-    xv.x = fma(a, dv.x, xv.x);
-    xv.y = fma(a, dv.y, xv.y);
-    rv.x = fma(-a, qv.x, rv.x);
-    rv.y = fma(-a, qv.y, rv.y);
-    x[i] = xv;
+    x[i] = fma(a, d[i], x[i]);
+    const T rv = fma(-a, q[i], r[i]);
     r[i] = rv;
-    const double l = (double)L[i % kvol];
-    acc = fma(l, (double)rv.x * (double)rv.x + (double)rv.y * (double)rv.y, acc);
+    acc = fma((double)Lw[i % kvol], (double)rv * (double)rv, acc);
   }
   acc = block_sum(acc);
   if (threadIdx.x == 0) partial[blockIdx.x] = acc;
@@ -653,20 +557,14 @@ void terminal_field(const T* m, const T* y, int diff, double coef, T* out, Dims 
 }
 
 template <typename T>
-void hermitianize(const cplx<T>* in, cplx<T>* out, int ncomp, Band b, cudaStream_t st) {
-  k_hermitianize<T><<<blocks_for(ncomp * b.vol()), kThreads, 0, st>>>(in, out, ncomp, b);
-}
-
-template <typename T>
-void axpby(cplx<T>* out, double a, const cplx<T>* x, double bcoef, const cplx<T>* y, long long n,
-           cudaStream_t st) {
+void axpby(T* out, double a, const T* x, double bcoef, const T* y, long long n, cudaStream_t st) {
   k_axpby<T><<<blocks_for(n), kThreads, 0, st>>>(out, (T)a, x, (T)bcoef, y, n);
 }
 
 void pcg_init(double* s, cudaStream_t st) { k_pcg_init<<<1, 1, 0, st>>>(s); }
 
 template <typename T>
-void scale_L(cplx<T>* out, const cplx<T>* x, const T* Lhat, int ncomp, long long kvol, cudaStream_t st) {
+void scale_L(T* out, const T* x, const T* Lhat, int ncomp, long long kvol, cudaStream_t st) {
   k_scale_L<T><<<blocks_for(ncomp * kvol), kThreads, 0, st>>>(out, x, Lhat, kvol, ncomp * kvol);
 }
 
@@ -677,19 +575,19 @@ void sum_sq_diff(const T* a, const T* b, long long n, double* partial, double* o
 }
 
 template <typename T>
-void inner_V(const cplx<T>* a, const cplx<T>* b, const T* Lhat, int ncomp, long long kvol,
-             double* partial, double* out, cudaStream_t st) {
-  k_inner_V<T><<<kReduceBlocks, kThreads, 0, st>>>(a, b, Lhat, kvol, ncomp * kvol, partial);
+void inner_V(const T* a, const T* b, const T* Lw, int ncomp, long long kvol, double* partial, double* out,
+             cudaStream_t st) {
+  k_inner_V<T><<<kReduceBlocks, kThreads, 0, st>>>(a, b, Lw, kvol, ncomp * kvol, partial);
   k_finalize<<<1, kThreads, 0, st>>>(partial, kReduceBlocks, out);
 }
 
 template <typename T>
-void pcg_step(cplx<T>* x, cplx<T>* r, cplx<T>* d, const cplx<T>* q, const T* Lhat, long long kvol, int ncomp,
+void pcg_step(T* x, T* r, T* d, const T* q, const T* Lw, long long kvol, int ncomp,
               double* partial, double* s, double tol, cudaStream_t st) {
   const long long n = ncomp * kvol;
-  k_inner_V<T><<<kReduceBlocks, kThreads, 0, st>>>(d, q, Lhat, kvol, n, partial);
+  k_inner_V<T><<<kReduceBlocks, kThreads, 0, st>>>(d, q, Lw, kvol, n, partial);
   k_finalize_alpha<<<1, kThreads, 0, st>>>(partial, kReduceBlocks, s);
-  k_pcg_xr<T><<<kReduceBlocks, kThreads, 0, st>>>(x, r, d, q, Lhat, kvol, n, s, partial);
+  k_pcg_xr<T><<<kReduceBlocks, kThreads, 0, st>>>(x, r, d, q, Lw, kvol, n, s, partial);
   k_finalize_beta<<<1, kThreads, 0, st>>>(partial, kReduceBlocks, s, tol);
   k_axpy_dev<T><<<blocks_for(n), kThreads, 0, st>>>(d, r, d, s, PCG_BETA, 1.0, n);
 }
@@ -710,19 +608,13 @@ void def_force(const T* gs, const T* m1, const T* I1, const T* du, T* dm_out, do
   k_def_force<T><<<blocks_for(vol), kThreads, 0, st>>>(gs, m1, I1, du, dm_out, (T)c, f, vol);
 }
 
-template <typename T>
-void def_products(int mode, const T* fields, const T* cached, T* out, long long vol, cudaStream_t st) {
-  k_def_products<T><<<blocks_for(vol), kThreads, 0, st>>>(mode, fields, cached, out, vol);
-}
-
 #define LDDMM_INST(T)                                                                              \
-  template void pcg_step<T>(cplx<T>*, cplx<T>*, cplx<T>*, const cplx<T>*, const T*, long long, int,  \
+  template void pcg_step<T>(T*, T*, T*, const T*, const T*, long long, int,  \
                             double*, double*, double, cudaStream_t);                                \
   template void central_grad<T>(const T*, T*, Dims, cudaStream_t);                                 \
   template void def_sample<T>(const T*, const T*, const T*, T*, T*, Dims, cudaStream_t);           \
   template void def_force<T>(const T*, const T*, const T*, const T*, T*, double, T*, long long,    \
                              cudaStream_t);                                                        \
-  template void def_products<T>(int, const T*, const T*, T*, long long, cudaStream_t);            \
   template void transport_step<T>(const T*, const T*, const T*, T*, T*, Dims, double,            \
                                   cudaStream_t);                                                 \
   template void grad_dot<T>(const T*, const T*, T*, Dims, cudaStream_t);                         \
@@ -733,12 +625,11 @@ void def_products(int mode, const T* fields, const T* cached, T* out, long long 
                                 double, cudaStream_t);                                              \
   template void scaled_diff<T>(const T*, const T*, double, T*, long long, cudaStream_t);          \
   template void terminal_newton<T>(const T*, const T*, const T*, double, T*, Dims, cudaStream_t);  \
-  template void hermitianize<T>(const cplx<T>*, cplx<T>*, int, Band, cudaStream_t);             \
-  template void axpby<T>(cplx<T>*, double, const cplx<T>*, double, const cplx<T>*, long long,    \
+  template void axpby<T>(T*, double, const T*, double, const T*, long long,    \
                          cudaStream_t);                                                          \
-  template void scale_L<T>(cplx<T>*, const cplx<T>*, const T*, int, long long, cudaStream_t);    \
+  template void scale_L<T>(T*, const T*, const T*, int, long long, cudaStream_t);    \
   template void sum_sq_diff<T>(const T*, const T*, long long, double*, double*, cudaStream_t);   \
-  template void inner_V<T>(const cplx<T>*, const cplx<T>*, const T*, int, long long, double*,    \
+  template void inner_V<T>(const T*, const T*, const T*, int, long long, double*,    \
                            double*, cudaStream_t);
 LDDMM_INST(float)
 LDDMM_INST(double)

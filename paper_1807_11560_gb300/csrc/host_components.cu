@@ -9,27 +9,23 @@ template <typename T>
 void Impl<T>::iota_call(const void* a, int ncomp, void* out) {
   for (int c0 = 0; c0 < ncomp; c0 += 3) {
     const int nc = std::min(3, ncomp - c0);
-    cuda(cudaMemcpyAsync(vin, (const C*)a + (long long)c0 * Kvol, (size_t)nc * Kvol * sizeof(C),
+    cuda(cudaMemcpyAsync(zin, (const Z*)a + (long long)c0 * Kuser, (size_t)nc * Kuser * sizeof(Z),
                          cudaMemcpyDefault, st), "copy");
-    hermitianize<T>(vin, px, nc, K, st);
+    band_load<T>(zin, px, nc, K, st);
     ++launches;
-    IotaDesc<T> d{};
+    IotaList<T> d{};
     d.nf = nc;
     for (int c = 0; c < nc; ++c) {
       d.src[c] = px + c * Kvol;
       d.dst[c] = fterm + c * Nvol;
-      d.deriv[c] = -1;
-      d.applyL[c] = 0;
     }
-    iota_batch<T>(full, d, Lhat, T2, st, use_tc() ? dres + 7 : nullptr);
+    cuda(iota_fields<T>(full, d, T1, st), "iota");
     launches += kIotaLaunches;
     check_launch("iota");
     cuda(cudaMemcpyAsync((T*)out + (long long)c0 * Nvol, fterm, (size_t)nc * Nvol * sizeof(T),
                          cudaMemcpyDefault, st), "copy");
   }
-  cuda(cudaMemcpyAsync(hres + 7, dres + 7, sizeof(double), cudaMemcpyDeviceToHost, st), "read flag");
   sync("iota");
-  check_flag(hres[7]);
 }
 
 template <typename T>
@@ -38,18 +34,17 @@ void Impl<T>::pi_call(const void* f, int ncomp, void* out) {
     const int nc = std::min(3, ncomp - c0);
     cuda(cudaMemcpyAsync(fterm, (const T*)f + (long long)c0 * Nvol, (size_t)nc * Nvol * sizeof(T),
                          cudaMemcpyDefault, st), "copy");
-    PiSrc<T> ps{};
-    ps.nf = nc;
-    for (int c = 0; c < nc; ++c) ps.src[c] = fterm + c * Nvol;
+    const T* src[3] = {fterm, fterm + Nvol, fterm + 2 * Nvol};
     PiEpi<T> e = epi(nc, 1);
     e.grp[0] = 0;
     e.coef[0] = (T)(1.0 / (double)Nvol);
     e.applyK[0] = 0;
     add_out(e, vout, 0, 1.0, {});
-    pi_batch<T>(full, ps, e, Lhat, T2, st);
-    launches += kPiLaunches;
+    cuda(pi_fields<T>(full, src, e, Lhat, P1, st), "pi");
+    band_store<T>(vout, zout, nc, K, st);
+    launches += kPiLaunches + 1;
     check_launch("pi");
-    cuda(cudaMemcpyAsync((C*)out + (long long)c0 * Kvol, vout, (size_t)nc * Kvol * sizeof(C),
+    cuda(cudaMemcpyAsync((Z*)out + (long long)c0 * Kuser, zout, (size_t)nc * Kuser * sizeof(Z),
                          cudaMemcpyDefault, st), "copy");
   }
   sync("pi");
@@ -65,6 +60,7 @@ void Impl<T>::ad_dagger_call(const void* v, const void* u, void* out) {
   e.applyK[0] = 1;
   add_out(e, vout, 0, 1.0, {});
   eval(PW_F, slot(trial, 0), px, pr, e);   // P(v, L u): v-fields from px, L-fields from pr
+  flush();
   store_bl(vout, out);
   sync("ad_dagger");
 }
@@ -81,6 +77,7 @@ void Impl<T>::ad_call(const void* v, const void* w, void* out) {
   e.grp[2] = 0; e.coef[2] = (T)(1.0 / (double)Mvol);
   add_out(e, vout, 0, 1.0, {});
   eval(PW_GT, vslot, pr, pr, e);
+  flush();
   store_bl(vout, out);
   sync("ad");
 }

@@ -9,7 +9,7 @@ namespace host {
 
 template <typename T>
 void Impl<T>::energy_terms(State<T>& S) {
-  inner_V<T>(S.vh, S.vh, Lhat, 3, Kvol, partial, dres, st);
+  inner_V<T>(S.vh, S.vh, Lw, 3, Kvol, partial, dres, st);
   sum_sq_diff<T>(m1(S), I1, Nvol, partial, dres + 1, st);
   launches += 4;
   check_launch("energy reductions");
@@ -25,7 +25,7 @@ double Impl<T>::read_energy() {
 
 template <typename T>
 double Impl<T>::dot_V(const C* a, const C* b) {
-  inner_V<T>(a, b, Lhat, 3, Kvol, partial, dres + 2, st);
+  inner_V<T>(a, b, Lw, 3, Kvol, partial, dres + 2, st);
   launches += 2;
   cuda(cudaMemcpyAsync(hres + 2, dres + 2, 6 * sizeof(double), cudaMemcpyDeviceToHost, st), "read dot");
   sync("inner product");
@@ -247,6 +247,7 @@ void Impl<T>::build_graph(bool newton) {
     enqueue_hessvec(newton);
   } catch (...) {
     capturing = false;
+    pending = false;
     cudaStreamEndCapture(cap, &g);
     if (g) cudaGraphDestroy(g);
     st = user;

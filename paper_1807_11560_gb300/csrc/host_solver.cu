@@ -43,12 +43,12 @@ void Impl<T>::gn_solve(void* v0, int n_gn, int n_pcg, lddmm_report* rep) {
     ++launches;
     // the scalars stay on the device; the host looks at the stop flag every
     // fourth iteration (iterations after a stop only repeat the product)
-    inner_V<T>(pr, pr, Lhat, 3, Kvol, partial, dpcg + PCG_R, st);
+    inner_V<T>(pr, pr, Lw, 3, Kvol, partial, dpcg + PCG_R, st);
     pcg_init(dpcg, st);
     launches += 3;
     for (int k = 1; k <= n_pcg; ++k) {
       hessvec_dev(opts.newton != 0);
-      pcg_step<T>(px, pr, dvh, vout, Lhat, Kvol, 3, partial, dpcg, opts.pcg_tol, st);
+      pcg_step<T>(px, pr, dvh, vout, Lw, Kvol, 3, partial, dpcg, opts.pcg_tol, st);
       launches += 5;
       if (k % 4 == 0 && k < n_pcg) {
         cuda(cudaMemcpyAsync(hres, dpcg + PCG_DONE, sizeof(double), cudaMemcpyDeviceToHost, st), "read");

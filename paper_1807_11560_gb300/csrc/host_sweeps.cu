@@ -1,5 +1,5 @@
-// Host side, time sweeps: one bracket evaluation (three kernels or a
-// persistent sweep), the Heun shoot (Eq. 51), the state transport (Eq. 52),
+// Host side, time sweeps: one evaluation (two kernels, or part of a persistent
+// sweep), the Heun shoot (Eq. 51), the state transport (Eq. 52),
 // the tangent (Eq. 30) and the backward adjoint Jacobi sweeps (Eqs. 53-54),
 // the full-Newton sweep (Eqs. 56-57) and the exact discrete adjoint.
 #include "impl.h"
@@ -10,29 +10,43 @@ namespace host {
 template <typename T>
 void Impl<T>::eval(PwMode mode, T* slot, const C* srcA, const C* srcB, const PiEpi<T>& e, T* slot2) {
   if (rec) {
+    if (!rec->empty()) link(rec->back().epi, srcA, srcB);
     rec->push_back(EvalDesc<T>{srcA, srcB, slot, slot2, e});
     return;
   }
-  pb(PR_IOTA_AB);
-  bracket_iota<T>(pad, block24(srcA, srcB, slot), Lhat, T2, st, use_tc_pad() ? dres + 7 : nullptr);
-  pe(PR_IOTA_AB, flops_iota_ab());
-  pb(PR_CPW);
-  bracket_cpw<T>(pad, mode, T2, slot, slot2, P2, st, use_tc_pad() ? dres + 7 : nullptr);
-  pe(PR_CPW, flops_cpw(mode));
+  if (pending && pend_mode != mode) flush();
+  const bool proj = pending && pend_epi.nout > 0;
+  if (proj) link(pend_epi, srcA, srcB);
   pb(PR_PI_BA);
-  bracket_pi<T>(pad, e, Lhat, P2, st, use_tc_pad() ? dres + 7 : nullptr);
-  pe(PR_PI_BA, flops_pi_ba(e.nper));
-  launches += kBracketLaunches;
-  check_launch("bracket evaluation");
+  cuda(band_phase<T>(pad, mode, proj ? &pend_epi : nullptr, P1, srcA, srcB, T1, Lhat, st), "band phase");
+  pe(PR_PI_BA, 2.0 * K.vol() * M.n1 * (mode_in(mode) + (proj ? mode_out(pend_mode) : 0)) * 0.5);
+  pb(PR_CPW);
+  cuda(plane_phase<T>(pad, mode, T1, slot, slot2, P1, st), "plane phase");
+  pe(PR_CPW, eval_flops(mode) - (double)K.vol() * M.n1 * (mode_in(mode) + mode_out(mode)));
+  launches += kEvalLaunches;
+  pending = true;
+  pend_mode = mode;
+  pend_epi = e;
+}
+
+template <typename T>
+void Impl<T>::flush() {
+  if (rec || !pending) return;
+  pending = false;
+  if (pend_epi.nout == 0) return;
+  pb(PR_PI_BA);
+  cuda(band_phase<T>(pad, pend_mode, &pend_epi, P1, nullptr, nullptr, T1, Lhat, st), "band phase");
+  pe(PR_PI_BA, (double)K.vol() * M.n1 * mode_out(pend_mode));
+  ++launches;
 }
 
 template <typename T>
 void Impl<T>::run_sweep(PwMode mode, const EvalDesc<T>* ev, int nev) {
   if (nev == 0) nev = 2 * Nt;
   pb(PR_SWEEP);
-  cuda(sweep_launch<T>(pad, mode, ev, nev, Lhat, T2, P2, bar, dres + 7, st, opts.debug_stall),
+  cuda(sweep_launch<T>(pad, mode, ev, nev, Lhat, T1, P1, bar, dres + 7, st, opts.debug_stall),
        "persistent sweep");
-  pe(PR_SWEEP, sweep_flops[mode] * nev / (2.0 * Nt));
+  pe(PR_SWEEP, eval_flops(mode) * nev);
   ++launches;
 }
 
@@ -40,61 +54,52 @@ template <typename T>
 void Impl<T>::to_grid(const C* hist, int count, T* grid) {
   for (int v0 = 0; v0 < count; v0 += 11) {
     const int nv = std::min(11, count - v0);
-    IotaDesc<T> d{};
+    IotaList<T> d{};
     d.nf = 3 * nv;
     for (int v = 0; v < nv; ++v)
       for (int c = 0; c < 3; ++c) {
         const int f = 3 * v + c;
         d.src[f] = hist + ((long long)(v0 + v) * 3 + c) * Kvol;
         d.dst[f] = grid + ((long long)(v0 + v) * 3 + c) * Nvol;
-        d.deriv[f] = -1;
-        d.applyL[f] = 0;
       }
     pb(PR_IOTA_FULL);
-    iota_batch<T>(full, d, Lhat, T2, st, use_tc() ? dres + 7 : nullptr);
-    pe(PR_IOTA_FULL, iota_flops(d.nf));
+    cuda(iota_fields<T>(full, d, T1, st), "iota to image grid");
+    pe(PR_IOTA_FULL, grid_flops(N, d.nf));
     launches += kIotaLaunches;
   }
-  check_launch("iota to image grid");
 }
 
 template <typename T>
 void Impl<T>::project_K(const T* f3, C* out, bool applyK) {
-  PiSrc<T> ps{};
-  ps.nf = 3;
-  for (int c = 0; c < 3; ++c) ps.src[c] = f3 + c * Nvol;
+  const T* src[3] = {f3, f3 + Nvol, f3 + 2 * Nvol};
   PiEpi<T> e = epi(3, 1);
   e.grp[0] = 0;
   e.coef[0] = (T)(1.0 / (double)Nvol);
   e.applyK[0] = applyK ? 1 : 0;
   add_out(e, out, 0, 1.0, {});
   pb(PR_PI_FULL);
-  pi_batch<T>(full, ps, e, Lhat, T2, st);
-  pe(PR_PI_FULL, iota_flops(3));
+  cuda(pi_fields<T>(full, src, e, Lhat, P1, st), "projection");
+  pe(PR_PI_FULL, grid_flops(N, 3));
   launches += kPiLaunches;
-  check_launch("projection");
 }
 
 template <typename T>
 void Impl<T>::project_adjoint(const T* f3, C* out) {
-  PiSrc<T> ps{};
-  ps.nf = 3;
-  for (int c = 0; c < 3; ++c) ps.src[c] = f3 + c * Nvol;
+  const T* src[3] = {f3, f3 + Nvol, f3 + 2 * Nvol};
   PiEpi<T> e = epi(3, 1);
   e.grp[0] = 0;
   e.coef[0] = (T)1;
   e.applyK[0] = 1;
   add_out(e, out, 0, 1.0, {});
   pb(PR_PI_FULL);
-  pi_batch<T>(full, ps, e, Lhat, T2, st);
-  pe(PR_PI_FULL, iota_flops(3));
+  cuda(pi_fields<T>(full, src, e, Lhat, P1, st), "projection");
+  pe(PR_PI_FULL, grid_flops(N, 3));
   launches += kPiLaunches;
-  check_launch("projection");
 }
 
 template <typename T>
 void Impl<T>::shoot(State<T>& S) {
-  if (persistent()) {
+  if (run_persistent()) {
     run_sweep(PW_F, &S == &lin ? ev_shoot_lin : ev_shoot_trial);
     return;
   }
@@ -117,6 +122,7 @@ void Impl<T>::shoot(State<T>& S) {
     add_out(e2, vn1, 0, 0.5 * dt, {{vn, 1.0}, {k1, 0.5 * dt}});
     eval(PW_F, slot(S, 2 * n + 1), vs, vs, e2);
   }
+  flush();
 }
 
 template <typename T>
@@ -159,7 +165,7 @@ template <typename T>
 void Impl<T>::backward(State<T>& S) {
   const double m = 1.0 / (double)Mvol;
   if (!rec) cuda(cudaMemsetAsync(W, 0, (size_t)3 * Kvol * sizeof(C), st), "memset W");
-  if (persistent()) {
+  if (run_persistent()) {
     run_sweep(PW_GT, ev_backward);
     return;
   }
@@ -181,15 +187,17 @@ void Impl<T>::backward(State<T>& S) {
     add_out(e2, W, 1, 0.5 * dt, {{W, 1.0}, {aW, 0.5 * dt}, {Ut, 0.5 * dt}});
     eval(PW_GT, slot(S, 2 * n), Wt, Ut, e2);
   }
+  flush();
 }
 
 template <typename T>
 void Impl<T>::tangent(State<T>& S, bool cache) {
-  if (persistent()) {
-    run_sweep(PW_T, cache ? ev_tangent_c : ev_tangent);
+  if (run_persistent()) {
+    run_sweep(cache ? PW_TC : PW_T, cache ? ev_tangent_c : ev_tangent);
     return;
   }
   const double m = 1.0 / (double)Mvol;
+  const PwMode mode = cache ? PW_TC : PW_T;
   for (int n = 0; n < Nt; ++n) {
     C* dn = vec(dvh, n);
     C* dn1 = vec(dvh, n + 1);
@@ -200,14 +208,15 @@ void Impl<T>::tangent(State<T>& S, bool cache) {
     e1.applyK[0] = 1;
     add_out(e1, k1, 0, 1.0, {});
     add_out(e1, dstar, 0, dt, {{dn, 1.0}});
-    eval(PW_T, slot(S, 2 * n), dn, dn, e1, cache ? tslot(2 * n) : nullptr);
+    eval(mode, slot(S, 2 * n), dn, dn, e1, cache ? tslot(2 * n) : nullptr);
     PiEpi<T> e2 = epi(3, 1);
     e2.grp[0] = 0;
     e2.coef[0] = (T)(-m);
     e2.applyK[0] = 1;
     add_out(e2, dn1, 0, 0.5 * dt, {{dn, 1.0}, {k1, 0.5 * dt}});
-    eval(PW_T, slot(S, 2 * n + 1), dstar, dstar, e2, cache ? tslot(2 * n + 1) : nullptr);
+    eval(mode, slot(S, 2 * n + 1), dstar, dstar, e2, cache ? tslot(2 * n + 1) : nullptr);
   }
+  flush();
 }
 
 template <typename T>
@@ -216,7 +225,7 @@ void Impl<T>::backward_sources(State<T>& S) {
   if (!rec)
     cuda(cudaMemcpyAsync(W, srcs + (long long)Nt * 3 * Kvol, (size_t)3 * Kvol * sizeof(C),
                          cudaMemcpyDeviceToDevice, st), "copy source");
-  if (persistent()) {
+  if (run_persistent()) {
     run_sweep(PW_GT, ev_exact);
     return;
   }
@@ -235,13 +244,14 @@ void Impl<T>::backward_sources(State<T>& S) {
     add_out(e2, W, 1, 0.5 * dt, {{W, 1.0}, {aW, 0.5 * dt}, {srcs + (long long)n * 3 * Kvol, 1.0}});
     eval(PW_GT, slot(S, 2 * n), Wt, zero3, e2);
   }
+  flush();
 }
 
 template <typename T>
 void Impl<T>::backward_hist(State<T>& S) {
   const double m = 1.0 / (double)Mvol;
   if (!rec) cuda(cudaMemsetAsync(vec(Wh, Nt), 0, (size_t)3 * Kvol * sizeof(C), st), "memset W");
-  if (persistent()) {
+  if (run_persistent()) {
     run_sweep(PW_GT, ev_backward_hist);
     return;
   }
@@ -264,13 +274,14 @@ void Impl<T>::backward_hist(State<T>& S) {
     add_out(e2, vec(Wh, n), 1, 0.5 * dt, {{W1, 1.0}, {aW, 0.5 * dt}, {Ut_, 0.5 * dt}});
     eval(PW_GT, slot(S, 2 * n), Wt_, Ut_, e2);
   }
+  flush();
 }
 
 template <typename T>
 void Impl<T>::newton_backward(State<T>& S) {
   const double m = 1.0 / (double)Mvol;
   if (!rec) cuda(cudaMemsetAsync(W, 0, (size_t)3 * Kvol * sizeof(C), st), "memset W");
-  if (persistent()) {
+  if (run_persistent()) {
     run_sweep(PW_GT, ev_newton, 4 * Nt);
     return;
   }
@@ -305,6 +316,7 @@ void Impl<T>::newton_backward(State<T>& S) {
     add_out(e4, W, 1, 0.5 * dt, {{W, 1.0}, {aW, 0.5 * dt}, {bW, 0.5 * dt}});
     eval(PW_GT, tslot(2 * n), vec(Wth, n), vec(Uth, n), e4);
   }
+  flush();
 }
 
 template <typename T>
@@ -344,6 +356,8 @@ void Impl<T>::exact_backward() {
 
 // the members defined here, for both precisions
 template void Impl<float>::eval(PwMode mode, float* slot, const C* srcA, const C* srcB, const PiEpi<float>& e, float* slot2);
+template void Impl<float>::flush();
+template void Impl<double>::flush();
 template void Impl<float>::run_sweep(PwMode mode, const EvalDesc<float>* ev, int nev);
 template void Impl<float>::to_grid(const C* hist, int count, float* grid);
 template void Impl<float>::project_K(const float* f3, C* out, bool applyK);

@@ -2,12 +2,12 @@
 // C interface of include/lddmm.h (internal; not part of the interface).
 //
 // A context owns, per problem, every device buffer of the method:
-//   * twiddle tables of the image-grid plan (N) and of the padded product
-//     plan (M = ceil(3K/2)), and the symbol table L^(k);
+//   * the folded cosine/sine tables of the image-grid plan (N) and of the padded
+//     product plan (M = ceil(3K/2)), and the symbol table L^(k);
 //   * two trajectories ("lin", the Gauss-Newton linearisation point, and
 //     "trial", used by energy evaluations and component calls), each with the
-//     BL history v_n, the Heun predictors v*_{n+1}, the 24 padded-grid fields
-//     (v, Dv, L v, D(L v)) of every Heun stage point, the grid velocities
+//     BL history v_n, the Heun predictors v*_{n+1}, the 18 padded-grid fields
+//     (v, Dv, L v, curl L v) of every Heun stage point, the grid velocities
 //     iota(v_n), the state history m_n and the characteristic displacements;
 //   * the tangent history dv_n and its grid velocities, two ping-pong pairs
 //     for dm and s = grad m . dv, the transform scratch and BL temporaries;
@@ -20,7 +20,7 @@
 // CUDA graph and replayed.
 //
 // The members are defined by responsibility: host_context.cu (allocation,
-// plans, autotuner, probe), host_sweeps.cu (bracket evaluations and the time
+// plans, probe), host_sweeps.cu (bracket evaluations and the time
 // sweeps), host_deform.cu (the deformation-state form), host_objective.cu
 // (energy, gradient, Hessian-vector products, graph capture), host_solver.cu
 // (GN-Krylov), host_components.cu (the component calls); api.cu holds the C
@@ -58,38 +58,39 @@ const char* const kProbeNames[PR_COUNT] = {"transport", "inc_step", "iota_ab", "
 
 template <typename T>
 struct State {
-  cplx<T>* vh = nullptr;    // [Nt+1][3][Kvol]
-  cplx<T>* vsh = nullptr;   // [Nt][3][Kvol]
-  T* cache = nullptr;       // [2 Nt][cache_slot_elems]: 24 padded-grid fields per stage point
+  T* vh = nullptr;          // [Nt+1][3][Kvol]
+  T* vsh = nullptr;         // [Nt][3][Kvol]
+  T* cache = nullptr;       // [2 Nt][18][Mvol]: padded-grid fields per stage point
   T* vgrid = nullptr;       // [Nt+1][3][Nvol]  (recompute: [2][3][Nvol], step n in n & 1)
   T* mh = nullptr;          // [Nt+1][Nvol]     (recompute: [2][Nvol])
   T* off = nullptr;         // [Nt][3][Nvol]    (recompute: [3][Nvol], the current step)
   // deformation-state form (Section 3.3): band-limited inverse-map displacement
-  cplx<T>* uh = nullptr;    // [Nt+1][3][Kvol]
-  cplx<T>* ush = nullptr;   // [Nt][3][Kvol]    Heun predictors u*_n
+  T* uh = nullptr;          // [Nt+1][3][Kvol]
+  T* ush = nullptr;         // [Nt][3][Kvol]    Heun predictors u*_n
 };
 
 template <typename T>
 struct Impl {
-  using C = cplx<T>;
+  using C = T;               // element of a band vector (internal.h): 3 Kvol reals
+  using Z = cplx<T>;         // element of the caller's Hermitian arrays
   std::string* err = nullptr;
   int ndim = 3, duser = 3;
   Dims N{}, M{};
   Band K{};
   int Nt = 1, s = 2;
   double alpha = 0, sigma = 1, dt = 1;
-  long long Nvol = 0, Mvol = 0, Kvol = 0;
+  long long Nvol = 0, Mvol = 0, Kvol = 0, Kuser = 0;   // Kuser: complex slots of a user component
   lddmm_opts opts{};
-  int split = 0;             // FP32 tensor-core split of the image-grid transform: 0 3xTF32, 1 BF16x3
   cudaStream_t st = nullptr;
   Plan<T> full{}, pad{};
-  T* Lhat = nullptr;
+  T *Lhat = nullptr, *Lw = nullptr;   // L^ per slot; with the weights of the V product
   T *I0 = nullptr, *I1 = nullptr;
   State<T> lin, trial;
   bool have_images = false, have_lin = false, have_dm1 = false;
-  C *T2 = nullptr, *P2 = nullptr;
+  T *T1 = nullptr, *P1 = nullptr;     // transform scratch: plane fields, projected planes
+  Z *zin = nullptr, *zout = nullptr;  // [3][Kuser] staging of the caller's arrays
   C *k1 = nullptr, *aU = nullptr, *aW = nullptr, *Ut = nullptr, *Wt = nullptr, *U = nullptr,
-    *W = nullptr, *dstar = nullptr, *vin = nullptr, *vout = nullptr, *gbuf = nullptr;
+    *W = nullptr, *vout = nullptr, *gbuf = nullptr;
   C *px = nullptr, *pr = nullptr, *vsol = nullptr, *vtry = nullptr;
   C* dvh = nullptr;          // [Nt+1][3][Kvol]
   C* srcs = nullptr;         // [Nt+1][3][Kvol] band sources of the exact discrete adjoint
@@ -97,7 +98,7 @@ struct Impl {
   C *Uh = nullptr, *Wh = nullptr;     // [Nt+1][3][Kvol] gradient sweep (U, W) per time level
   C *Uth = nullptr, *Wth = nullptr;   // [Nt][3][Kvol] gradient sweep stage values (U~, W~)
   C *bU = nullptr, *bW = nullptr;     // full-Newton sweep scratch
-  T* tcache = nullptr;       // [2 Nt][cache_slot_elems] tangent stage-point fields (full Newton)
+  T* tcache = nullptr;       // [2 Nt][18][Mvol] tangent stage-point fields (full Newton)
   C* zero3 = nullptr;        // [3][Kvol] zeros
   T* dvgrid = nullptr;       // [Nt+1][3][Nvol]  (recompute: [2][3][Nvol])
   T *dm[2] = {nullptr, nullptr}, *sb[2] = {nullptr, nullptr};
@@ -111,7 +112,10 @@ struct Impl {
               *ev_backward = nullptr, *ev_exact = nullptr, *ev_tangent_c = nullptr,
               *ev_backward_hist = nullptr, *ev_newton = nullptr;
   unsigned* bar = nullptr;
-  double sweep_flops[3] = {0, 0, 0};   // algorithmic flops of one sweep per mode
+  // the evaluation whose projection and epilogue the next band phase runs
+  bool pending = false;
+  PwMode pend_mode = PW_F;
+  PiEpi<T> pend_epi{};
   long long launches = 0;
   std::vector<void*> allocs;
   unsigned long long device_bytes = 0;
@@ -121,9 +125,7 @@ struct Impl {
   bool have_zhist = false;   // Uh/Wh/Uth/Wth hold the last gradient's backward sweep
   // deformation-state form (Section 3.3)
   T* gI0 = nullptr;           // [3][Nvol] central-difference gradient of I0
-  T* defM = nullptr;          // [12][Mvol] padded-grid fields of the deformation products
   T* defcache = nullptr;      // [2 Nt][12][Mvol] {D u, v} at the stage points of lin's sweep
-  T* prodM = nullptr;         // [3][Mvol] their products
   C *dk1 = nullptr, *rhob = nullptr, *dua = nullptr, *dub = nullptr, *dup = nullptr;   // [3][Kvol]
   cudaStream_t cap = nullptr;
   cudaEvent_t ev = nullptr;
@@ -166,23 +168,16 @@ struct Impl {
   }
   void release();
 
-  static C tw(long long p, int G, int sign, double w = 1.0) {
-    const long long r = ((p % G) + G) % G;
+  // (cos, sin)(2 pi p / G), the sine exactly zero where it is
+  static Pair<T> tw(long long p, int G) {
+    const long long r = p % G;
     const double a = 2.0 * kPi * (double)r / (double)G;
-    return C{(T)(w * std::cos(a)), (T)(w * sign * std::sin(a))};
+    return Pair<T>{(T)std::cos(a), (2 * r) % G == 0 ? T(0) : (T)std::sin(a)};
   }
-  static int sfreq(int q, int Kq) { return (2 * q < Kq) ? q : q - Kq; }
 
   void make_plan(Plan<T>& p, Dims g);
 
   void make_state(State<T>& S);
-  // ------------------------------------------------------------ autotuner
-  // Times the candidate tile shapes of the three padded-grid bracket kernels
-  // on this context's sizes (CUDA events on the context stream, best of three
-  // after a warm-up launch) and keeps the fastest of each.  Tile shapes change
-  // no result: every sum keeps its order whatever the tiling.
-  void autotune();
-
   // image-grid history accessors (step n of a kept or a two-step rolling history)
   long long hstep(int n) const { return opts.recompute ? (n & 1) : n; }
   T* mstate(State<T>& S, int n) { return S.mh + hstep(n) * Nvol; }
@@ -249,28 +244,6 @@ struct Impl {
   void collect();
 
   // -------------------------------------------------------- descriptors
-  IotaDesc<T> block24(const C* srcA, const C* srcB, T* dst) const {
-    IotaDesc<T> d{};
-    d.nf = 24;
-    for (int c = 0; c < 3; ++c) {
-      d.src[c] = srcA + c * Kvol;
-      d.deriv[c] = -1;
-      d.applyL[c] = 0;
-      d.src[12 + c] = srcB + c * Kvol;
-      d.deriv[12 + c] = -1;
-      d.applyL[12 + c] = 1;
-      for (int j = 0; j < 3; ++j) {
-        d.src[3 + 3 * c + j] = srcA + c * Kvol;
-        d.deriv[3 + 3 * c + j] = (signed char)j;
-        d.applyL[3 + 3 * c + j] = 0;
-        d.src[15 + 3 * c + j] = srcB + c * Kvol;
-        d.deriv[15 + 3 * c + j] = (signed char)j;
-        d.applyL[15 + 3 * c + j] = 1;
-      }
-    }
-    for (int f = 0; f < 24; ++f) d.dst[f] = dst + f * Mvol;
-    return d;
-  }
   static PiEpi<T> epi(int ncomp, int nper) {
     PiEpi<T> e;
     std::memset(&e, 0, sizeof(e));
@@ -278,71 +251,63 @@ struct Impl {
     e.nper = nper;
     return e;
   }
+  // output dst = cR * (the fields of group r, each with its coefficient) + terms
   static void add_out(PiEpi<T>& e, C* dst, int r, double cR,
                       std::initializer_list<std::pair<const C*, double>> xs) {
     const int j = e.nout++;
     e.dst[j] = dst;
-    e.r[j] = r;
-    e.cR[j] = (T)cR;
-    e.nx[j] = 0;
+    for (int o = 0; o < e.nper; ++o) e.cY[j][o] = e.grp[o] == r ? (T)(cR * (double)e.coef[o]) : (T)0;
     for (auto& x : xs) {
-      e.X[j][e.nx[j]] = x.first;
-      e.cX[j][e.nx[j]] = (T)x.second;
-      ++e.nx[j];
+      e.X[e.nterm] = x.first;
+      e.cX[j][e.nterm++] = (T)x.second;
+    }
+  }
+  // marks the outputs that the next evaluation reads as its sources
+  static void link(PiEpi<T>& e, const C* A, const C* B) {
+    e.jA = e.jB = -1;
+    for (int j = 0; j < e.nout; ++j) {
+      if (e.dst[j] == A) e.jA = j;
+      if (e.dst[j] == B) e.jB = j;
     }
   }
 
-  // one evaluation of a bracket expression at a Heun stage point
-  // algorithmic flops of the three phases of one bracket evaluation
-  double flops_iota_ab() const {
-    const double H1 = K.h1, K2 = K.k2, K3 = K.k3, M2 = M.n2, M3 = M.n3;
-    return 8.0 * 24 * H1 * (K2 * K3 * M3 + K2 * M2 * M3);
+  // operations of the transforms of nf scalar fields between the band and grid g
+  // (folded cosine/sine sums: K/2 products per point and axis)
+  double grid_flops(const Dims& g, int nf) const {
+    const double k1 = K.k1, k2 = K.k2, k3 = K.k3, n1 = g.n1;
+    return nf * (k1 * n1 * k2 * k3 + n1 * k2 * g.n2 * k3 + n1 * (double)g.n2 * k3 * g.n3);
   }
-  double flops_cpw(PwMode mode) const {
-    const int NP = (mode == PW_GT) ? 9 : 3;
-    const double bflops = mode == PW_F ? 44.0 : (mode == PW_T ? 88.0 : 124.0);
-    return 4.0 * (24 + NP) * K.h1 * (double)Mvol + bflops * (double)Mvol;
-  }
-  double flops_pi_ba(int nper) const {
-    const double H1 = K.h1, K2 = K.k2, K3 = K.k3, M2 = M.n2, M3 = M.n3;
-    return 8.0 * 3 * nper * H1 * (K2 * M2 * M3 + K2 * K3 * M3);
+  // operations of one evaluation: its transforms and, roughly, the point products
+  double eval_flops(PwMode mode) const {
+    const double per_point[PW_MODES] = {30, 60, 60, 90, 21, 39, 18};
+    return grid_flops(M, mode_in(mode) + mode_out(mode)) + per_point[mode] * (double)Mvol;
   }
 
+  // One evaluation of a pseudo-spectral expression (PwMode) with sources srcA,
+  // srcB and projection epilogue e.  Its projection runs in the band phase of the
+  // next evaluation (one launch for both); flush() runs it when none follows.
   void eval(PwMode mode, T* slot, const C* srcA, const C* srcB, const PiEpi<T>& e, T* slot2 = nullptr);
+  void flush();
 
   // one band-limited sweep as a single persistent cooperative kernel
   void run_sweep(PwMode mode, const EvalDesc<T>* ev, int nev = 0);
-  // persistent sweeps pay off while the phases are latency-bound (small padded
-  // grids); beyond that one launch's worst-phase footprint costs occupancy
   static constexpr long long kPersistentMaxPadded = 32768;   // M1 M2 M3
-  // tensor-core image-grid transforms pay off once the grid write dominates
-  static constexpr long long kTensorMinVoxels = 1LL << 20;
-  bool use_tc() const {
-    return opts.tensor_cores == 2 || (opts.tensor_cores == 1 && Nvol >= kTensorMinVoxels);
-  }
-  // tensor-core iota A+B of the bracket evaluations: the per-evaluation
-  // launches of padded grids above the persistent-sweep size
-  bool use_tc_pad() const {
-    return !persistent() &&
-           (opts.tensor_cores == 2 || (opts.tensor_cores == 1 && Mvol > kPersistentMaxPadded));
-  }
   bool deform() const { return opts.state_eq == 1; }
   void state_form_only(const char* what) {
     if (!deform()) return;
     *err = std::string(what) + " is defined for the image state form only (opts.state_eq = 0)";
     throw Fail{LDDMM_EINVAL};
   }
+  // whether the options let sweeps run as persistent kernels (lddmm_batch_gn_solve
+  // refuses such contexts)
   bool persistent() const {
-    if (rec != nullptr || opts.persistent == 0) return false;
-    return opts.persistent == 2 || Mvol <= kPersistentMaxPadded;
+    return opts.persistent == 2 || (opts.persistent == 1 && Mvol <= kPersistentMaxPadded);
   }
-
-  // algorithmic flops of iota (or pi) of nf scalar fields on the image grid,
-  // Hermitian half spectrum along axis 1
-  double iota_flops(int nf) const {
-    const double H1 = K.h1, K2 = K.k2, K3 = K.k3;
-    return nf * (8.0 * H1 * (K2 * K3 * N.n3 + K2 * (double)N.n2 * N.n3) + 4.0 * H1 * (double)Nvol);
-  }
+  // and whether they do: on request only.  Two launches per evaluation, each
+  // starting as the one before drains, take less than the two grid barriers of a
+  // persistent kernel (us per shoot evaluation, launches / persistent: 9.4 / 11.3 at
+  // band 16^3, 50 / 51 at 2D 16^2 FP64).
+  bool run_persistent() const { return rec == nullptr && opts.persistent == 2; }
 
   // iota of `count` BL vectors (3 comps each) onto the image grid
   void to_grid(const C* hist, int count, T* grid);
@@ -355,7 +320,8 @@ struct Impl {
   void project_adjoint(const T* f3, C* out);
 
   // ------------------------------------------------------------- sweeps
-  T* slot(State<T>& S, int k) { return S.cache + (long long)k * cache_slot_elems<T>(pad); }
+  long long slot_elems() const { return (kSlotFields * Mvol + 3) / 4 * 4; }   // 16-byte aligned
+  T* slot(State<T>& S, int k) { return S.cache + k * slot_elems(); }
   C* vec(C* base, int n) { return base + (long long)n * 3 * Kvol; }
 
   // Heun shoot of BL EPDiff (Eq. 51); S.vh[0] must hold v0
@@ -371,19 +337,6 @@ struct Impl {
   void forward(State<T>& S);
 
   // ------------------------------------- deformation-state form (Section 3.3)
-  // Jacobian (d_j a_i in block 3 i + j) of band vector a and values of b onto
-  // the padded grid: iota fields base .. base + 11
-  void jac_val(IotaDesc<T>& d, int base, const C* a, const C* b);
-  // algorithmic flops of iota (or pi) of nf scalar fields on grid g
-  double grid_flops(const Dims& g, int nf) const {
-    const double H1 = K.h1, K2 = K.k2, K3 = K.k3;
-    return nf * (8.0 * H1 * (K2 * K3 * g.n3 + K2 * (double)g.n2 * g.n3) + 4.0 * H1 * (double)g.vol());
-  }
-  // one padded-grid product of the deformation form (def_products mode): iota
-  // of the fields {D a, b} into fl (defM when null), the product (mode 1 with
-  // the cached stage-point block {D u, v}) and pi with epilogue e
-  void def_eval(int mode, const C* a, const C* b, const PiEpi<T>& e, T* fl = nullptr,
-                const T* cached = nullptr);
   PiEpi<T> def_epi(bool applyK) const {
     PiEpi<T> e = epi(3, 1);
     e.grp[0] = 0;
@@ -393,7 +346,7 @@ struct Impl {
   }
 
   // padded-grid block {D u, v} of stage point k (2 n, 2 n + 1) of lin's sweep
-  T* def_slot(int k) { return defcache + (long long)k * 12 * Mvol; }
+  T* def_slot(int k) { return defcache + (long long)k * kDefFields * Mvol; }
 
   // Heun sweep of d/dt u~ = -v~ - D~u~ * v~ jointly with the shoot (stage 2 at
   // the EPDiff predictor v*_n), u~(0) = 0.  For lin the padded-grid fields of
@@ -422,7 +375,7 @@ struct Impl {
   void backward(State<T>& S);
 
   // incremental EPDiff (Eq. 30) from dvh[0], exact tangent of the Heun shoot
-  T* tslot(int k) { return tcache + (long long)k * cache_slot_elems<T>(pad); }
+  T* tslot(int k) { return tcache + k * slot_elems(); }
 
   // incremental BL EPDiff (Eq. 30) from dvh[0]; with cache, also stores the
   // padded-grid fields of dv_n and dv*_n (full-Newton products)

@@ -49,204 +49,200 @@ struct Band {
   __host__ __device__ long long vol() const { return (long long)k1 * k2 * k3; }
 };
 
-// Twiddle tables of one (grid, band) pair, device resident, precision T.
-//   E3f[k3][x3] = exp(+2 pi i f(k3) x3 / G3)          (iota, axis 3)
-//   E2f[k2][x2] = exp(+2 pi i f(k2) x2 / G2)          (iota, axis 2)
-//   E1f[h][x1]  = w(h) exp(+2 pi i h x1 / G1), w = 1 (h = 0) or 2
-//   E1b[x1][h]  = exp(-2 pi i h x1 / G1)              (pi, axis 1)
-//   E2b[x2][k2] = exp(-2 pi i f(k2) x2 / G2)
-//   E3b[x3][k3] = exp(-2 pi i f(k3) x3 / G3)
+// ---- band vectors ------------------------------------------------------------
+// A band-limited field is held as its real cosine/sine coefficients
+//   f(x) = sum V[q][h][2 s3 + s2][s1] phi_s1(h x1) phi_s2(a x2) phi_s3(b x3),
+// phi_0(k x) = cos(2 pi k x / G), phi_1 = sin, q = a K3h + b ("quad" of the
+// non-negative frequencies a, b of axes 2 and 3), h = 0..H1-1.  The K1 K2 K3
+// real degrees of freedom of a Hermitian array are stored once; the slots of
+// sin(0) are dead and hold zero (they take the place of the Nyquist slots).
+// A band vector is [3][Kq][H1][4][2] reals.
+struct Trig {
+  int H1, K2h, K3h;   // non-negative frequencies per axis (K/2; 1 for a degenerate axis)
+  __host__ __device__ int K1() const { return 2 * H1; }
+  __host__ __device__ int Kq() const { return K2h * K3h; }
+  __host__ __device__ long long vol() const { return (long long)Kq() * 2 * H1 * 4; }
+};
+__host__ __device__ inline Trig trig_of(const Band& b) { return Trig{b.h1, b.k2 / 2, b.k3 > 1 ? b.k3 / 2 : 1}; }
+
+// division by a fixed divisor n through a 32-bit reciprocal (m = 0: n = 1)
+struct FastDiv {
+  unsigned m;
+};
+inline FastDiv fast_div(int n) { return FastDiv{n <= 1 ? 0u : (unsigned)(0xffffffffu / (unsigned)n + 1u)}; }
+
+template <typename T>
+struct alignas(2 * sizeof(T)) Pair {
+  T x, y;
+};
+
+// ---- pseudo-spectral evaluations (dft.cu, sweep.cu) --------------------------
+// One evaluation on the padded plan: the scalar fields of a band vector pair
+// (A, B) on the product grid, point products, and the projection of the
+// product fields back to the band.  Writing m = L~B, Du for a Jacobian
+// (Du[i][j] = d_j u_i), the brackets are used in the form
+//   P(a, m) = (Da)^T m + (Dm) a + m div a = grad(a.m) - a x curl m + m div a
+//   Q(a, w) = Da w - Dw a
+// (Eqs. 4, 49): the gradient is applied to the projected scalar a.m, exactly
+// (truncated convolutions commute with spectral derivatives), so P needs ten
+// transformed fields (a, div a, m, curl m) and four projections (a.m and a
+// vector) in place of 24 and 3.  Modes, with their input and output fields:
+//   PW_F   P(A, m): inputs A, DA, m, curl m (18; all cached in slot); outputs a.m, vec
+//   PW_T   P(A, n) + P(v, m) with v, Dv, n, curl n cached: inputs A, div A, m,
+//          curl m (10); outputs the scalar and the vector
+//   PW_TC  the same from the 18 inputs of PW_F, which it stores in slot2
+//   PW_GT  P(v, m), P(A, n), Q(v, A): 18 inputs; outputs 4 + 4 + 3
+//   PW_D0  -(B + (DA) B): inputs DA, B (12; stored in slot unless null); outputs 3
+//   PW_D1  -(B + (DA) v + (Du) B), {Du, v} cached in slot: 12 inputs, 3 outputs
+//   PW_D2  B + (DA)^T B: 12 inputs, 3 outputs
+// A stage-point cache slot holds the 18 (or 12) fields of every product-grid point.
+enum PwMode : int { PW_F = 0, PW_T, PW_TC, PW_GT, PW_D0, PW_D1, PW_D2, PW_MODES };
+__host__ __device__ constexpr int mode_in(int m) { return m == PW_T ? 10 : (m >= PW_D0 ? 12 : 18); }
+__host__ __device__ constexpr int mode_out(int m) { return m == PW_GT ? 11 : (m >= PW_D0 ? 3 : 4); }
+__host__ __device__ constexpr int mode_nper(int m) { return m == PW_GT ? 3 : 1; }
+constexpr int kSlotFields = 18, kDefFields = 12, kMaxOutFields = 11, kMaxInFields = 18;
+
+// How an evaluation mode is cut into work items: the plane phase handles
+// `ppc` folded x2 pairs of one x1 plane per item (nparts items per plane), the
+// band phase 2^tqs quads per item.
+struct EvalGeom {
+  int ppc, nparts, tqs;
+};
+
+// Transform plan of one (grid, band) pair: the folded cosine/sine tables.  A
+// real sum over an axis of G points pairs x = t with x = G - t (t = 0..G/2):
+// cosines are even and sines odd in x, so both directions cost K/2 products
+// per point and K/2 tables rows.  Entries are (cos, sin) pairs.
+//   e1f[h][t], e1b[t][h]; e2f[a][t], e2b[t][a]; e3f[b][t], e3b[t][b]
+// zero-padded as the kernels stage them: rows of e1f to a multiple of 8 points, of
+// e1b to a multiple of 4 and of e2b to a multiple of 8 frequencies, of e3b to K3e
+// (even); e3f to K3e frequencies and e3b to NT3e points.
 template <typename T>
 struct Plan {
   Dims g;
   Band b;
-  cplx<T>* E3f;
-  cplx<T>* E2f;
-  cplx<T>* E1f;
-  cplx<T>* E1b;
-  cplx<T>* E2b;
-  cplx<T>* E3b;
-  // tile overrides of the bracket kernels, set by the autotuner (0: the size
-  // heuristics): tws 1 = twiddles from global memory, 2 = staged in shared
-  // memory (iota A+B); tp = pencils per tile (C/products/C'); kc = band rows
-  // per item (pi B'/A')
-  int tws = 0, tp = 0, kc = 0;
-  // split of the FP32 tensor-core image-grid transform: 0 3xTF32, 1 BF16x3
-  int split = 0;
-  // FP32 padded plans: the tcgen05 iota A+B twiddle operands, expanded once
-  // into the kernel's shared-memory layout (nullptr: expanded in the kernel)
-  const float* tc_ab = nullptr;
-  // FP32 padded plans: the tcgen05 pi B'+A' twiddle operands (real form, hi/lo,
-  // in the kernel's shared-memory layout); nullptr: the SIMT kernel runs
-  const float* tc_pi = nullptr;
-  // FP32 padded plans: the tcgen05 C / C' twiddle operands of the middle phase
-  // (tc_cpw.cu); with them set, tp is the tensor-core tile (8 pencils)
-  const float* tc_cpw = nullptr;
-  // the twiddle tiles exactly as the phase bodies stage them in shared memory
-  // (zero padded / transposed), so a phase copies them contiguously; nullptr:
-  // the phases build the tiles from the tables above
-  cplx<T>* E3fp = nullptr;   // [K3][G3e]  iota A (E3f, rows padded to even length)
-  cplx<T>* E2fp = nullptr;   // [K2][G2e]  iota B (E2f, padded to even length)
-  cplx<T>* E1fp = nullptr;   // [H1][G1q]  iota C (E1f, padded to a multiple of 4)
-  cplx<T>* E1bp = nullptr;   // [G1][H1q]  pi C' (E1b, padded to a multiple of 4)
-  cplx<T>* E3bt = nullptr;   // [K3][G3s]  pi A' (E3b transposed, bank-spread row stride)
+  Trig k;
+  int NT1, NT2, NT3;      // folded points per axis, G/2 + 1
+  int K3e, NT3e;          // even-rounded K3h and NT3
+  bool flat;              // 2D: one point and one frequency on axis 3
+  const Pair<T>*e1f, *e1b, *e2f, *e2b, *e3f, *e3b;
+  EvalGeom geom[PW_MODES];   // of the plan's evaluations (padded plans)
+  FastDiv dK3h, dK3p, dNT1, dNT3, dNT3h, dH1, dH1g;   // dK3p, dNT3h: pairs; dH1g: groups of 4 frequencies
 };
-
-// iota batch: field f is iota of (multiplier x one scalar band slab), where
-// the multiplier is L^(k) if applyL and 2 pi i f_deriv(k) if deriv >= 0.
-constexpr int kMaxIota = 36;
+inline int even_of(int n) { return n + (n & 1); }
 template <typename T>
-struct IotaDesc {
-  int nf;
-  const cplx<T>* src[kMaxIota];   // scalar band slab [K1][K2][K3]
-  T* dst[kMaxIota];               // grid field [G1][G2][G3]
-  signed char deriv[kMaxIota];    // -1 or axis 0..2
-  signed char applyL[kMaxIota];
-};
+void plan_sizes(Plan<T>& p, Dims g, const Band& b) {
+  p.g = g;
+  p.b = b;
+  p.k = trig_of(b);
+  p.NT1 = g.n1 / 2 + 1;
+  p.NT2 = g.n2 / 2 + 1;
+  p.NT3 = g.n3 / 2 + 1;
+  p.K3e = even_of(p.k.K3h);
+  p.flat = b.k3 == 1 && g.n3 == 1;
+  p.NT3e = even_of(p.NT3);
+  p.dK3h = fast_div(p.k.K3h);
+  p.dNT1 = fast_div(p.NT1);
+  p.dNT3 = fast_div(p.NT3);
+  p.dK3p = fast_div(p.K3e / 2);
+  p.dNT3h = fast_div((p.NT3 + 1) / 2);
+  p.dH1 = fast_div(p.k.H1);
+  p.dH1g = fast_div((p.k.H1 + 3) / 4);
+}
 
-// pi batch inputs: nf real grid fields.
-constexpr int kMaxPi = 36;
 template <typename T>
-struct PiSrc {
-  int nf;
-  const T* src[kMaxPi];
-};
+EvalGeom eval_geom(const Plan<T>& p, PwMode mode);
 
-// Epilogue of the last pi stage.  The pi fields are indexed f = o*ncomp + c
-// (o < nper).  For band slot k of component c:
-//   R_r(k) = sum_{o: grp[o]==r} coef[o] * (applyK[o] ? 1/L^(k) : 1) * pi_o(k)
-//   dst_j(k) = cR[j] * R_{r[j]}(k) + sum_i cX[j][i] * X[j][i](k)
-// coef includes the 1/(G1 G2 G3) normalisation.  X and dst are band vectors
-// [ncomp][K1][K2][K3]; outputs are written Hermitian with zero Nyquist slots.
-constexpr int kMaxPer = 3, kMaxOut = 4, kMaxX = 4;
+// Epilogue of a projection.  The projected fields are first combined into
+// ncomp-component fields Y_o (o < nper, see PwMode); then for band slot k of
+// component c
+//   dst_j(k) = sum_o cY[j][o] (applyK[o] ? 1/L^(k) : 1) Y_o(k) + sum_i cX[j][i] X_i(k)
+// cY includes the 1/(G1 G2 G3) normalisation.  X and dst are band vectors; a dst
+// may be one of the X terms.  jA, jB: outputs that are the sources A, B of the
+// evaluation that follows in the same launch (-1: read from memory).
+constexpr int kMaxPer = 3, kMaxOut = 4, kMaxTerm = 6;
 template <typename T>
 struct PiEpi {
   int ncomp, nper;
-  int grp[kMaxPer];
-  T coef[kMaxPer];
+  int grp[kMaxPer];          // host side: the output group and coefficient of each Y_o,
+  T coef[kMaxPer];           // folded into cY when an output is added
   int applyK[kMaxPer];
-  int nout;
-  cplx<T>* dst[kMaxOut];
-  int r[kMaxOut];
-  T cR[kMaxOut];
-  int nx[kMaxOut];
-  const cplx<T>* X[kMaxOut][kMaxX];
-  T cX[kMaxOut][kMaxX];
+  int nout, nterm;
+  int jA, jB;
+  T* dst[kMaxOut];
+  const T* X[kMaxTerm];
+  T cY[kMaxOut][kMaxPer];
+  T cX[kMaxOut][kMaxTerm];
 };
 
-// ---- transforms (dft.cu) --------------------------------------------------
-// Scratch: T2 holds [F][h1][G2][G3] complex (iota intermediate, and the C'
-// output of pi), P2 holds [9][h1][M2][M3] complex (C' of a bracket evaluation).
-// tc_flag != nullptr selects the tcgen05 3xTF32 form of stage C (FP32 plans
-// it supports); the kernel sets *tc_flag = 1 if its bounded MMA wait gives up.
-template <typename T>
-void iota_batch(const Plan<T>& p, const IotaDesc<T>& d, const T* Lhat, cplx<T>* T2,
-                cudaStream_t st, double* tc_flag = nullptr);
-// stage C of iota alone (T2 from bracket_iota): the tcgen05 form where
-// tc_flag != nullptr and the plan supports it, else the SIMT kernel
-template <typename T>
-void iota_c_stage(const Plan<T>& p, const IotaDesc<T>& d, cplx<T>* T2, cudaStream_t st, double* tc_flag);
-// stage C' of pi alone: the C' sums of s into P2 [nf][h1][G2][G3] (for bracket_pi)
-template <typename T>
-void pi_c_stage(const Plan<T>& p, const PiSrc<T>& s, cplx<T>* P2, cudaStream_t st);
-// tcgen05 image-grid stage C (tc_iota.cu)
-bool iota_C_tc_supported(const Plan<float>& p);
-// tcgen05 iota stages A + B of a padded-grid bracket block (tc_bracket.cu)
-bool iota_ab_tc_supported(const Plan<float>& p);
-// floats of the expanded twiddle operands, and the expansion into dst (device)
-size_t iota_ab_tc_twiddle_floats(const Plan<float>& p);
-cudaError_t iota_ab_tc_twiddles(const Plan<float>& p, float* dst, cudaStream_t st);
-cudaError_t iota_ab_tc(const Plan<float>& p, const IotaDesc<float>& d, const float* Lhat, float2* T2,
-                       double* flag, cudaStream_t st);
-cudaError_t iota_C_tc(const Plan<float>& p, const IotaDesc<float>& d, const float2* T2, double* flag,
-                      cudaStream_t st);
-// tcgen05 C + bracket products + C' of a padded-grid bracket block (tc_cpw.cu)
-enum PwMode : int;
-bool cpw_tc_supported(const Plan<float>& p);
-int cpw_tc_tile();
-size_t cpw_tc_twiddle_floats(const Plan<float>& p);
-cudaError_t cpw_tc_twiddles(const Plan<float>& p, float* dst, cudaStream_t st);
-cudaError_t cpw_tc(const Plan<float>& p, PwMode mode, const float2* T2, float* slot, float* slot2, float2* P2,
-                   double* flag, cudaStream_t st);
-// tcgen05 pi stages B' + A' with the epilogue on a padded-grid bracket block (tc_pi.cu)
-bool pi_ba_tc_supported(const Plan<float>& p);
-size_t pi_ba_tc_twiddle_floats(const Plan<float>& p);
-cudaError_t pi_ba_tc_twiddles(const Plan<float>& p, float* dst, cudaStream_t st);
-cudaError_t pi_ba_tc(const Plan<float>& p, const PiEpi<float>& e, const float* Lhat, const float2* P2,
-                     double* flag, cudaStream_t st);
-template <typename T>
-void pi_batch(const Plan<T>& p, const PiSrc<T>& s, const PiEpi<T>& e, const T* Lhat,
-              cplx<T>* P2, cudaStream_t st);
-// number of kernel launches of one iota_batch / pi_batch call
-constexpr int kIotaLaunches = 2, kPiLaunches = 2, kBracketLaunches = 3;
-
-enum PwMode : int { PW_F = 0, PW_T = 1, PW_GT = 2 };
-// One bracket evaluation on the padded plan p runs three kernels:
-//   bracket_iota  iota stages A+B of the 24 fields of d (layout per field
-//                 block: value[3], jac[3][3], Lvalue[3], Ljac[3][3], with
-//                 jac[c][j] = d_j a_c) -> T2;
-//   bracket_cpw   stage C, the bracket products and pi stage C' of the 3
-//                 (PW_F: P(v, L v); PW_T: P(dv, L v) + P(v, L dv)) or 9
-//                 (PW_GT: P(v, L U), P(W, L v), Q(v, W)) product fields -> P2;
-//                 slot holds the 24 fields of the stage point, written in PW_F
-//                 (d's own fields) and read in PW_T and PW_GT;
-//   bracket_pi    pi stages B'+A' of P2 and the epilogue e.
-template <typename T>
-void bracket_iota(const Plan<T>& p, const IotaDesc<T>& d, const T* Lhat, cplx<T>* T2, cudaStream_t st,
-                  double* tc_flag = nullptr);
-template <typename T>
-void bracket_cpw(const Plan<T>& p, PwMode mode, const cplx<T>* T2, T* slot, T* slot2, cplx<T>* P2,
-                 cudaStream_t st, double* tc_flag = nullptr);
-// tc_flag != nullptr selects the tcgen05 form (FP32 plans with p.tc_pi set)
-template <typename T>
-void bracket_pi(const Plan<T>& p, const PiEpi<T>& e, const T* Lhat, const cplx<T>* P2,
-                cudaStream_t st, double* tc_flag = nullptr);
-// One bracket evaluation of a persistent sweep: iota sources (value/Jacobian
-// block from srcA, L~ block from srcB), stage-point slot and pi epilogue.
+// One evaluation of a sweep.
 template <typename T>
 struct EvalDesc {
-  const cplx<T>* srcA;
-  const cplx<T>* srcB;
+  const T* A;
+  const T* B;
   T* slot;
-  T* slot2;      // tangent sweeps: where to cache the fields of A (nullptr: none)
+  T* slot2;
   PiEpi<T> epi;
 };
+
+// Band phase: projects the product fields P1 of the previous evaluation of the
+// same mode (unless prev is null or has no outputs), applies its epilogue, and
+// prepares the plane fields T1 of the next one (sources A and B, unless A is null).
+template <typename T>
+cudaError_t band_phase(const Plan<T>& p, PwMode mode, const PiEpi<T>* prev, const T* P1, const T* A, const T* B,
+                       T* T1, const T* Lhat, cudaStream_t st);
+// Plane phase: T1 -> fields on the product grid -> products -> P1.
+template <typename T>
+cudaError_t plane_phase(const Plan<T>& p, PwMode mode, const T* T1, T* slot, T* slot2, T* P1, cudaStream_t st);
 // Every evaluation of a band-limited sweep in one cooperative launch
 // (sweep.cu); ev is a device array of nev descriptors of one mode.  bar:
-// kSweepBarWords device unsigned ints of barrier state (the grid-barrier
-// arrival counter and one completion counter per (component, h) band slab);
-// flag: device double set to 1 if a wait gave up.  stall > 0 is the test hook
-// of the time-out path: the first grid barrier then waits for one arrival more
-// than the grid has and every wait gives up after `stall` polls.
-constexpr int kSweepBarWords = 128;
+// kSweepBarWords device unsigned ints of barrier state; flag: device double set
+// to 1 if a wait gave up.  stall > 0 is the test hook of the time-out path: the
+// first grid barrier then waits for one arrival more than the grid has and
+// every wait gives up after `stall` polls.
+constexpr int kSweepBarWords = 32;
 template <typename T>
-cudaError_t sweep_launch(const Plan<T>& p, PwMode mode, const EvalDesc<T>* ev, int nev, const T* Lhat,
-                         cplx<T>* T2, cplx<T>* P2, unsigned* bar, double* flag, cudaStream_t st,
-                         int stall = 0);
+cudaError_t sweep_launch(const Plan<T>& p, PwMode mode, const EvalDesc<T>* ev, int nev, const T* Lhat, T* T1,
+                         T* P1, unsigned* bar, double* flag, cudaStream_t st, int stall = 0);
+// elements of the two scratch arrays of evaluations on plan p
+template <typename T>
+long long eval_T1_elems(const Plan<T>& p);
+template <typename T>
+long long eval_P1_elems(const Plan<T>& p);
 
-// largest dynamic shared memory the transform kernels need on plan p when pi
-// batches hold up to nper_max fields per component and (brackets) bracket
-// evaluations run on it; SIZE_MAX if the plan's G3 is too long for the pi
-// kernel's accumulators.  smem_limit() is the configured maximum.
+// ---- image-grid transforms (dft.cu) ---------------------------------------
+// iota of nf scalar fields: band fields src[f] -> grid fields dst[f]
+constexpr int kMaxIota = 36;
 template <typename T>
-size_t max_smem_needed(const Plan<T>& p, int nper_max, bool brackets);
-size_t smem_limit();
-// floats of one stage-point cache slot of a bracket evaluation: the 24 grid
-// fields of every pencil tile of the C/products/C' phase, tile-major
-// [tile][24][M1][TP] so that a tile's fields are one contiguous block
+struct IotaList {
+  int nf;
+  const T* src[kMaxIota];
+  T* dst[kMaxIota];
+};
 template <typename T>
-long long cache_slot_elems(const Plan<T>& p);
-// row lengths of the staged twiddle tiles: G3e, G2e, G1q, H1q, G3s
+cudaError_t iota_fields(const Plan<T>& p, const IotaList<T>& d, T* T1, cudaStream_t st);
+// pi of nf <= 3 grid fields (components 0..nf-1) with epilogue e (nper = 1)
 template <typename T>
-void staged_twiddle_dims(const Plan<T>& p, int* G3e, int* G2e, int* G1q, int* H1q, int* G3s);
-// tile shapes in effect for a padded-grid plan (overrides or size heuristics):
-// twiddle staging of iota A+B (1 off, 2 on), pencils per tile of the
-// C/products/C' phase, band rows per pi B'/A' item (for 3 product fields)
+cudaError_t pi_fields(const Plan<T>& p, const T* const* src, const PiEpi<T>& e, const T* Lhat, T* P1,
+                      cudaStream_t st);
+// elements of the scratch: T1 of nf fields, P1 of three
 template <typename T>
-void tile_config(const Plan<T>& p, int* tws, int* tp, int* kc);
-// whether a tile override is usable on this plan
+long long iota_T1_elems(const Plan<T>& p, int nf);
 template <typename T>
-bool tile_valid(const Plan<T>& p, int tws, int tp, int kc);
+long long pi_P1_elems(const Plan<T>& p);
+constexpr int kIotaLaunches = 2, kPiLaunches = 2, kEvalLaunches = 2;
+
+// Hermitian complex band arrays [ncomp][K1][K2][K3] (symmetrised on the way in)
+// <-> band vectors; components beyond ncomp are not touched.
+template <typename T>
+void band_load(const cplx<T>* in, T* out, int ncomp, const Band& b, cudaStream_t st);
+template <typename T>
+void band_store(const T* in, cplx<T>* out, int ncomp, const Band& b, cudaStream_t st);
+
+// whether a grid and band of these sizes are accepted: nper product fields per
+// component are projected at once, `brackets`: evaluations run on the plan
+template <typename T>
+bool sizes_accepted(const Dims& g, const Band& b, int nper, bool brackets);
 
 // ---- grid kernels (grid.cu) -----------------------------------------------
 // Semi-Lagrangian state step (Eq. 52): m_next(x) = m(X_n(x)), foot point from
@@ -279,13 +275,6 @@ void def_sample(const T* I0, const T* gI0, const T* u, T* m1, T* gs, Dims g, cud
 template <typename T>
 void def_force(const T* gs, const T* m1, const T* I1, const T* du, T* dm_out, double c, T* f, long long vol,
                cudaStream_t st);
-// padded-grid products (blocks of 12 fields [12][vol]: Jacobian D[3 i + j] = d_j a_i,
-// then 3 values):
-//   0: out_i = -(v_i + D_ij v_j)                 fields {D u, v}
-//   1: out_i = -(dv_i + dD_ij v_j + D_ij dv_j)    fields {D du, dv}, cached {D u, v}
-//   2: out_i = r_i + D_ji r_j                     fields {D u, r}
-template <typename T>
-void def_products(int mode, const T* fields, const T* cached, T* out, long long vol, cudaStream_t st);
 // one reversed step of the exact discrete adjoint of the state transport:
 // lam_out (zeroed by the caller) and gcur gain atomic scatters, gnext gains the
 // per-voxel terms (see grid.cu); off is the step's stored displacement.
@@ -301,22 +290,20 @@ template <typename T>
 void scaled_diff(const T* a, const T* b, double c, T* out, long long n, cudaStream_t st);
 
 // ---- band vectors and reductions (grid.cu) --------------------------------
+// out = a x + b y (band vectors of n reals; y may be null).
 template <typename T>
-void hermitianize(const cplx<T>* in, cplx<T>* out, int ncomp, Band b, cudaStream_t st);
-// out = a x + b y (complex arrays of n entries; y may be null).
-template <typename T>
-void axpby(cplx<T>* out, double a, const cplx<T>* x, double bcoef, const cplx<T>* y,
-           long long n, cudaStream_t st);
+void axpby(T* out, double a, const T* x, double bcoef, const T* y, long long n, cudaStream_t st);
 // out = L^ x per band slot (V representative -> l2 gradient).
 template <typename T>
-void scale_L(cplx<T>* out, const cplx<T>* x, const T* Lhat, int ncomp, long long kvol, cudaStream_t st);
+void scale_L(T* out, const T* x, const T* Lhat, int ncomp, long long kvol, cudaStream_t st);
 // FP64 reductions written to a device double (deterministic two-pass tree).
 template <typename T>
 void sum_sq_diff(const T* a, const T* b, long long n, double* partial, double* out,
                  cudaStream_t st);
+// <a, b>_V = sum Lw a b, Lw = L^ times 1/2 per axis of nonzero frequency
 template <typename T>
-void inner_V(const cplx<T>* a, const cplx<T>* b, const T* Lhat, int ncomp, long long kvol,
-             double* partial, double* out, cudaStream_t st);
+void inner_V(const T* a, const T* b, const T* Lw, int ncomp, long long kvol, double* partial, double* out,
+             cudaStream_t st);
 constexpr int kReduceBlocks = 304;   // 2 x 152 SMs
 // device-resident conjugate-gradient scalars (grid.cu)
 enum PcgSlot { PCG_R = 0, PCG_B, PCG_DQ, PCG_A, PCG_RN, PCG_BETA, PCG_DONE, PCG_ITS, PCG_K, PCG_COPY,
@@ -326,7 +313,7 @@ void pcg_init(double* s, cudaStream_t st);                 // ||b|| = sqrt(rho),
 // (or the curvature stop) folded into their sum; x, r updates with the
 // <r, r>_V partials; beta (or the residual stop) folded into their sum; d
 template <typename T>
-void pcg_step(cplx<T>* x, cplx<T>* r, cplx<T>* d, const cplx<T>* q, const T* Lhat, long long kvol, int ncomp,
+void pcg_step(T* x, T* r, T* d, const T* q, const T* Lw, long long kvol, int ncomp,
               double* partial, double* s, double tol, cudaStream_t st);
 
 }  // namespace lddmm
