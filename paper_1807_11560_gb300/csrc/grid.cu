@@ -133,42 +133,33 @@ k_transport(const T* __restrict__ m, const T* __restrict__ vn, const T* __restri
   for (int j = 0; j < 3; ++j) off[j * vol + idx] = dsp[j];
 }
 
+// The incremental step is linear in dm and s along one characteristic, so what is
+// carried is the single grid q_n = dm_n - dt/2 s_n, s_n = grad m_n . dv_n:
+//   dm_{n+1} = q_n(X_n) - dt/2 s_{n+1},   q_{n+1} = q_n(X_n) - dt s_{n+1}
+// out = q(X) - c s: c = dt on the way, dt/2 for dm(1); q null: out = -c s (q_0).
+// HBM-bound with eight gathers in flight per voxel: 36 bytes are streamed (m and its
+// stencil, dv, the displacement, q read and written).
 template <typename T, bool G3D>
 __global__ void __launch_bounds__(kThreads)
-k_grad_dot(const T* __restrict__ m, const T* __restrict__ dv, T* __restrict__ s, Dims g) {
-  const long long vol = g.vol();
-  unsigned idx;
-  int ix[3];
-  if (!voxel<G3D>(g, idx, ix)) return;
-  T acc = T(0);
-#pragma unroll
-  for (int j = 0; j < 3; ++j) acc = fma(cdiff(m, ix, j, g), dv[j * vol + idx], acc);
-  s[idx] = acc;
-}
-
-template <typename T, bool G3D>
-__global__ void __launch_bounds__(kThreads)
-k_inc_step(const T* __restrict__ dm, const T* __restrict__ s, const T* __restrict__ mnext,
-           const T* __restrict__ dvn, const T* __restrict__ off, T* __restrict__ dmn,
-           T* __restrict__ sn, Dims g, T dt) {
+k_inc_step(const T* __restrict__ q, const T* __restrict__ m, const T* __restrict__ dv, const T* __restrict__ off,
+           T* __restrict__ out, Dims g, T c) {
   const long long vol = g.vol();
   unsigned idx;
   int ix[3];
   if (!voxel<G3D>(g, idx, ix)) return;
   const int n[3] = {g.n1, g.n2, g.n3};
-  T snew = T(0);
+  T s = T(0), v = T(0);
 #pragma unroll
-  for (int j = 0; j < 3; ++j) snew = fma(cdiff(mnext, ix, j, g), dvn[j * vol + idx], snew);
-  int c0[3], c1[3];
-  T w[3];
-  int o[8];
+  for (int j = 0; j < 3; ++j) s = fma(cdiff(m, ix, j, g), dv[j * vol + idx], s);
+  if (q != nullptr) {
+    int c0[3], c1[3], o[8];
+    T w[3];
 #pragma unroll
-  for (int j = 0; j < 3; ++j) cell(ix[j], off[j * vol + idx], n[j], c0[j], c1[j], w[j]);
-  corners(c0, c1, g.n2, g.n3, o);
-  const T dmi = dm ? trilin(dm, o, w) : T(0);
-  const T si = trilin(s, o, w);
-  dmn[idx] = dmi - T(0.5) * dt * (si + snew);
-  sn[idx] = snew;
+    for (int j = 0; j < 3; ++j) cell(ix[j], off[j * vol + idx], n[j], c0[j], c1[j], w[j]);
+    corners(c0, c1, g.n2, g.n3, o);
+    v = trilin(q, o, w);
+  }
+  out[idx] = fma(-c, s, v);
 }
 
 // weights of the 8 cell corners in the order of corners(); w = upper-node weights
@@ -516,22 +507,11 @@ void transport_step(const T* m, const T* vnext, const T* vcur, T* mnext, T* off,
 }
 
 template <typename T>
-void grad_dot(const T* m, const T* dv, T* s, Dims g, cudaStream_t st) {
+void inc_step(const T* q, const T* m, const T* dv, const T* off, T* out, Dims g, double c, cudaStream_t st) {
   if (plane_launch(g))
-    k_grad_dot<T, true><<<plane_grid(g), dim3(32, 8), 0, st>>>(m, dv, s, g);
+    k_inc_step<T, true><<<plane_grid(g), dim3(32, 8), 0, st>>>(q, m, dv, off, out, g, (T)c);
   else
-    k_grad_dot<T, false><<<blocks_for(g.vol()), kThreads, 0, st>>>(m, dv, s, g);
-}
-
-template <typename T>
-void inc_step(const T* dm, const T* s, const T* mnext, const T* dvnext, const T* off, T* dmnext,
-              T* snext, Dims g, double dt, cudaStream_t st) {
-  if (plane_launch(g))
-    k_inc_step<T, true><<<plane_grid(g), dim3(32, 8), 0, st>>>(dm, s, mnext, dvnext, off, dmnext, snext, g,
-                                                               (T)dt);
-  else
-    k_inc_step<T, false><<<blocks_for(g.vol()), kThreads, 0, st>>>(dm, s, mnext, dvnext, off, dmnext, snext,
-                                                                   g, (T)dt);
+    k_inc_step<T, false><<<blocks_for(g.vol()), kThreads, 0, st>>>(q, m, dv, off, out, g, (T)c);
 }
 
 template <typename T>
@@ -617,9 +597,7 @@ void def_force(const T* gs, const T* m1, const T* I1, const T* du, T* dm_out, do
                              cudaStream_t);                                                        \
   template void transport_step<T>(const T*, const T*, const T*, T*, T*, Dims, double,            \
                                   cudaStream_t);                                                 \
-  template void grad_dot<T>(const T*, const T*, T*, Dims, cudaStream_t);                         \
-  template void inc_step<T>(const T*, const T*, const T*, const T*, const T*, T*, T*, Dims,      \
-                            double, cudaStream_t);                                               \
+  template void inc_step<T>(const T*, const T*, const T*, const T*, T*, Dims, double, cudaStream_t);  \
   template void terminal_field<T>(const T*, const T*, int, double, T*, Dims, cudaStream_t);      \
   template void adjoint_step<T>(const T*, const T*, const T*, const T*, const T*, T*, T*, T*, Dims,  \
                                 double, cudaStream_t);                                              \

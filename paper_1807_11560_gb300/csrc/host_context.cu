@@ -144,10 +144,7 @@ void Impl<T>::create(int nd, const int* grid, const int* band, double a, int s_,
   alloc(zero3, (size_t)3 * Kvol);
   cuda(cudaMemset(zero3, 0, (size_t)3 * Kvol * sizeof(C)), "memset");
   alloc(dvgrid, (opts.recompute ? 2 : (size_t)Nt + 1) * 3 * Nvol);
-  for (int i = 0; i < 2; ++i) {
-    alloc(dm[i], (size_t)Nvol);
-    alloc(sb[i], (size_t)Nvol);
-  }
+  for (int i = 0; i < 2; ++i) alloc(dm[i], (size_t)Nvol);
   alloc(fterm, (size_t)3 * Nvol);
   if (deform()) {
     alloc(gI0, (size_t)3 * Nvol);

@@ -78,7 +78,8 @@ void Impl<T>::enqueue_hessvec(bool newton) {
     to_grid(S.vh, 1, vgr(S, 0));
     to_grid(dvh, 1, dvg(0));
   }
-  grad_dot<T>(mstate(S, 0), dvg(0), sb[0], N, st);
+  // q_0, then q_n along the characteristics; the last step leaves dm(1) (grid.cu)
+  inc_step<T>(nullptr, mstate(S, 0), dvg(0), nullptr, dm[0], N, 0.5 * dt, st);
   ++launches;
   for (int n = 0; n < Nt; ++n) {
     if (opts.recompute) {                   // step n + 1 of the state and velocity histories
@@ -87,8 +88,7 @@ void Impl<T>::enqueue_hessvec(bool newton) {
       state_step(S, n);
     }
     pb(PR_INC);
-    inc_step<T>(n == 0 ? nullptr : dm[n & 1], sb[n & 1], mstate(S, n + 1), dvg(n + 1), offp(S, n),
-                dm[(n + 1) & 1], sb[(n + 1) & 1], N, dt, st);
+    inc_step<T>(dm[n & 1], mstate(S, n + 1), dvg(n + 1), offp(S, n), dm[(n + 1) & 1], N, n + 1 < Nt ? dt : 0.5 * dt, st);
     pe(PR_INC, 12.0 * (double)Nvol);
   }
   launches += Nt;

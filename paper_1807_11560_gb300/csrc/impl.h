@@ -9,8 +9,8 @@
 //     BL history v_n, the Heun predictors v*_{n+1}, the 18 padded-grid fields
 //     (v, Dv, L v, curl L v) of every Heun stage point, the grid velocities
 //     iota(v_n), the state history m_n and the characteristic displacements;
-//   * the tangent history dv_n and its grid velocities, two ping-pong pairs
-//     for dm and s = grad m . dv, the transform scratch and BL temporaries;
+//   * the tangent history dv_n and its grid velocities, a ping-pong
+//     pair for the incremental transport, the transform scratch and BL temporaries;
 //   * with the deformation state equation (Section 3.3, opts.state_eq = 1):
 //     per trajectory the band-limited inverse-map displacement u_n and its
 //     predictors, the padded-grid fields {D u, v} of lin's stage points, and
@@ -101,7 +101,7 @@ struct Impl {
   T* tcache = nullptr;       // [2 Nt][18][Mvol] tangent stage-point fields (full Newton)
   C* zero3 = nullptr;        // [3][Kvol] zeros
   T* dvgrid = nullptr;       // [Nt+1][3][Nvol]  (recompute: [2][3][Nvol])
-  T *dm[2] = {nullptr, nullptr}, *sb[2] = {nullptr, nullptr};
+  T* dm[2] = {nullptr, nullptr};   // q_n of the incremental transport, ping-pong; dm(1) in dm[Nt & 1]
   T* fterm = nullptr;        // [3][Nvol]
   double *partial = nullptr, *dres = nullptr;   // dres[7]: sweep barrier time-out flag
   double* dpcg = nullptr;    // [PCG_SLOTS] device conjugate-gradient scalars

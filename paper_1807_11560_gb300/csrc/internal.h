@@ -250,14 +250,12 @@ bool sizes_accepted(const Dims& g, const Band& b, int nper, bool brackets);
 template <typename T>
 void transport_step(const T* m, const T* vnext, const T* vcur, T* mnext, T* off,
                     Dims g, double dt, cudaStream_t st);
-// s = grad m . dv (central differences).
+// One step of the incremental state (Eq. 31): out = q(X) - c grad m . dv with the
+// foot point X of the stored displacement, central differences; q null: q = 0.
+// With q_n = dm_n - dt/2 grad m_n . dv_n this carries the trapezoid source along
+// the characteristic (see grid.cu).
 template <typename T>
-void grad_dot(const T* m, const T* dv, T* s, Dims g, cudaStream_t st);
-// Incremental state step (Eq. 31) along the stored characteristic; dm may be
-// null (dm_0 = 0).
-template <typename T>
-void inc_step(const T* dm, const T* s, const T* mnext, const T* dvnext, const T* off,
-              T* dmnext, T* snext, Dims g, double dt, cudaStream_t st);
+void inc_step(const T* q, const T* m, const T* dv, const T* off, T* out, Dims g, double c, cudaStream_t st);
 // out_j = coef * r * d_j m, r = (m - y) if diff else y.
 template <typename T>
 void terminal_field(const T* m, const T* y, int diff, double coef, T* out, Dims g,
