@@ -21,7 +21,6 @@ using namespace dev;
 
 constexpr int kImgThreads = 256;
 constexpr int kIotaGroup = 3;     // fields per image-plane item (one velocity)
-constexpr int kIotaPT = 8;        // row pairs per thread of its k2 -> x2
 constexpr int kIotaBandGroup = 6; // fields per k1 -> x1 item
 constexpr int kSMs = 152;         // sizing only: fixed, so that sums never depend on the device
 
@@ -92,6 +91,7 @@ k_plane_flat(const __grid_constant__ Plan<T> p, const T* T1, T* slot, T* slot2, 
 
 // ---- image grid ----------------------------------------------------------------
 constexpr int kChunk = 32;        // folded x1 points per twiddle chunk
+constexpr int kIotaPT = 8;        // row pairs per thread of k2 -> x2
 
 template <typename T>
 __global__ void __launch_bounds__(kImgThreads)
@@ -122,29 +122,28 @@ k_iota_band(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList<
   }
 }
 
-// One x1 plane, ppc row pairs, up to three fields.  k3 -> x3 costs K3/2 products
-// per point and dominates: a lane owns TL points t (and their partners G3 - t) of
-// RB rows, so a row's coefficients are read once per warp (broadcast) and a
-// twiddle once per RB rows.
+// iota of up to three fields on `ppi` row pairs of one x1 plane.  k3 -> x3 costs
+// K3/2 products per point and dominates: a lane owns TL points t (and their
+// partners G3 - t) of RB rows, so a row's coefficients are read once per warp
+// (broadcast) and a twiddle once per RB rows.
 template <typename T, int TL, int RB>
 __global__ void __launch_bounds__(kImgThreads)
-k_iota_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList<T> d, int ppc, const T* T1) {
+k_iota_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList<T> d, int ppi, const T* T1) {
   extern __shared__ __align__(16) unsigned char smraw[];
   V2<T>* sm = reinterpret_cast<V2<T>*>(smraw);
   const int f0 = blockIdx.y * kIotaGroup, NF = min(kIotaGroup, d.nf - f0), x1 = blockIdx.z;
-  const int t0 = blockIdx.x * ppc, np = min(ppc, p.NT2 - t0);
-  const PlaneShape<T> s = plane_shape(p, kIotaGroup, 0, ppc, kIotaPT);
+  const int t0 = blockIdx.x * ppi, np = min(ppi, p.NT2 - t0);
+  const PlaneShape<T> s = plane_shape(p, kIotaGroup, 0, ppi, kIotaPT);
   const int R = s.R, K3e = p.K3e, K3s = s.K3s, NT3 = p.NT3, G2 = p.g.n2, G3 = p.g.n3;
-  const long long Kq = p.k.Kq();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   V2<T>* S1 = sm + s.off_s;
   pdl_trigger();
   plane_tables<T, kImgThreads, kIotaPT>(p, s, t0, np, true, false, sm);
   pdl_wait();
   __syncthreads();
-  rows_from_band<T, kImgThreads, kIotaGroup, kIotaPT>(p, T1 + ((long long)x1 * d.nf + f0) * Kq * 4, NF, np, s,
-                                                sm + s.off_2f, S1);
+  rows_from_band<T, kImgThreads, kIotaGroup, kIotaPT>(p, T1 + ((long long)x1 * d.nf + f0) * p.k.Kq() * 4, NF, np, s,
+                                                      sm + s.off_2f, S1);
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ntb = (NT3 + 32 * TL - 1) / (32 * TL), nrb = (2 * np + RB - 1) / RB;
   for (int it = warp; it < NF * nrb * ntb; it += kImgThreads / 32) {
     const int tb = it % ntb, r = it / ntb;
@@ -154,11 +153,11 @@ k_iota_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList
     for (int i = 0; i < RB; ++i)
 #pragma unroll
       for (int j = 0; j < TL; ++j) acc[i][j] = zero2<T>();
-    const V2<T>* v = S1 + (f * R + row0) * K3s;
-    int tt[TL];
+    int tt[TL], rr[RB];
 #pragma unroll
     for (int j = 0; j < TL; ++j) tt[j] = min(tb * 32 * TL + 32 * j + lane, NT3 - 1);
-    const int last = 2 * np - 1 - row0;                    // rows past the item repeat its last row
+#pragma unroll
+    for (int i = 0; i < RB; ++i) rr[i] = (f * R + min(row0 + i, 2 * np - 1)) * K3s;   // past the item: its last row
     for (int b = 0; b < K3e; b += 2) {
       V2<T> w0[TL], w1[TL];
 #pragma unroll
@@ -169,7 +168,7 @@ k_iota_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList
 #pragma unroll
       for (int i = 0; i < RB; ++i) {
         V2<T> a0, a1;
-        ld2(v + min(i, last) * K3s + b, a0, a1);
+        ld2(S1 + rr[i] + b, a0, a1);
 #pragma unroll
         for (int j = 0; j < TL; ++j) acc[i][j] = fma2(a1, w1[j], fma2(a0, w0[j], acc[i][j]));
       }
@@ -193,41 +192,53 @@ k_iota_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList
   }
 }
 
-// Part of one x1 plane of grid field f: rows folded along x3 into shared memory,
-// x3 -> k3, then x2 -> k2 as a partial plane.
-template <typename T>
+// the projected field (PiKind) at a point, formed as the rows are folded
+template <typename T, int KIND>
+__device__ __forceinline__ T pi_source(const T* __restrict__ fld, const PiField<T>& s, const Dims& g, int f, int x1,
+                                       int x2, int x3) {
+  const long long at = ((long long)x1 * g.n2 + x2) * g.n3 + x3;
+  if (KIND == PI_FIELD) return fld[at];
+  const int n = f == 0 ? g.n1 : (f == 1 ? g.n2 : g.n3), x = f == 0 ? x1 : (f == 1 ? x2 : x3);
+  const long long st = f == 0 ? (long long)g.n2 * g.n3 : (f == 1 ? g.n3 : 1);
+  const long long up = at + (x + 1 == n ? (1 - n) : 1) * st, dn = at + (x == 0 ? n - 1 : -1) * st;
+  const T h = T(0.5) * T(n);
+  const T dm = (s.m[up] - s.m[dn]) * h;
+  if (KIND == PI_RESIDUAL) return s.c * (s.m[at] - s.y[at]) * dm;
+  if (KIND == PI_INCREMENT) return s.c * s.y[at] * dm;
+  return s.c * (s.dm[at] * dm + (s.m[at] - s.y[at]) * ((s.dm[up] - s.dm[dn]) * h));
+}
+
+// pi of `ppi` row pairs of one x1 plane of one field: the rows folded along x3 into
+// shared memory, x3 -> k3, then x2 -> k2 as a partial plane.
+template <typename T, int KIND>
 __global__ void __launch_bounds__(kImgThreads)
-k_pi_plane(const __grid_constant__ Plan<T> p, const T* f0, const T* f1, const T* f2, int ppc, T* __restrict__ P1) {
+k_pi_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ PiField<T> src, int ppi, T* __restrict__ P1) {
   extern __shared__ __align__(16) unsigned char smraw[];
   V2<T>* sm = reinterpret_cast<V2<T>*>(smraw);
-  const int part = blockIdx.x, f = blockIdx.y, x1 = blockIdx.z;
-  const int t0 = part * ppc, np = min(ppc, p.NT2 - t0);
-  const PlaneShape<T> s = plane_shape(p, 0, 1, ppc, 1);
+  const int f = blockIdx.y, x1 = blockIdx.z, t0 = blockIdx.x * ppi, np = min(ppi, p.NT2 - t0);
+  const PlaneShape<T> s = plane_shape(p, 0, 1, ppi, 1);
   const int NT3 = p.NT3, NT3e = p.NT3e, G2 = p.g.n2, G3 = p.g.n3;
-  const long long Kq = p.k.Kq();
   V2<T>*Z = sm + s.off_s, *sP = sm + s.off_p;
   pdl_trigger();
   plane_tables<T, kImgThreads, 1>(p, s, t0, np, false, true, sm);
   pdl_wait();
-  const T* __restrict__ src = (f == 0 ? f0 : (f == 1 ? f1 : f2)) + (long long)x1 * G2 * G3;
+  const T* fld = src.f[f];
 #pragma unroll 4
   for (int it = threadIdx.x; it < 2 * np * NT3; it += kImgThreads) {
-    const int row = fdiv(it, p.dNT3), t = it - row * NT3;
-    const int u = t0 + (row >> 1);
-    const bool two = t > 0 && 2 * t != G3;
-    const bool live = !((row & 1) && (u == 0 || 2 * u == G2));
-    const T* v = src + (long long)((row & 1) && live ? G2 - u : u) * G3;
-    const T a = v[t], b = two ? v[G3 - t] : T(0);
+    const int row = fdiv(it, p.dNT3), t = it - row * NT3, u = t0 + (row >> 1);
+    const bool live = !((row & 1) && (u == 0 || 2 * u == G2)), two = t > 0 && 2 * t != G3;
+    const int x2 = (row & 1) && live ? G2 - u : u;
+    const T a = pi_source<T, KIND>(fld, src, p.g, f, x1, x2, t);
+    const T b = pi_source<T, KIND>(fld, src, p.g, f, x1, x2, two ? G3 - t : t);
     V2<T>* o = sP + row * NT3e + t;
     *o = two ? mk2(a + b, a - b) : mk2(a, T(0));
     if (t == NT3 - 1 && NT3e > NT3) o[1] = zero2<T>();
   }
   __syncthreads();
-  rows_to_k3<T, kImgThreads, 1, 1>(p, sP, t0, ppc, np, sm + s.off_3b, Z);
+  rows_to_k3<T, kImgThreads, 1, 1>(p, sP, t0, ppi, np, sm + s.off_3b, Z);
   __syncthreads();
-  T* out = P1 + (((long long)x1 * gridDim.x + part) * gridDim.y + f) * Kq * 4;
-  if (p.k.K2h >= 16) band_from_rows<T, kImgThreads, 1, 8>(p, Z, ppc, np, sm + s.off_2b, out);
-  else band_from_rows<T, kImgThreads, 1, 4>(p, Z, ppc, np, sm + s.off_2b, out);
+  T* out = P1 + (((long long)x1 * gridDim.x + blockIdx.x) * gridDim.y + f) * p.k.Kq() * 4;
+  band_from_rows<T, kImgThreads, 1, 2>(p, Z, ppi, np, sm + s.off_2b, out);
 }
 
 // the two plane steps of a 2D image: one output per thread
@@ -250,21 +261,22 @@ k_iota_plane_flat(const __grid_constant__ Plan<T> p, const __grid_constant__ Iot
   o[t] = E + O;
   if (t > 0 && 2 * t != G2) o[G2 - t] = E - O;
 }
-template <typename T>
+template <typename T, int KIND>
 __global__ void __launch_bounds__(kImgThreads)
-k_pi_plane_flat(const __grid_constant__ Plan<T> p, const T* f0, const T* f1, const T* f2, T* __restrict__ P1) {
+k_pi_plane_flat(const __grid_constant__ Plan<T> p, const __grid_constant__ PiField<T> src, T* __restrict__ P1) {
   const int K2h = p.k.K2h, K2p = up8(K2h), G2 = p.g.n2, a = blockIdx.x * kImgThreads + threadIdx.x, f = blockIdx.y,
             x1 = blockIdx.z;
   pdl_trigger();
   pdl_wait();
   if (a >= K2h) return;
-  const T* __restrict__ src = (f == 0 ? f0 : (f == 1 ? f1 : f2)) + (long long)x1 * G2;
+  const T* fld = src.f[f];
   const V2<T>* w = reinterpret_cast<const V2<T>*>(p.e2b) + a;
   V2<T> acc = zero2<T>();
 #pragma unroll 4
   for (int t = 0; t < p.NT2; ++t) {
     const bool two = t > 0 && 2 * t != G2;
-    const T u = src[t], v = two ? src[G2 - t] : T(0);
+    const T u = pi_source<T, KIND>(fld, src, p.g, f, x1, t, 0);
+    const T v = two ? pi_source<T, KIND>(fld, src, p.g, f, x1, G2 - t, 0) : T(0);
     acc = fma2(two ? mk2(u + v, u - v) : mk2(u, T(0)), w[(long long)t * K2p], acc);
   }
   stq(P1 + (((long long)x1 * gridDim.y + f) * K2h + a) * 4, Quad<T>{acc, zero2<T>()});
@@ -416,12 +428,24 @@ int band_tqs(const Plan<T>& p, int mode) {
   return s;
 }
 
-int iota_ppc(int NT2) { return std::min(NT2, 16); }
-int pi_ppc(int NT2) { return std::min(NT2, 8); }
+// Row pairs per image-plane item: as many as give every thread a k2 -> x2 (or x3 ->
+// k3) sum, so that one pass of loads feeds the item, then cut evenly.
+inline int even_pairs(int NT2, int most, int step) {
+  const int parts = (NT2 + most - 1) / most, pairs = (NT2 + parts - 1) / parts;
+  return (pairs + step - 1) / step * step;
+}
 template <typename T>
-int fit_ppc(const Plan<T>& p, int NF, int NO, int ppc) {
-  while (ppc > 1 && plane_shape(p, NF, NO, ppc, NF > 0 ? kIotaPT : 1).smem > (size_t)96 * 1024) --ppc;
-  return ppc;
+int iota_pairs(const Plan<T>& p) {
+  int most = std::max(1, kImgThreads / (kIotaGroup * p.k.K3h)) * kIotaPT;
+  while (most > kIotaPT && plane_shape(p, kIotaGroup, 0, most, kIotaPT).smem > (size_t)96 * 1024) most -= kIotaPT;
+  return even_pairs(p.NT2, most, kIotaPT);
+}
+template <typename T>
+int pi_pairs(const Plan<T>& p) {
+  if (p.flat) return p.NT2;
+  int most = std::max(1, 2 * kImgThreads / p.K3e);
+  while (most > 1 && plane_shape(p, 0, 1, most, 1).smem > (size_t)96 * 1024) --most;
+  return even_pairs(p.NT2, most, 1);
 }
 
 template <typename T, int MODE, int PT, int TT>
@@ -484,13 +508,26 @@ cudaError_t launch_band(const Plan<T>& p, const PiEpi<T>* prev, const T* P1, con
 
 template <typename T, int TL, int RB>
 cudaError_t launch_iota_plane(const Plan<T>& p, const IotaList<T>& d, const T* T1, cudaStream_t st) {
-  const int ppc = fit_ppc(p, kIotaGroup, 0, iota_ppc(p.NT2));
+  const unsigned groups = (unsigned)((d.nf + kIotaGroup - 1) / kIotaGroup);
+  const int ppi = iota_pairs(p);
   cudaError_t e = allow_smem<k_iota_plane<T, TL, RB>>();
   if (e != cudaSuccess) return e;
-  const dim3 grid((unsigned)((p.NT2 + ppc - 1) / ppc), (unsigned)((d.nf + kIotaGroup - 1) / kIotaGroup),
-                  (unsigned)p.g.n1);
-  return launch_chain(k_iota_plane<T, TL, RB>, grid, kImgThreads, plane_shape(p, kIotaGroup, 0, ppc, kIotaPT).smem, st, p, d,
-                      ppc, T1);
+  return launch_chain(k_iota_plane<T, TL, RB>,
+                      dim3((unsigned)((p.NT2 + ppi - 1) / ppi), groups, (unsigned)p.g.n1), kImgThreads,
+                      plane_shape(p, kIotaGroup, 0, ppi, kIotaPT).smem, st, p, d, ppi, T1);
+}
+
+template <typename T, int KIND>
+cudaError_t launch_pi_plane(const Plan<T>& p, const PiField<T>& s, int nf, T* P1, cudaStream_t st) {
+  if (p.flat)
+    return launch_chain(k_pi_plane_flat<T, KIND>,
+                        dim3((unsigned)((p.k.K2h + kImgThreads - 1) / kImgThreads), (unsigned)nf, (unsigned)p.g.n1),
+                        kImgThreads, 0, st, p, s, P1);
+  const int ppi = pi_pairs(p);
+  cudaError_t e = allow_smem<k_pi_plane<T, KIND>>();
+  if (e != cudaSuccess) return e;
+  return launch_chain(k_pi_plane<T, KIND>, dim3((unsigned)((p.NT2 + ppi - 1) / ppi), (unsigned)nf, (unsigned)p.g.n1),
+                      kImgThreads, plane_shape(p, 0, 1, ppi, 1).smem, st, p, s, ppi, P1);
 }
 
 }  // namespace
@@ -588,26 +625,19 @@ cudaError_t iota_fields(const Plan<T>& p, const IotaList<T>& d, T* T1, cudaStrea
 
 template <typename T>
 long long pi_P1_elems(const Plan<T>& p) {
-  const int ppc = fit_ppc(p, 0, 1, pi_ppc(p.NT2));
-  return (long long)p.g.n1 * ((p.NT2 + ppc - 1) / ppc) * 3 * p.k.Kq() * 4;
+  const int ppi = pi_pairs(p);
+  return (long long)p.g.n1 * ((p.NT2 + ppi - 1) / ppi) * 3 * p.k.Kq() * 4;
 }
 template <typename T>
-cudaError_t pi_fields(const Plan<T>& p, const T* const* src, const PiEpi<T>& e, const T* Lhat, T* P1,
+cudaError_t pi_fields(const Plan<T>& p, PiKind kind, const PiField<T>& s, const PiEpi<T>& e, const T* Lhat, T* P1,
                       cudaStream_t st) {
-  const int nf = e.ncomp;
-  int nparts = 1;
+  const int nf = e.ncomp, ppi = pi_pairs(p), nparts = (p.NT2 + ppi - 1) / ppi;
   cudaError_t rc;
-  if (p.flat) {
-    rc = launch_chain(k_pi_plane_flat<T>,
-                      dim3((unsigned)((p.k.K2h + kImgThreads - 1) / kImgThreads), (unsigned)nf, (unsigned)p.g.n1),
-                      kImgThreads, 0, st, p, src[0], src[nf > 1 ? 1 : 0], src[nf > 2 ? 2 : 0], P1);
-  } else {
-    const int ppc = fit_ppc(p, 0, 1, pi_ppc(p.NT2));
-    nparts = (p.NT2 + ppc - 1) / ppc;
-    if ((rc = allow_smem<k_pi_plane<T>>()) != cudaSuccess) return rc;
-    rc = launch_chain(k_pi_plane<T>, dim3((unsigned)nparts, (unsigned)nf, (unsigned)p.g.n1), kImgThreads,
-                      plane_shape(p, 0, 1, ppc, 1).smem, st, p, src[0], src[nf > 1 ? 1 : 0], src[nf > 2 ? 2 : 0], ppc,
-                      P1);
+  switch (kind) {
+    case PI_FIELD: rc = launch_pi_plane<T, PI_FIELD>(p, s, nf, P1, st); break;
+    case PI_RESIDUAL: rc = launch_pi_plane<T, PI_RESIDUAL>(p, s, nf, P1, st); break;
+    case PI_INCREMENT: rc = launch_pi_plane<T, PI_INCREMENT>(p, s, nf, P1, st); break;
+    default: rc = launch_pi_plane<T, PI_NEWTON>(p, s, nf, P1, st); break;
   }
   if (rc != cudaSuccess) return rc;
   const int tqs = p.k.Kq() >= 2 * kSMs ? 1 : 0, PC = 4 << tqs, H1 = p.k.H1;
@@ -676,7 +706,8 @@ bool sizes_accepted(const Dims& g, const Band& b, int nper, bool brackets) {
   template long long iota_T1_elems<T>(const Plan<T>&, int);                                                        \
   template cudaError_t iota_fields<T>(const Plan<T>&, const IotaList<T>&, T*, cudaStream_t);                       \
   template long long pi_P1_elems<T>(const Plan<T>&);                                                               \
-  template cudaError_t pi_fields<T>(const Plan<T>&, const T* const*, const PiEpi<T>&, const T*, T*, cudaStream_t); \
+  template cudaError_t pi_fields<T>(const Plan<T>&, PiKind, const PiField<T>&, const PiEpi<T>&, const T*, T*,      \
+                                    cudaStream_t);                                                                 \
   template void band_load<T>(const cplx<T>*, T*, int, const Band&, cudaStream_t);                                  \
   template void band_store<T>(const T*, cplx<T>*, int, const Band&, cudaStream_t);                                 \
   template bool sizes_accepted<T>(const Dims&, const Band&, int, bool);

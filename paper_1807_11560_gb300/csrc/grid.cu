@@ -1,7 +1,6 @@
 // Grid-point kernels of the GB300 LDDMM library (sm_103a):
 //   * semi-Lagrangian state and incremental-state transport on the image grid
 //     (Eqs. 52 and 31),
-//   * terminal adjoint fields lambda(1) grad m(1) (Eq. 55, Eq. 58 under GN),
 //   * band-vector updates and deterministic FP64 reductions (Eq. 47, Eq. 50),
 //   * the deformation-state form (Section 3.3): terminal sampling of I0 at the
 //     inverse map, its force fields, and the padded-grid products of the
@@ -243,40 +242,11 @@ k_adj_step(const T* __restrict__ lam, const T* __restrict__ m, const T* __restri
 
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
-k_terminal_newton(const T* __restrict__ m, const T* __restrict__ y, const T* __restrict__ dm, T c,
-                  T* __restrict__ out, Dims g) {
-  const long long vol = g.vol();
-  const unsigned idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= vol) return;
-  int ix[3];
-  unflat(idx, g.n2, g.n3, ix);
-  const T d = dm[idx], r = m[idx] - y[idx];
-#pragma unroll
-  for (int j = 0; j < 3; ++j) out[j * vol + idx] = c * (d * cdiff(m, ix, j, g) + r * cdiff(dm, ix, j, g));
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
 k_scaled_diff(const T* __restrict__ a, const T* __restrict__ b, T c, T* __restrict__ out, long long n) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = c * (a[i] - b[i]);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
-k_terminal(const T* __restrict__ m, const T* __restrict__ y, int diff, T coef, T* __restrict__ out,
-           Dims g) {
-  const long long vol = g.vol();
-  const unsigned idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= vol) return;
-  int ix[3];
-  unflat(idx, g.n2, g.n3, ix);
-  const T r = coef * (diff ? (m[idx] - y[idx]) : y[idx]);
-#pragma unroll
-  for (int j = 0; j < 3; ++j) out[j * vol + idx] = r * cdiff(m, ix, j, g);
-}
-
-// ---- band vectors -----------------------------------------------------------------
 // ---- conjugate gradients with device-resident scalars (Eq. 45) ------------------
 // s[] holds rho, ||b||, <d, Hd>, alpha, rho_new, beta, the stop flag, the
 // iterations done, the iteration counter and the "x = d" flag; every update
@@ -522,18 +492,8 @@ void adjoint_step(const T* lam, const T* m, const T* vcur, const T* vnext, const
 }
 
 template <typename T>
-void terminal_newton(const T* m, const T* y, const T* dm, double c, T* out, Dims g, cudaStream_t st) {
-  k_terminal_newton<T><<<blocks_for(g.vol()), kThreads, 0, st>>>(m, y, dm, (T)c, out, g);
-}
-
-template <typename T>
 void scaled_diff(const T* a, const T* b, double c, T* out, long long n, cudaStream_t st) {
   k_scaled_diff<T><<<blocks_for(n), kThreads, 0, st>>>(a, b, (T)c, out, n);
-}
-
-template <typename T>
-void terminal_field(const T* m, const T* y, int diff, double coef, T* out, Dims g, cudaStream_t st) {
-  k_terminal<T><<<blocks_for(g.vol()), kThreads, 0, st>>>(m, y, diff, (T)coef, out, g);
 }
 
 template <typename T>
@@ -598,11 +558,9 @@ void def_force(const T* gs, const T* m1, const T* I1, const T* du, T* dm_out, do
   template void transport_step<T>(const T*, const T*, const T*, T*, T*, Dims, double,            \
                                   cudaStream_t);                                                 \
   template void inc_step<T>(const T*, const T*, const T*, const T*, T*, Dims, double, cudaStream_t);  \
-  template void terminal_field<T>(const T*, const T*, int, double, T*, Dims, cudaStream_t);      \
   template void adjoint_step<T>(const T*, const T*, const T*, const T*, const T*, T*, T*, T*, Dims,  \
                                 double, cudaStream_t);                                              \
   template void scaled_diff<T>(const T*, const T*, double, T*, long long, cudaStream_t);          \
-  template void terminal_newton<T>(const T*, const T*, const T*, double, T*, Dims, cudaStream_t);  \
   template void axpby<T>(T*, double, const T*, double, const T*, long long,    \
                          cudaStream_t);                                                          \
   template void scale_L<T>(T*, const T*, const T*, int, long long, cudaStream_t);    \

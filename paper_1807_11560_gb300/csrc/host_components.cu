@@ -34,13 +34,13 @@ void Impl<T>::pi_call(const void* f, int ncomp, void* out) {
     const int nc = std::min(3, ncomp - c0);
     cuda(cudaMemcpyAsync(fterm, (const T*)f + (long long)c0 * Nvol, (size_t)nc * Nvol * sizeof(T),
                          cudaMemcpyDefault, st), "copy");
-    const T* src[3] = {fterm, fterm + Nvol, fterm + 2 * Nvol};
+    const PiField<T> src{{fterm, fterm + Nvol, fterm + 2 * Nvol}, nullptr, nullptr, nullptr, T(0)};
     PiEpi<T> e = epi(nc, 1);
     e.grp[0] = 0;
     e.coef[0] = (T)(1.0 / (double)Nvol);
     e.applyK[0] = 0;
     add_out(e, vout, 0, 1.0, {});
-    cuda(pi_fields<T>(full, src, e, Lhat, P1, st), "pi");
+    cuda(pi_fields<T>(full, PI_FIELD, src, e, Lhat, P1, st), "pi");
     band_store<T>(vout, zout, nc, K, st);
     launches += kPiLaunches + 1;
     check_launch("pi");
@@ -113,9 +113,7 @@ void Impl<T>::transport_vjp(const void* v0, const void* gm1, void* out) {
   forward(lin);
   cuda(cudaMemcpyAsync(dm[0], gm1, (size_t)Nvol * sizeof(T), cudaMemcpyDefault, st), "copy grad m1");
   // lambda(1) = -N dL/dm(1): the L2_h adjoint of the grid values
-  terminal_field<T>(m1(lin), dm[0], 0, -(double)Nvol, fterm, N, st);
-  ++launches;
-  project_K(fterm, U);
+  project_terminal(PI_INCREMENT, m1(lin), dm[0], nullptr, -(double)Nvol, U);
   backward(lin);
   scale_L<T>(gbuf, W, Lhat, 3, Kvol, st);
   ++launches;

@@ -92,12 +92,11 @@ void Impl<T>::enqueue_hessvec(bool newton) {
     pe(PR_INC, 12.0 * (double)Nvol);
   }
   launches += Nt;
+  const double lam = -2.0 / (sigma * sigma);
   if (newton)
-    terminal_newton<T>(m1(S), I1, dm[Nt & 1], -2.0 / (sigma * sigma), fterm, N, st);
+    project_terminal(PI_NEWTON, m1(S), I1, dm[Nt & 1], lam, U);
   else
-    terminal_field<T>(m1(S), dm[Nt & 1], 0, -2.0 / (sigma * sigma), fterm, N, st);
-  ++launches;
-  project_K(fterm, U);
+    project_terminal(PI_INCREMENT, m1(S), dm[Nt & 1], nullptr, lam, U);
   if (newton)
     newton_backward(S);
   else
@@ -156,9 +155,7 @@ double Impl<T>::gradient_tail(C* gdev) {
     project_K(fterm, rhob, false);
     terminal_deform(rhob, vec(lin.uh, Nt), vec(Uh, Nt));
   } else {
-    terminal_field<T>(m1(lin), I1, 1, -2.0 / (sigma * sigma), fterm, N, st);
-    ++launches;
-    project_K(fterm, vec(Uh, Nt));
+    project_terminal(PI_RESIDUAL, m1(lin), I1, nullptr, -2.0 / (sigma * sigma), vec(Uh, Nt));
   }
   backward_hist(lin);
   axpby<T>(gdev, 1.0, lin.vh, 1.0, Wh, 3 * Kvol, st);

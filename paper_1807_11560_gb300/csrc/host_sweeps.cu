@@ -70,31 +70,32 @@ void Impl<T>::to_grid(const C* hist, int count, T* grid) {
 }
 
 template <typename T>
-void Impl<T>::project_K(const T* f3, C* out, bool applyK) {
-  const T* src[3] = {f3, f3 + Nvol, f3 + 2 * Nvol};
+void Impl<T>::project(PiKind kind, const PiField<T>& f, C* out, double coef, bool applyK) {
   PiEpi<T> e = epi(3, 1);
   e.grp[0] = 0;
-  e.coef[0] = (T)(1.0 / (double)Nvol);
+  e.coef[0] = (T)coef;
   e.applyK[0] = applyK ? 1 : 0;
   add_out(e, out, 0, 1.0, {});
   pb(PR_PI_FULL);
-  cuda(pi_fields<T>(full, src, e, Lhat, P1, st), "projection");
+  cuda(pi_fields<T>(full, kind, f, e, Lhat, P1, st), "projection");
   pe(PR_PI_FULL, grid_flops(N, 3));
   launches += kPiLaunches;
 }
 
 template <typename T>
+void Impl<T>::project_K(const T* f3, C* out, bool applyK) {
+  project(PI_FIELD, PiField<T>{{f3, f3 + Nvol, f3 + 2 * Nvol}, nullptr, nullptr, nullptr, T(0)}, out,
+          1.0 / (double)Nvol, applyK);
+}
+
+template <typename T>
+void Impl<T>::project_terminal(PiKind kind, const T* m, const T* y, const T* dm1, double c, C* out) {
+  project(kind, PiField<T>{{nullptr, nullptr, nullptr}, m, y, dm1, (T)c}, out, 1.0 / (double)Nvol, true);
+}
+
+template <typename T>
 void Impl<T>::project_adjoint(const T* f3, C* out) {
-  const T* src[3] = {f3, f3 + Nvol, f3 + 2 * Nvol};
-  PiEpi<T> e = epi(3, 1);
-  e.grp[0] = 0;
-  e.coef[0] = (T)1;
-  e.applyK[0] = 1;
-  add_out(e, out, 0, 1.0, {});
-  pb(PR_PI_FULL);
-  cuda(pi_fields<T>(full, src, e, Lhat, P1, st), "projection");
-  pe(PR_PI_FULL, grid_flops(N, 3));
-  launches += kPiLaunches;
+  project(PI_FIELD, PiField<T>{{f3, f3 + Nvol, f3 + 2 * Nvol}, nullptr, nullptr, nullptr, T(0)}, out, 1.0, true);
 }
 
 template <typename T>
@@ -360,7 +361,9 @@ template void Impl<float>::flush();
 template void Impl<double>::flush();
 template void Impl<float>::run_sweep(PwMode mode, const EvalDesc<float>* ev, int nev);
 template void Impl<float>::to_grid(const C* hist, int count, float* grid);
+template void Impl<float>::project(PiKind kind, const PiField<float>& f, C* out, double coef, bool applyK);
 template void Impl<float>::project_K(const float* f3, C* out, bool applyK);
+template void Impl<float>::project_terminal(PiKind kind, const float* m, const float* y, const float* dm1, double c, C* out);
 template void Impl<float>::project_adjoint(const float* f3, C* out);
 template void Impl<float>::shoot(State<float>& S);
 template void Impl<float>::state_step(State<float>& S, int n);
@@ -376,7 +379,9 @@ template void Impl<float>::exact_backward();
 template void Impl<double>::eval(PwMode mode, double* slot, const C* srcA, const C* srcB, const PiEpi<double>& e, double* slot2);
 template void Impl<double>::run_sweep(PwMode mode, const EvalDesc<double>* ev, int nev);
 template void Impl<double>::to_grid(const C* hist, int count, double* grid);
+template void Impl<double>::project(PiKind kind, const PiField<double>& f, C* out, double coef, bool applyK);
 template void Impl<double>::project_K(const double* f3, C* out, bool applyK);
+template void Impl<double>::project_terminal(PiKind kind, const double* m, const double* y, const double* dm1, double c, C* out);
 template void Impl<double>::project_adjoint(const double* f3, C* out);
 template void Impl<double>::shoot(State<double>& S);
 template void Impl<double>::state_step(State<double>& S, int n);

@@ -313,7 +313,11 @@ struct Impl {
   void to_grid(const C* hist, int count, T* grid);
 
   // K~ pi (or pi alone) of a 3-component image-grid field -> band vector out
+  void project(PiKind kind, const PiField<T>& f, C* out, double coef, bool applyK);
   void project_K(const T* f3, C* out, bool applyK = true);
+
+  // K~ pi of a terminal field (PI_RESIDUAL, PI_INCREMENT or PI_NEWTON)
+  void project_terminal(PiKind kind, const T* m, const T* y, const T* dm1, double c, C* out);
 
   // K~ sum_x f(x) e^{-2 pi i k.x} of a 3-component grid field: the V-representer
   // of the cotangent of iota (the adjoint of iota is N pi)

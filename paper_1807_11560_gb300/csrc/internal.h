@@ -221,9 +221,21 @@ struct IotaList {
 };
 template <typename T>
 cudaError_t iota_fields(const Plan<T>& p, const IotaList<T>& d, T* T1, cudaStream_t st);
-// pi of nf <= 3 grid fields (components 0..nf-1) with epilogue e (nper = 1)
+// pi of e.ncomp <= 3 grid fields with epilogue e (nper = 1); the fields, by kind:
+//   PI_FIELD      f[0..2]
+//   PI_RESIDUAL   c (m - y) d_j m                   (lambda(1) grad m(1))
+//   PI_INCREMENT  c y d_j m                         (its Gauss-Newton increment, y = dm(1))
+//   PI_NEWTON     c (dm d_j m + (m - y) d_j dm)     (the full-Newton increment)
+// d_j: periodic central difference along axis j, taken while the rows are read
+enum PiKind { PI_FIELD = 0, PI_RESIDUAL, PI_INCREMENT, PI_NEWTON };
 template <typename T>
-cudaError_t pi_fields(const Plan<T>& p, const T* const* src, const PiEpi<T>& e, const T* Lhat, T* P1,
+struct PiField {
+  const T* f[3];
+  const T *m, *y, *dm;
+  T c;
+};
+template <typename T>
+cudaError_t pi_fields(const Plan<T>& p, PiKind kind, const PiField<T>& s, const PiEpi<T>& e, const T* Lhat, T* P1,
                       cudaStream_t st);
 // elements of the scratch: T1 of nf fields, P1 of three
 template <typename T>
@@ -256,10 +268,6 @@ void transport_step(const T* m, const T* vnext, const T* vcur, T* mnext, T* off,
 // the characteristic (see grid.cu).
 template <typename T>
 void inc_step(const T* q, const T* m, const T* dv, const T* off, T* out, Dims g, double c, cudaStream_t st);
-// out_j = coef * r * d_j m, r = (m - y) if diff else y.
-template <typename T>
-void terminal_field(const T* m, const T* y, int diff, double coef, T* out, Dims g,
-                    cudaStream_t st);
 // ---- deformation-state form (Section 3.3) ----
 // central-difference gradient of an image -> [3][vol]
 template <typename T>
@@ -279,10 +287,6 @@ void def_force(const T* gs, const T* m1, const T* I1, const T* du, T* dm_out, do
 template <typename T>
 void adjoint_step(const T* lam, const T* m, const T* vcur, const T* vnext, const T* off, T* lam_out, T* gnext,
                   T* gcur, Dims g, double dt, cudaStream_t st);
-// out_j = c (dm d_j m + (m - y) d_j dm): the terminal field of the full-Newton
-// incremental adjoint (central differences)
-template <typename T>
-void terminal_newton(const T* m, const T* y, const T* dm, double c, T* out, Dims g, cudaStream_t st);
 // out = c (a - b)
 template <typename T>
 void scaled_diff(const T* a, const T* b, double c, T* out, long long n, cudaStream_t st);
