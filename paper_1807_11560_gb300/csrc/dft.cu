@@ -63,8 +63,9 @@ struct BandArgs {
   int tqs, nparts, prev;
 };
 
-template <typename T, int MODE, bool FLAT>
-__global__ void __launch_bounds__(kPhaseThreads, 1)
+// (MINB = 2: at most 128 registers, two CTAs per SM)
+template <typename T, int MODE, bool FLAT, int MINB>
+__global__ void __launch_bounds__(kPhaseThreads, MINB)
 k_band(const __grid_constant__ BandArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   pdl_trigger();
@@ -72,13 +73,13 @@ k_band(const __grid_constant__ BandArgs<T> a) {
                                          blockIdx.x, reinterpret_cast<V2<T>*>(smraw));
 }
 
-template <typename T, int MODE, int PT, int TT>
-__global__ void __launch_bounds__(kPhaseThreads, 1)
+template <typename T, int MODE, int PT>
+__global__ void __launch_bounds__(plane_threads<T>(PT), 1)
 k_plane(const __grid_constant__ Plan<T> p, int ppc, int nparts, const T* T1, T* slot, T* slot2, T* P1) {
   extern __shared__ __align__(16) unsigned char smraw[];
   pdl_trigger();
-  plane_item<T, MODE, kPhaseThreads, PT, TT>(p, ppc, nparts, T1, slot, slot2, P1, blockIdx.x,
-                                             reinterpret_cast<V2<T>*>(smraw));
+  plane_item<T, MODE, plane_threads<T>(PT), PT>(p, ppc, nparts, T1, slot, slot2, P1, blockIdx.x,
+                                              reinterpret_cast<V2<T>*>(smraw));
 }
 
 template <typename T, int MODE>
@@ -406,12 +407,6 @@ __global__ void k_band_store(const T* __restrict__ in, cplx<T>* __restrict__ out
 
 // row pairs per thread of k2 -> x2: all of an item's where that fits the registers
 int plane_pt(int ppc) { return ppc <= 3 ? 3 : (ppc <= 5 ? 5 : 9); }
-// x3 points per thread of k3 -> x3: two while that leaves a thread for most lanes
-template <typename T>
-int plane_tt(const Plan<T>& p, int ppc) {
-  return sizeof(T) == 4 && 2 * ppc * ((p.NT3 + 1) / 2) >= 160 ? 2 : 1;
-}
-
 template <typename T>
 size_t plane_smem(const Plan<T>& p, int mode, int ppc) {
   return plane_shape(p, mode_in(mode), mode_out(mode), ppc, plane_pt(ppc)).smem;
@@ -448,12 +443,12 @@ int pi_pairs(const Plan<T>& p) {
   return even_pairs(p.NT2, most, 1);
 }
 
-template <typename T, int MODE, int PT, int TT>
+template <typename T, int MODE, int PT>
 cudaError_t launch_plane_pt(const Plan<T>& p, const T* T1, T* slot, T* slot2, T* P1, cudaStream_t st) {
   const EvalGeom g = p.geom[MODE];
-  cudaError_t e = allow_smem<k_plane<T, MODE, PT, TT>>();
+  cudaError_t e = allow_smem<k_plane<T, MODE, PT>>();
   if (e != cudaSuccess) return e;
-  return launch_chain(k_plane<T, MODE, PT, TT>, dim3((unsigned)(p.g.n1 * g.nparts)), kPhaseThreads,
+  return launch_chain(k_plane<T, MODE, PT>, dim3((unsigned)(p.g.n1 * g.nparts)), plane_threads<T>(PT),
                       plane_smem(p, MODE, g.ppc), st, p, g.ppc, g.nparts, T1, slot, slot2, P1);
 }
 template <typename T, int MODE>
@@ -465,18 +460,12 @@ cudaError_t launch_plane(const Plan<T>& p, const T* T1, T* slot, T* slot2, T* P1
     return launch_chain(k_plane_flat<T, MODE>, dim3((unsigned)p.g.n1), kPhaseThreads, plane_flat_smem(p, MODE), st, p,
                         T1, slot, slot2, P1);
   }
-  if constexpr (sizeof(T) == 4) {
-    if (plane_tt(p, p.geom[MODE].ppc) == 2) {
-      if (pt == 5) return launch_plane_pt<T, MODE, 5, 2>(p, T1, slot, slot2, P1, st);
-      if (pt == 9) return launch_plane_pt<T, MODE, 9, 2>(p, T1, slot, slot2, P1, st);
-    }
-  }
-  if (pt == 3) return launch_plane_pt<T, MODE, 3, 1>(p, T1, slot, slot2, P1, st);
-  if (pt == 5) return launch_plane_pt<T, MODE, 5, 1>(p, T1, slot, slot2, P1, st);
-  return launch_plane_pt<T, MODE, 9, 1>(p, T1, slot, slot2, P1, st);
+  if (pt == 3) return launch_plane_pt<T, MODE, 3>(p, T1, slot, slot2, P1, st);
+  if (pt == 5) return launch_plane_pt<T, MODE, 5>(p, T1, slot, slot2, P1, st);
+  return launch_plane_pt<T, MODE, 9>(p, T1, slot, slot2, P1, st);
 }
 
-template <typename T, int MODE, bool FLAT>
+template <typename T, int MODE, bool FLAT, int MINB>
 cudaError_t launch_band_as(const Plan<T>& p, const PiEpi<T>* prev, const T* P1, const T* A, const T* B, T* T1,
                            const T* Lhat, cudaStream_t st) {
   BandArgs<T> a{};
@@ -494,16 +483,21 @@ cudaError_t launch_band_as(const Plan<T>& p, const PiEpi<T>* prev, const T* P1, 
   } else if (A == nullptr) {
     return cudaSuccess;
   }
-  cudaError_t e = allow_smem<k_band<T, MODE, FLAT>>();
+  cudaError_t e = allow_smem<k_band<T, MODE, FLAT, MINB>>();
   if (e != cudaSuccess) return e;
-  return launch_chain(k_band<T, MODE, FLAT>, dim3((unsigned)((p.k.Kq() + (1 << a.tqs) - 1) >> a.tqs)), kPhaseThreads,
+  return launch_chain(k_band<T, MODE, FLAT, MINB>, dim3((unsigned)((p.k.Kq() + (1 << a.tqs) - 1) >> a.tqs)), kPhaseThreads,
                       band_shape(p, 1 << a.tqs, fields_out(MODE, FLAT), fields_in(MODE, FLAT)).smem, st, a);
 }
 template <typename T, int MODE>
 cudaError_t launch_band(const Plan<T>& p, const PiEpi<T>* prev, const T* P1, const T* A, const T* B, T* T1,
                         const T* Lhat, cudaStream_t st) {
-  return p.flat ? launch_band_as<T, MODE, true>(p, prev, P1, A, B, T1, Lhat, st)
-                : launch_band_as<T, MODE, false>(p, prev, P1, A, B, T1, Lhat, st);
+  if (p.flat) return launch_band_as<T, MODE, true, 1>(p, prev, P1, A, B, T1, Lhat, st);
+  // more items than SMs: two to an SM (band 64^3: 166 us per evaluation against 182
+  // with one, band 40^3: 36.4 / 39.6); below that the registers are worth more (32^3:
+  // 21.6 / 19.5)
+  if (sizeof(T) == 4 && (p.k.Kq() >> p.geom[MODE].tqs) > kSMs)
+    return launch_band_as<T, MODE, false, sizeof(T) == 4 ? 2 : 1>(p, prev, P1, A, B, T1, Lhat, st);
+  return launch_band_as<T, MODE, false, 1>(p, prev, P1, A, B, T1, Lhat, st);
 }
 
 template <typename T, int TL, int RB>

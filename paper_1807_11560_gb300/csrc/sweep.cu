@@ -100,7 +100,7 @@ k_sweep(const __grid_constant__ SweepArgs<T> a) {
     if (!grid_barrier(a.bar, target, a.flag, a.spin_limit, ev == 0 ? a.stall : 0u)) return;
     for (int i = blockIdx.x; i < n_plane; i += gridDim.x) {
       if constexpr (PT == 0) plane_item_flat<T, MODE, NT>(p, a.T1, cur->slot, cur->slot2, a.P1, i, sm);
-      else plane_item<T, MODE, NT, PT, 1>(p, a.g.ppc, a.g.nparts, a.T1, cur->slot, cur->slot2, a.P1, i, sm);
+      else plane_item<T, MODE, NT, PT>(p, a.g.ppc, a.g.nparts, a.T1, cur->slot, cur->slot2, a.P1, i, sm);
       __syncthreads();
     }
     if (!grid_barrier(a.bar, target, a.flag, a.spin_limit)) return;

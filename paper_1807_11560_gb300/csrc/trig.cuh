@@ -26,6 +26,7 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.h"
 
@@ -34,10 +35,14 @@ namespace dev {
 
 constexpr double kTwoPi = 6.283185307179586476925286766559;
 constexpr int kMaxSmem = 224 * 1024;
-// Threads of both phases.  The contractions are bound by issue slots, so a thread
-// takes a large register tile (few shared-memory reads per packed FMA) rather than
-// one of many small ones.
+// Threads of the two phases.  The contractions are bound by issue slots and by the
+// register write-back of shared-memory reads (one pair per lane costs two packed
+// FMAs), so a thread takes a register tile of several sums.
 constexpr int kPhaseThreads = 256;
+// Plane phase: on large items enough warps to overlap one's reads with another's
+// sums (us per evaluation at 256 / 512 threads: band 32^3 19.5 / 18.7, 64^3 166 /
+// 161); small ones have work for 256 only (16^3 9.8 / 10.3).
+template <typename T> __host__ __device__ constexpr int plane_threads(int PT) { return sizeof(T) == 4 && PT > 5 ? 512 : 256; }
 
 // Programmatic dependent launch: a kernel launched with programmatic stream
 // serialisation may start while its predecessor runs; it stages its constant
@@ -272,48 +277,55 @@ __device__ __forceinline__ void fold_planes(const Plan<T>& p, const T* P1, int N
                                             int t0, int nt, FastDiv dnt, V2<T>* sE) {
   const int G1 = p.g.n1, PC = 4 << tqs;
   const long long Kq = p.k.Kq(), pstride = NO * Kq * 4;   // pstride: one partial plane
-  // two items per thread and round: their loads are in flight together
-  const int n = (NO * nt) << tqs;
-  for (int i0 = threadIdx.x; i0 < n; i0 += 2 * NT) {
-    const T *a[2], *b[2];
+  // A lane sums one side (x or G1 - x) of one (field, point, quad); neighbouring lanes
+  // hold the two sides, exchange half of their sums and fold one pair of columns
+  // each.  Two sums per thread and round, four partial planes of each in flight.
+  const int n = (NO * nt) << (tqs + 1), side = threadIdx.x & 1;
+  for (int i0 = 0; i0 < n; i0 += 2 * NT) {
+    const T* a[2];
     V2<T>* d[2];
     bool two[2], live[2];
+    V2<T> c[2], q[2];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      const int it = min(i0 + j * NT, n - 1);
-      const int ql = it & ((1 << tqs) - 1), r = it >> tqs;
+      const int it = i0 + j * NT + (int)threadIdx.x, ix = min(it, n - 1) >> 1;
+      const int ql = ix & ((1 << tqs) - 1), r = ix >> tqs;
       const int o = fdiv(r, dnt), t = r - o * nt, x = t0 + t;
-      live[j] = i0 + j * NT < n && ql < nq;
+      live[j] = it < n && ql < nq;
       two[j] = x > 0 && 2 * x != G1;
-      const T* base = P1 + ((long long)o * Kq + q0 + min(ql, nq - 1)) * 4;
-      a[j] = base + (long long)x * nparts * pstride;
-      b[j] = base + (long long)(two[j] ? G1 - x : x) * nparts * pstride;
-      d[j] = sE + (o * nt + t) * PC + 4 * ql;
+      a[j] = P1 + (long long)(side && two[j] ? G1 - x : x) * nparts * pstride +
+             ((long long)o * Kq + q0 + min(ql, nq - 1)) * 4;
+      d[j] = sE + (o * nt + t) * PC + 4 * ql + 2 * side;
+      c[j] = q[j] = zero2<T>();
     }
-    V2<T> u[2][2], v[2][2];                                // [item][s3] sums at x and G1 - x
+    for (int k0 = 0; k0 < nparts; k0 += 4) {
+      Quad<T> u[2][4];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) u[j][0] = u[j][1] = v[j][0] = v[j][1] = zero2<T>();
-#pragma unroll 2
-    for (int k = 0; k < nparts; ++k) {
+      for (int k = 0; k < 4; ++k)
+        if (k0 + k < nparts) {
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const Quad<T> qa = ldq(a[j] + k * pstride), qb = ldq(b[j] + k * pstride);
-        u[j][0] = sum2(u[j][0], qa.c);
-        u[j][1] = sum2(u[j][1], qa.s);
-        v[j][0] = sum2(v[j][0], qb.c);
-        v[j][1] = sum2(v[j][1], qb.s);
-      }
+          for (int j = 0; j < 2; ++j) u[j][k] = ldq(a[j] + (k0 + k) * pstride);
+        }
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (k0 + k < nparts) {
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            c[j] = sum2(c[j], u[j][k].c);
+            q[j] = sum2(q[j], u[j][k].s);
+          }
+        }
     }
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      if (!live[j]) continue;
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        T u0, u1, v0, v1;
-        un2(u[j][i], u0, u1);
-        un2(v[j][i], v0, v1);
-        d[j][2 * i] = two[j] ? mk2(u0 + v0, u0 - v0) : mk2(u0, T(0));
-        d[j][2 * i + 1] = two[j] ? mk2(u1 + v1, u1 - v1) : mk2(u1, T(0));
+      const V2<T> got = shfl2<T>(side ? c[j] : q[j], 1);   // the other side of this lane's columns
+      const V2<T> near = side ? got : c[j], far = side ? q[j] : got;
+      T u0, u1, v0, v1;
+      un2(near, u0, u1);                                   // side 0: x in near; side 1: x in got
+      un2(far, v0, v1);
+      if (live[j]) {
+        d[j][0] = two[j] ? mk2(u0 + v0, u0 - v0) : mk2(u0, T(0));
+        d[j][1] = two[j] ? mk2(u1 + v1, u1 - v1) : mk2(u1, T(0));
       }
     }
   }
@@ -597,7 +609,7 @@ __host__ __device__ inline PlaneShape<T> plane_shape(const Plan<T>& p, int NF, i
 template <typename T, int NT, int NF, int PT>
 __device__ __forceinline__ void rows_from_band(const Plan<T>& p, const T* V, int nf, int np, const PlaneShape<T>& sh,
                                                const V2<T>* tw2f, V2<T>* S1) {
-  constexpr int PTe = PT + (PT & 1), U = sizeof(T) == 4 ? 8 : 4;
+  constexpr int PTe = PT + (PT & 1), U = sizeof(T) == 4 ? (NF > 3 ? 16 : 8) : 4;
   const int K2h = p.k.K2h, K3h = p.k.K3h, K3e = p.K3e;
   const long long Kq = p.k.Kq();
   const int ng = (np + PT - 1) / PT;
@@ -625,15 +637,20 @@ __device__ __forceinline__ void rows_from_band(const Plan<T>& p, const T* V, int
     };
     const int da = K3h * 4;
     int a = 0;
-    for (; a + U <= K2h; a += U) {                         // U loads in flight
-      Quad<T> q[U];
+    auto rows = [&](auto n_) {                             // n loads in flight
+      constexpr int N = decltype(n_)::value;
+      for (; a + N <= K2h; a += N) {
+        Quad<T> q[N];
 #pragma unroll
-      for (int u = 0; u < U; ++u) q[u] = ldq(v + u * da);
-      v += U * da;
+        for (int u = 0; u < N; ++u) q[u] = ldq(v + u * da);
+        v += N * da;
 #pragma unroll
-      for (int u = 0; u < U; ++u) row(q[u], w + u * sh.ppe);
-      w += U * sh.ppe;
-    }
+        for (int u = 0; u < N; ++u) row(q[u], w + u * sh.ppe);
+        w += N * sh.ppe;
+      }
+    };
+    rows(std::integral_constant<int, U>{});
+    rows(std::integral_constant<int, 4>{});
     for (; a < K2h; ++a, v += da, w += sh.ppe) row(ldq(v), w);
 #pragma unroll
     for (int i = 0; i < PT; ++i) {
@@ -860,6 +877,11 @@ __device__ __forceinline__ void products(const T* x, const T* c, T* o) {
   }
 }
 
+// product fields per thread of x3 -> k3: fewer on small items, for a thread per sum
+__host__ __device__ constexpr int k3_fields(int NO, int PT) {
+  return PT <= 3 || NO <= 4 ? 1 : (PT <= 5 ? 2 : 3);
+}
+
 // constant tables of one plane item (rows t0 .. t0 + np of axis 2)
 template <typename T, int NT, int PT>
 __device__ __forceinline__ void plane_tables(const Plan<T>& p, const PlaneShape<T>& s, int t0, int np, bool fwd,
@@ -880,9 +902,8 @@ __device__ __forceinline__ void plane_tables(const Plan<T>& p, const PlaneShape<
   }
 }
 
-// one plane-phase item: plane x1, row pairs [part ppc, ...).  TT: folded x3 points
-// per thread of the k3 -> x3 stage.
-template <typename T, int MODE, int NT, int PT, int TT>
+// one plane-phase item: plane x1, row pairs [part ppc, ...)
+template <typename T, int MODE, int NT, int PT>
 __device__ __forceinline__ void plane_item(const Plan<T>& p, int ppc, int nparts, const T* T1, T* slot, T* slot2, T* P1,
                                            int item, V2<T>* sm) {
   constexpr int NF = mode_in(MODE), NO = mode_out(MODE), NC = mode_cached(MODE);
@@ -898,78 +919,73 @@ __device__ __forceinline__ void plane_item(const Plan<T>& p, int ppc, int nparts
   __syncthreads();
   rows_from_band<T, NT, NF, PT>(p, T1 + (long long)x1 * NF * Kq * 4, NF, np, s, sm + s.off_2f, S1);
   __syncthreads();
-  // k3 -> x3 and the products: one row and TT x3 pairs per thread, every field's
-  // sums in registers; the cached fields are loaded before the sums
-  const int nth = TT == 1 ? NT3 : (NT3 + 1) / 2;
-  for (int it = threadIdx.x; it < 2 * np * nth; it += NT) {
-    const int row = fdiv(it, TT == 1 ? p.dNT3 : p.dNT3h), tl = it - row * nth;
-    const int u = t0 + (row >> 1);
-    if ((row & 1) && (u == 0 || 2 * u == G2)) continue;
-    const long long at = ((long long)x1 * G2 + ((row & 1) ? G2 - u : u)) * G3;
-    int t[TT];
-    bool two[TT];
-    T ca[TT][NC > 0 ? NC : 1], cb[TT][NC > 0 ? NC : 1];
-#pragma unroll
-    for (int j = 0; j < TT; ++j) {
-      t[j] = min(tl + j * nth, NT3 - 1);
-      two[j] = t[j] > 0 && 2 * t[j] != G3;
-      if (NC > 0) {
-        load_cached<T, MODE>(slot, vol, at + t[j], ca[j]);
-        load_cached<T, MODE>(slot, vol, at + (two[j] ? G3 - t[j] : t[j]), cb[j]);
-      }
+  // k3 -> x3 and the products.  Two lanes 16 apart share a row and the x3 pairs tl and
+  // tl + nth: each sums half of the fields at both (a row's coefficients are then read
+  // once for two points), they exchange, and each finishes one pair.  The cached
+  // fields are loaded before the sums.
+  constexpr int FH = NF / 2;
+  static_assert(NF % 2 == 0, "fields in two halves");
+  const int nth = (NT3 + 1) / 2, half = (threadIdx.x >> 4) & 1;
+  const int n = 2 * np * nth;                              // (row, tl) items, 16 per warp and round
+  for (int i0 = 0; i0 < n; i0 += NT / 2) {
+    const int it = i0 + (threadIdx.x >> 5) * 16 + (threadIdx.x & 15);
+    const int ic = min(it, n - 1), row = fdiv(ic, p.dNT3h), tl = ic - row * nth;
+    const int u = t0 + (row >> 1), tm = min(tl + half * nth, NT3 - 1);   // tm: the pair this lane finishes
+    const bool two = tm > 0 && 2 * tm != G3;
+    const bool mine = it < n && tl + half * nth < NT3 && !((row & 1) && (u == 0 || 2 * u == G2));
+    const long long at = ((long long)x1 * G2 + ((row & 1) && u > 0 ? G2 - u : u)) * G3;
+    T ca[NC > 0 ? NC : 1], cb[NC > 0 ? NC : 1];
+    if (NC > 0) {
+      load_cached<T, MODE>(slot, vol, at + tm, ca);
+      load_cached<T, MODE>(slot, vol, at + (two ? G3 - tm : tm), cb);
     }
-    V2<T> acc[TT][NF];
+    V2<T> acc[2][FH];
 #pragma unroll
-    for (int j = 0; j < TT; ++j)
-#pragma unroll
-      for (int f = 0; f < NF; ++f) acc[j][f] = zero2<T>();
-    const V2<T>* v = S1 + row * K3s;
-    const V2<T>* w = sm;
+    for (int f = 0; f < FH; ++f) acc[0][f] = acc[1][f] = zero2<T>();
+    const V2<T>* v = S1 + (half * FH * R + row) * K3s;
+    const V2<T>* w = sm + tl;
+    const int t2 = min(tl + nth, NT3 - 1) - tl;            // to the second pair
     for (int b = 0; b < K3e; b += 2) {
-      V2<T> w0[TT], w1[TT];
-#pragma unroll
-      for (int j = 0; j < TT; ++j) {
-        w0[j] = w[t[j]];
-        w1[j] = w[NT3 + t[j]];
-      }
+      const V2<T> w00 = w[0], w01 = w[t2], w10 = w[NT3], w11 = w[NT3 + t2];
       w += 2 * NT3;
 #pragma unroll
-      for (int f = 0; f < NF; ++f) {
+      for (int f = 0; f < FH; ++f) {
         V2<T> a0, a1;
         ld2(v + f * R * K3s + b, a0, a1);
-#pragma unroll
-        for (int j = 0; j < TT; ++j) acc[j][f] = fma2(a1, w1[j], fma2(a0, w0[j], acc[j][f]));
+        acc[0][f] = fma2(a1, w10, fma2(a0, w00, acc[0][f]));
+        acc[1][f] = fma2(a1, w11, fma2(a0, w01, acc[1][f]));
       }
     }
+    T xa[NF], xb[NF];
 #pragma unroll
-    for (int j = 0; j < TT; ++j) {
-      if (j > 0 && tl + j * nth >= NT3) continue;
-      T xa[NF], xb[NF];
+    for (int f = 0; f < FH; ++f) {
+      const V2<T> own = half ? acc[1][f] : acc[0][f], got = shfl2<T>(half ? acc[0][f] : acc[1][f], 16);
+      T E, O;
+      un2(half ? got : own, E, O);
+      xa[f] = E + O;
+      xb[f] = E - O;
+      un2(half ? own : got, E, O);
+      xa[FH + f] = E + O;
+      xb[FH + f] = E - O;
+    }
+    if (!mine) continue;
+    T* out = MODE == PW_F || MODE == PW_D0 ? slot : (MODE == PW_TC ? slot2 : nullptr);
+    if ((MODE == PW_F || MODE == PW_D0 || MODE == PW_TC) && out != nullptr) {
+      store_cached<T, MODE>(out, vol, at + tm, xa);
+      if (two) store_cached<T, MODE>(out, vol, at + G3 - tm, xb);
+    }
+    T oa[NO], ob[NO];
+    products<T, MODE>(xa, ca, oa);
+    products<T, MODE>(xb, cb, ob);
+    V2<T>* d = sP + row * NT3e + tm;
 #pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        T E, O;
-        un2(acc[j][f], E, O);
-        xa[f] = E + O;
-        xb[f] = E - O;
-      }
-      T* out = MODE == PW_F || MODE == PW_D0 ? slot : (MODE == PW_TC ? slot2 : nullptr);
-      if ((MODE == PW_F || MODE == PW_D0 || MODE == PW_TC) && out != nullptr) {
-        store_cached<T, MODE>(out, vol, at + t[j], xa);
-        if (two[j]) store_cached<T, MODE>(out, vol, at + G3 - t[j], xb);
-      }
-      T oa[NO], ob[NO];
-      products<T, MODE>(xa, ca[j], oa);
-      products<T, MODE>(xb, cb[j], ob);
-      V2<T>* d = sP + row * NT3e + t[j];
-#pragma unroll
-      for (int o = 0; o < NO; ++o) {
-        d[o * R * NT3e] = two[j] ? mk2(oa[o] + ob[o], oa[o] - ob[o]) : mk2(oa[o], T(0));
-        if (t[j] == NT3 - 1 && NT3e > NT3) d[o * R * NT3e + 1] = zero2<T>();
-      }
+    for (int o = 0; o < NO; ++o) {
+      d[o * R * NT3e] = two ? mk2(oa[o] + ob[o], oa[o] - ob[o]) : mk2(oa[o], T(0));
+      if (tm == NT3 - 1 && NT3e > NT3) d[o * R * NT3e + 1] = zero2<T>();
     }
   }
   __syncthreads();
-  rows_to_k3<T, NT, NO, (NO > 6 ? 6 : NO)>(p, sP, t0, ppc, np, sm + s.off_3b, S1);
+  rows_to_k3<T, NT, NO, k3_fields(NO, PT)>(p, sP, t0, ppc, np, sm + s.off_3b, S1);
   __syncthreads();
   T* out = P1 + ((long long)x1 * nparts + part) * NO * Kq * 4;
   if (p.k.K2h >= 16) band_from_rows<T, NT, NO, 8>(p, S1, ppc, np, sm + s.off_2b, out);
