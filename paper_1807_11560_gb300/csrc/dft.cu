@@ -159,12 +159,14 @@ k_iota_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList
     for (int j = 0; j < TL; ++j) tt[j] = min(tb * 32 * TL + 32 * j + lane, NT3 - 1);
 #pragma unroll
     for (int i = 0; i < RB; ++i) rr[i] = (f * R + min(row0 + i, 2 * np - 1)) * K3s;   // past the item: its last row
-    for (int b = 0; b < K3e; b += 2) {
+    const V2<T>* w = sm;
+#pragma unroll 2
+    for (int b = 0; b < K3e; b += 2, w += 2 * NT3) {
       V2<T> w0[TL], w1[TL];
 #pragma unroll
       for (int j = 0; j < TL; ++j) {
-        w0[j] = sm[b * NT3 + tt[j]];
-        w1[j] = sm[(b + 1) * NT3 + tt[j]];
+        w0[j] = w[tt[j]];
+        w1[j] = w[NT3 + tt[j]];
       }
 #pragma unroll
       for (int i = 0; i < RB; ++i) {
@@ -174,20 +176,35 @@ k_iota_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList
         for (int j = 0; j < TL; ++j) acc[i][j] = fma2(a1, w1[j], fma2(a0, w0[j], acc[i][j]));
       }
     }
-    T* __restrict__ dst = d.dst[f0 + f] + (long long)x1 * G2 * G3;
+    // rows come in pairs x2 = u, G2 - u (row0 is even): two row pointers that walk
+    // towards each other, the points of a lane at fixed distances from them
+    static_assert(RB % 2 == 0, "row pairs");
+    bool ok[TL], two[TL];
+#pragma unroll
+    for (int j = 0; j < TL; ++j) {
+      const int t = tb * 32 * TL + 32 * j + lane;
+      ok[j] = t < NT3;
+      two[j] = ok[j] && t > 0 && 2 * t != G3;
+    }
+    const int u0 = t0 + (row0 >> 1), first = tb * 32 * TL + lane;
+    T* ra = d.dst[f0 + f] + ((long long)x1 * G2 + u0) * G3;
+    T* rb = d.dst[f0 + f] + ((long long)x1 * G2 + G2 - u0) * G3;
 #pragma unroll
     for (int i = 0; i < RB; ++i) {
-      const int row = row0 + i, u = t0 + (row >> 1);
-      if (row >= 2 * np || ((row & 1) && (u == 0 || 2 * u == G2))) continue;
-      T* o = dst + (long long)((row & 1) ? G2 - u : u) * G3;
+      const int u = u0 + i / 2;
+      const bool live = row0 + i < 2 * np && !((i & 1) && (u == 0 || 2 * u == G2));
+      T* up = ((i & 1) ? rb : ra) + first;
+      T* dn = ((i & 1) ? rb : ra) + (G3 - first);
 #pragma unroll
       for (int j = 0; j < TL; ++j) {
-        const int t = tb * 32 * TL + 32 * j + lane;
-        if (t >= NT3) continue;
         T E, O;
         un2(acc[i][j], E, O);
-        o[t] = E + O;
-        if (t > 0 && 2 * t != G3) o[G3 - t] = E - O;
+        if (live && ok[j]) up[32 * j] = E + O;
+        if (live && two[j]) dn[-32 * j] = E - O;
+      }
+      if (i & 1) {
+        ra += G3;
+        rb -= G3;
       }
     }
   }
