@@ -9,21 +9,26 @@ template <typename T>
 void Impl<T>::iota_call(const void* a, int ncomp, void* out) {
   for (int c0 = 0; c0 < ncomp; c0 += 3) {
     const int nc = std::min(3, ncomp - c0);
-    cuda(cudaMemcpyAsync(zin, (const Z*)a + (long long)c0 * Kuser, (size_t)nc * Kuser * sizeof(Z),
-                         cudaMemcpyDefault, st), "copy");
-    band_load<T>(zin, px, nc, K, st);
+    const Z* src = (const Z*)a + (long long)c0 * Kuser;
+    const bool grid_direct = in_place((T*)out + (long long)c0 * Nvol, (size_t)nc * Nvol * sizeof(T), sizeof(T));
+    if (!in_place(src, (size_t)nc * Kuser * sizeof(Z), sizeof(Z))) {
+      cuda(cudaMemcpyAsync(zin, src, (size_t)nc * Kuser * sizeof(Z), cudaMemcpyDefault, st), "copy");
+      src = zin;
+    }
+    band_load<T>(src, px, nc, K, st);
     ++launches;
     IotaList<T> d{};
     d.nf = nc;
     for (int c = 0; c < nc; ++c) {
       d.src[c] = px + c * Kvol;
-      d.dst[c] = fterm + c * Nvol;
+      d.dst[c] = (grid_direct ? (T*)out + (long long)c0 * Nvol : fterm) + c * Nvol;
     }
     cuda(iota_fields<T>(full, d, T1, st), "iota");
     launches += kIotaLaunches;
     check_launch("iota");
-    cuda(cudaMemcpyAsync((T*)out + (long long)c0 * Nvol, fterm, (size_t)nc * Nvol * sizeof(T),
-                         cudaMemcpyDefault, st), "copy");
+    if (!grid_direct)
+      cuda(cudaMemcpyAsync((T*)out + (long long)c0 * Nvol, fterm, (size_t)nc * Nvol * sizeof(T),
+                           cudaMemcpyDefault, st), "copy");
   }
   sync("iota");
 }
@@ -32,20 +37,25 @@ template <typename T>
 void Impl<T>::pi_call(const void* f, int ncomp, void* out) {
   for (int c0 = 0; c0 < ncomp; c0 += 3) {
     const int nc = std::min(3, ncomp - c0);
-    cuda(cudaMemcpyAsync(fterm, (const T*)f + (long long)c0 * Nvol, (size_t)nc * Nvol * sizeof(T),
-                         cudaMemcpyDefault, st), "copy");
-    const PiField<T> src{{fterm, fterm + Nvol, fterm + 2 * Nvol}, nullptr, nullptr, nullptr, T(0)};
+    const T* g = (const T*)f + (long long)c0 * Nvol;
+    if (!in_place(g, (size_t)nc * Nvol * sizeof(T), sizeof(T))) {
+      cuda(cudaMemcpyAsync(fterm, g, (size_t)nc * Nvol * sizeof(T), cudaMemcpyDefault, st), "copy");
+      g = fterm;
+    }
+    const PiField<T> src{{g, g + (nc > 1 ? Nvol : 0), g + (nc > 2 ? 2 * Nvol : 0)}, nullptr, nullptr, nullptr, T(0)};
     PiEpi<T> e = epi(nc, 1);
     e.grp[0] = 0;
     e.coef[0] = (T)(1.0 / (double)Nvol);
     e.applyK[0] = 0;
     add_out(e, vout, 0, 1.0, {});
     cuda(pi_fields<T>(full, PI_FIELD, src, e, Lhat, P1, st), "pi");
-    band_store<T>(vout, zout, nc, K, st);
+    Z* dst = (Z*)out + (long long)c0 * Kuser;
+    const bool direct = in_place(dst, (size_t)nc * Kuser * sizeof(Z), sizeof(Z));
+    band_store<T>(vout, direct ? dst : zout, nc, K, st);
     launches += kPiLaunches + 1;
     check_launch("pi");
-    cuda(cudaMemcpyAsync((Z*)out + (long long)c0 * Kuser, zout, (size_t)nc * Kuser * sizeof(Z),
-                         cudaMemcpyDefault, st), "copy");
+    if (!direct)
+      cuda(cudaMemcpyAsync(dst, zout, (size_t)nc * Kuser * sizeof(Z), cudaMemcpyDefault, st), "copy");
   }
   sync("pi");
 }

@@ -93,6 +93,7 @@ void Impl<T>::create(int nd, const int* grid, const int* band, double a, int s_,
   Kuser = K.vol();
   opts = o;
   st = (cudaStream_t)o.stream;
+  cuda(cudaGetDevice(&device), "device");
   cuda(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking), "stream");
   cuda(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "event");
 
@@ -192,22 +193,65 @@ void Impl<T>::record_sweeps() {
   rec = nullptr;
 }
 
+namespace {
+// the allocation that holds a device address (driver call, looked up once)
+using AddressRange = int (*)(unsigned long long* base, size_t* size, unsigned long long p);
+AddressRange address_range() {
+  static const AddressRange f = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &p, 12000, cudaEnableDefault, &q) !=
+            cudaSuccess || q != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
+    return reinterpret_cast<AddressRange>(p);
+  }();
+  return f;
+}
+}  // namespace
+
+// Whether the kernels can read or write the bytes at p in place: memory of this
+// context's device, aligned as the element, all of it inside one allocation.
+// Anything else (host and managed arrays, another device, a range that is too
+// short) goes through the staging buffers and the copy's own checks.
+template <typename T>
+bool Impl<T>::in_place(const void* p, size_t bytes, size_t align) {
+  const unsigned long long a = reinterpret_cast<uintptr_t>(p);
+  if (a % align != 0 || !address_range()) return false;
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (at.type != cudaMemoryTypeDevice || at.device != device) return false;
+  unsigned long long base = 0;
+  size_t size = 0;
+  return address_range()(&base, &size, a) == 0 && a + bytes <= base + size;
+}
+
 template <typename T>
 void Impl<T>::load_bl(const void* user, C* dst) {
-  cuda(cudaMemcpyAsync(zin, user, (size_t)duser * Kuser * sizeof(Z), cudaMemcpyDefault, st), "copy BL input");
+  const Z* src = static_cast<const Z*>(user);
+  if (!in_place(user, (size_t)duser * Kuser * sizeof(Z), sizeof(Z))) {
+    cuda(cudaMemcpyAsync(zin, user, (size_t)duser * Kuser * sizeof(Z), cudaMemcpyDefault, st), "copy BL input");
+    src = zin;
+  }
   if (duser < 3)
     cuda(cudaMemsetAsync(dst + (size_t)duser * Kvol, 0, (size_t)(3 - duser) * Kvol * sizeof(T), st), "memset");
-  band_load<T>(zin, dst, duser, K, st);
+  band_load<T>(src, dst, duser, K, st);
   ++launches;
   check_launch("band load");
 }
 
 template <typename T>
 void Impl<T>::store_bl(const C* src, void* user) {
-  band_store<T>(src, zout, duser, K, st);
+  const bool direct = in_place(user, (size_t)duser * Kuser * sizeof(Z), sizeof(Z));
+  band_store<T>(src, direct ? static_cast<Z*>(user) : zout, duser, K, st);
   ++launches;
   check_launch("band store");
-  cuda(cudaMemcpyAsync(user, zout, (size_t)duser * Kuser * sizeof(Z), cudaMemcpyDefault, st), "copy BL output");
+  if (!direct)
+    cuda(cudaMemcpyAsync(user, zout, (size_t)duser * Kuser * sizeof(Z), cudaMemcpyDefault, st), "copy BL output");
 }
 
 template <typename T>
@@ -266,6 +310,8 @@ template void Impl<float>::make_plan(Plan<float>& p, Dims g);
 template void Impl<float>::make_state(State<float>& S);
 template void Impl<float>::create(int nd, const int* grid, const int* band, double a, int s_, double sg, int nt, const lddmm_opts& o);
 template void Impl<float>::record_sweeps();
+template bool Impl<float>::in_place(const void* p, size_t bytes, size_t align);
+template bool Impl<double>::in_place(const void* p, size_t bytes, size_t align);
 template void Impl<float>::load_bl(const void* user, C* dst);
 template void Impl<float>::store_bl(const C* src, void* user);
 template void Impl<float>::collect();

@@ -74,7 +74,7 @@ struct Impl {
   using C = T;               // element of a band vector (internal.h): 3 Kvol reals
   using Z = cplx<T>;         // element of the caller's Hermitian arrays
   std::string* err = nullptr;
-  int ndim = 3, duser = 3;
+  int ndim = 3, duser = 3, device = 0;
   Dims N{}, M{};
   Band K{};
   int Nt = 1, s = 2;
@@ -203,6 +203,7 @@ struct Impl {
 
   // ------------------------------------------------------------ staging
   // user BL vector (duser comps) -> hermitian 3-comp device vector
+  bool in_place(const void* p, size_t bytes, size_t align);
   void load_bl(const void* user, C* dst);
   void store_bl(const C* src, void* user);
   void sync(const char* what) {
