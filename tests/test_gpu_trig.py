@@ -4,6 +4,8 @@ and two to an SM, the image-grid kernels' edges of tiles, the 2D kernels, and de
 pointers used in place; against the FP64 oracle.  Tolerances are those of the
 per-transform and per-product tests of the other modules."""
 
+import gc
+
 import numpy as np
 import pytest
 
@@ -21,6 +23,15 @@ GRAD_TOL = {"fp64": 1e-9, "fp32": 1e-5}
 # pass takes, thin and long axes, band items two to an SM, K2/2 below and above 16
 BANDS = [(2, 2, 2), (4, 8, 6), (6, 34, 2), (16, 16, 16), (24, 24, 24), (64, 6, 10), (60, 14, 22), (26, 30, 34),
          (32, 32, 32), (40, 40, 40), (64, 30, 44)]
+
+
+@pytest.fixture(autouse=True, scope="module")
+def _no_garbage():
+    """Tracebacks of the tests before keep device tensors in reference cycles; drop
+    them here, so that they are not freed in the middle of a later memory check."""
+    gc.collect()
+    yield
+    gc.collect()
 
 
 def _empty(shape, precision, cplx):
