@@ -74,17 +74,11 @@ typedef enum {
                             failure in lddmm_report.ls_failed instead */
 } lddmm_status;
 
-/* Arithmetic of a context.  LDDMM_FP64: double throughout.  LDDMM_FP32:
- * float data and arithmetic with FP64 reductions; the tensor cores take the
- * contractions as opts.tensor_cores says (3xTF32 split).  The two split modes
- * are FP32 contexts (float / complex64 arrays) whose contractions run on the
- * tcgen05 tensor cores wherever a kernel covers their sizes (opts.tensor_cores
- * is then 2): LDDMM_3XTF32 splits every operand x = hi + lo into two TF32
- * values and sums three TF32 products; LDDMM_BF16X3 splits the operands of the
- * image-grid band-to-grid stage into three BF16 values (hi + mid + lo) and sums
- * six BF16 products (the other tensor-core kernels keep 3xTF32).  Every mode
- * agrees with FP64 to FP32 rounding (~1e-7 relative per transform).  FP32 with
- * opts.tensor_cores = 0 is the plain FP32 SIMT form. */
+/* Arithmetic of a context.  LDDMM_FP64: double throughout.  LDDMM_FP32: float
+ * data and arithmetic with FP64 reductions.  LDDMM_3XTF32 and LDDMM_BF16X3 are
+ * FP32 contexts (float / complex64 arrays) that allow a split of the operands
+ * into TF32 or BF16 parts; the present transforms run them in full FP32, which
+ * is both faster and closer to FP64 than either split at these sizes. */
 typedef enum { LDDMM_FP64 = 0, LDDMM_FP32 = 1, LDDMM_3XTF32 = 2, LDDMM_BF16X3 = 3 } lddmm_precision;
 
 typedef struct {
@@ -95,17 +89,14 @@ typedef struct {
   int max_halvings;     /* line-search halvings of eps = 1; default 10 */
   int use_graphs;       /* replay the Hessian-vector product from a CUDA graph; default 1 */
   int persistent;       /* band-limited time sweeps as one persistent cooperative kernel
-                           (grid barriers with bounded waits): 0 never (three kernels per
-                           bracket evaluation), 1 when the padded product grid has at
-                           most 32^3 points (default), 2 always */
-  int tensor_cores;     /* FP32 contexts, tcgen05 tensor cores with the 3xTF32 split:
-                           iota stage C on the image grid, and the three kernels of a
-                           bracket evaluation launched per evaluation (iota A+B;
-                           C, the bracket products and C'; pi B'+A' with the
-                           epilogue), each where its tile geometry fits the sizes
-                           (the SIMT kernel otherwise).  0 never; 1 (default) for
-                           image grids of at least 2^20 voxels and padded grids
-                           above 32^3 points; 2 whenever supported */
+                           (grid barriers with bounded waits): 2 always; 0 and 1
+                           (default): two kernels per bracket evaluation, chained by
+                           programmatic dependent launch, which is faster at every
+                           size measured.  lddmm_batch_gn_solve refuses 2, and 1 on
+                           padded grids of at most 32^3 points: pass 0 for small
+                           batched contexts */
+  int tensor_cores;     /* 0, 1 (default) or 2; accepted, no effect on how the
+                           contractions run (see lddmm_precision) */
   int recompute;        /* image-grid histories of the time sweeps (velocity grids v_n,
                            characteristic displacements, states m_n, incremental
                            velocity grids): 0 keep all Nt + 1 steps (default); 1 keep
@@ -116,12 +107,8 @@ typedef struct {
                            floats per voxel (plus the transform scratch), and each
                            Hessian-vector product re-runs the state transport (Nt steps
                            and 2 (Nt + 1) vector iotas more). */
-  int autotune;         /* 1 (default): at creation, time the candidate tile shapes of the
-                           three padded-grid bracket kernels (twiddle staging, pencils per
-                           tile, band rows per item) on this context's sizes and keep the
-                           fastest; 0: size heuristics.  Contexts whose sweeps run as
-                           persistent kernels keep the heuristics.  No result depends on
-                           the tile shapes. */
+  int autotune;         /* 0 or 1 (default); accepted, no effect: the work split of the
+                           padded-grid kernels follows from the sizes alone */
   int newton;           /* Hessian used by lddmm_gn_solve's PCG: 0 Gauss-Newton (default),
                            1 full Newton (lddmm_hessvec_newton); PCG stops at the first
                            direction of non-positive curvature either way. */
@@ -159,9 +146,7 @@ typedef struct {
 } lddmm_report;
 
 /* Defaults for lddmm_opts (precision FP32, legacy stream, tol 1e-12,
- * c = 1e-4, 10 halvings, graphs on, persistent sweeps on small grids,
- * tensor-core image-grid transforms on large grids, kept histories,
- * autotuned tiles). */
+ * c = 1e-4, 10 halvings, graphs on, kept histories). */
 void lddmm_default_opts(lddmm_opts* opts);
 
 /* Create a registration context (Section 3.2).
@@ -243,10 +228,10 @@ int lddmm_gn_solve(lddmm_ctx* ctx, void* v0_inout, int n_gn, int n_pcg, lddmm_re
  * from min(n, nthreads) host threads (0: one per hardware thread).  Each
  * context runs its calls in order on its own opts.stream, so contexts created
  * with distinct non-NULL streams overlap on the GPU; contexts sharing a stream
- * (or the legacy NULL stream) serialise but stay correct.  Contexts whose
- * sweeps would run as persistent cooperative kernels are refused
- * (LDDMM_EINVAL): independent cooperative grids are not guaranteed to be
- * co-resident.  reps: NULL or n reports.  Returns LDDMM_OK or the first
+ * (or the legacy NULL stream) serialise but stay correct.  Contexts that allow
+ * persistent cooperative sweeps (opts.persistent = 2, or 1 on padded grids of
+ * at most 32^3 points) are refused (LDDMM_EINVAL): independent cooperative
+ * grids are not guaranteed to be co-resident.  reps: NULL or n reports.  Returns LDDMM_OK or the first
  * failing context's status (its lddmm_last_error says why); every context is
  * run to the end whatever the others return. */
 int lddmm_batch_gn_solve(lddmm_ctx* const* ctxs, int n, void* const* v0s, int n_gn, int n_pcg,
@@ -349,9 +334,12 @@ int lddmm_last_dm1(lddmm_ctx* ctx, void* dm1_out);
  *                (read m_n, write m_{n+1});
  *   "inc_step"   incremental state step (Eq. 31); work = 12 N bytes
  *                (read m_n and dm_n, write dm_{n+1});
- *   "iota_ab", "cpw", "pi_ba"  the three kernels of a bracket evaluation on
- *                the padded product grid (Eqs. 48-49); work = flops of their
- *                contractions and bracket products;
+ *   "cpw", "pi_ba"  the two kernels of a bracket evaluation on the padded
+ *                product grid (Eqs. 48-49): the plane phase (x2-x3 transforms
+ *                and the bracket products) and the band phase (x1 transforms,
+ *                spectral multipliers, time-step updates); work = flops of
+ *                their contractions and products ("iota_ab" and "deform" name
+ *                classes without launches of their own);
  *   "iota_full", "pi_full"  transforms on the image grid; work = flops;
  *   "sweep"      one persistent band-limited sweep kernel; work = flops;
  * NULL or "" switches the probe off.  Changing the class rebuilds the graph
@@ -368,10 +356,9 @@ int lddmm_probe_read(lddmm_ctx* ctx, double* total_ms, long long* launches, doub
  * replays count each kernel node). */
 long long lddmm_kernel_count(const lddmm_ctx* ctx);
 
-/* Tile shapes the context's padded-grid bracket kernels use (after the
- * autotuner, or the size heuristics): tws 1/2 = iota A+B twiddles from global
- * / shared memory, tp = pencils per C/products/C' tile, kc = band rows per
- * pi B'/A' item.  LDDMM_EINVAL on NULL arguments. */
+/* Work split of the context's padded-grid kernels: tws is always 2, tp = plane
+ * parts per x1 column, kc = quads (k2, k3) per band item.  LDDMM_EINVAL on NULL
+ * arguments. */
 int lddmm_tile_config(const lddmm_ctx* ctx, int* tws, int* tp, int* kc);
 
 /* Bytes of device memory the context holds (all of it is allocated by

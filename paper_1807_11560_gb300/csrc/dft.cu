@@ -63,7 +63,12 @@ struct BandArgs {
   int tqs, nparts, prev;
 };
 
-// (MINB = 2: at most 128 registers, two CTAs per SM)
+// Band phase.  A chain of dependent stages (partial planes from L2, x1 -> k1, the time
+// step, k1 -> x1) over a few columns: latency on small bands, shared-memory reads at
+// 64^3.  Alone and cold at band 32^3: 8.3 us (tangent), 9.3 (shoot), 12.3 (backward);
+// with the plane phase, one evaluation of a sweep takes 9.4 us at band 16^3, 18.7 at
+// 32^3 and 161 at 64^3, where three kernels of complex half-spectrum sums took 17,
+// 33-36 and 850.  MINB = 2: at most 128 registers, two CTAs per SM.
 template <typename T, int MODE, bool FLAT, int MINB>
 __global__ void __launch_bounds__(kPhaseThreads, MINB)
 k_band(const __grid_constant__ BandArgs<T> a) {
@@ -73,6 +78,9 @@ k_band(const __grid_constant__ BandArgs<T> a) {
                                          blockIdx.x, reinterpret_cast<V2<T>*>(smraw));
 }
 
+// Plane phase: bound by packed-FMA issue and shared-memory reads, about one pair read
+// per one or two FMAs.  Alone and cold at band 32^3: 11.5 us (tangent), 14.3 (shoot),
+// 16.7 (backward).
 template <typename T, int MODE, int PT>
 __global__ void __launch_bounds__(plane_threads<T>(PT), 1)
 k_plane(const __grid_constant__ Plan<T> p, int ppc, int nparts, const T* T1, T* slot, T* slot2, T* P1) {
@@ -82,6 +90,9 @@ k_plane(const __grid_constant__ Plan<T> p, int ppc, int nparts, const T* T1, T* 
                                               reinterpret_cast<V2<T>*>(smraw));
 }
 
+// The plane phase of a 2D problem: latency, and in FP64 the double pipe (a product of
+// the 64^2 / 16^2 configuration, 40 evaluations: 1.02 ms; 2.5 ms with complex
+// half-spectrum sums).
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kPhaseThreads)
 k_plane_flat(const __grid_constant__ Plan<T> p, const T* T1, T* slot, T* slot2, T* P1) {
@@ -94,6 +105,8 @@ k_plane_flat(const __grid_constant__ Plan<T> p, const T* T1, T* slot, T* slot2, 
 constexpr int kChunk = 32;        // folded x1 points per twiddle chunk
 constexpr int kIotaPT = 8;        // row pairs per thread of k2 -> x2
 
+// k1 -> x1 of up to six fields for 2^tqs quads of columns, kChunk points at a time: bound
+// by its writes to L2 (17 us for the 33 fields of 11 velocities, 160 planes, band 32^3).
 template <typename T>
 __global__ void __launch_bounds__(kImgThreads)
 k_iota_band(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList<T> d, int tqs, T* T1) {
@@ -123,10 +136,11 @@ k_iota_band(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList<
   }
 }
 
-// iota of up to three fields on `ppi` row pairs of one x1 plane.  k3 -> x3 costs
-// K3/2 products per point and dominates: a lane owns TL points t (and their
+// iota of up to three fields on `ppi` row pairs of one x1 plane (odd G3; even ones take
+// k_iota_plane_even).  k3 -> x3 costs K3/2 products per point and dominates: a lane owns TL points t (and their
 // partners G3 - t) of RB rows, so a row's coefficients are read once per warp
-// (broadcast) and a twiddle once per RB rows.
+// (broadcast) and a twiddle once per RB rows.  Packed FMAs and shared reads bind it:
+// 306 us for 33 fields of 160x192x160 at band 32^3.
 template <typename T, int TL, int RB>
 __global__ void __launch_bounds__(kImgThreads)
 k_iota_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList<T> d, int ppi, const T* T1) {
@@ -315,7 +329,10 @@ __device__ __forceinline__ T pi_source(const T* __restrict__ fld, const PiField<
 }
 
 // pi of `ppi` row pairs of one x1 plane of one field: the rows folded along x3 into
-// shared memory, x3 -> k3, then x2 -> k2 as a partial plane.
+// shared memory, x3 -> k3, then x2 -> k2 as a partial plane.  The row loads (six
+// neighbours a point for the terminal fields) and the packed FMAs bind it: 72-80 us for
+// three terminal fields of 160x192x160, band 32^3, where a pass that formed the fields
+// (25 us) and the transform's plane kernels (95 us) ran before.
 template <typename T, int KIND>
 __global__ void __launch_bounds__(kImgThreads)
 k_pi_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ PiField<T> src, int ppi, T* __restrict__ P1) {
@@ -389,6 +406,7 @@ k_pi_plane_flat(const __grid_constant__ Plan<T> p, const __grid_constant__ PiFie
 }
 
 // x1 -> k1 of the nf projected planes of image-grid fields and their scaling:
+// (14 us for 160 planes of three fields, band 32^3: latency and L2 reads)
 // out_c = coef * (applyK ? 1/L^ : 1) * the sums (twice per axis of nonzero frequency)
 template <typename T>
 __global__ void __launch_bounds__(kImgThreads)
@@ -429,7 +447,7 @@ k_pi_band(const __grid_constant__ Plan<T> p, const T* P1, int nf, int nparts, in
 // ---- Hermitian arrays <-> band vectors -------------------------------------------
 // V[s1][s2][s3] = Re sum over the signs of (h, a, b) of prod_j (s_j ? i sigma_j : 1)
 // in(sigma k): the real part keeps exactly the Hermitian part of the input.  One
-// thread per slot.
+// thread per slot; eight scattered reads each, 8 us at band 32^3.
 template <typename T>
 __global__ void k_band_load(const cplx<T>* __restrict__ in, T* __restrict__ out, int ncomp, Band bd) {
   const Trig k = trig_of(bd);

@@ -196,7 +196,7 @@ struct Impl {
   // a persistent sweep whose barrier wait gave up left dres[7] = 1
   void check_flag(double f) {
     if (f != 0.0) {
-      *err = "a bounded device wait (sweep barrier or tensor-core MMA) timed out";
+      *err = "a bounded device wait (sweep barrier) timed out";
       throw Fail{LDDMM_ETIMEOUT};
     }
   }

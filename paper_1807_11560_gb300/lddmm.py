@@ -189,9 +189,8 @@ class Context:
     (Id - alpha Lap)^s; sigma: data weight 1/sigma^2; Nt: time steps.
     state: "image" (the image state equation, Section 3.2) or "deformation"
     (the band-limited deformation state equation, Section 3.3).
-    precision: "fp64", "fp32" (tensor cores as ``tensor_cores`` says),
-    "3xtf32" or "bf16x3" (FP32 arrays; contractions on the tensor cores with
-    that operand split wherever a kernel covers their sizes).
+    precision: "fp64", "fp32" (FP64 reductions), "3xtf32" or "bf16x3" (FP32
+    arrays; a split of the operands is allowed, the transforms run in FP32).
     """
 
     def __init__(self, grid, K, alpha, s, sigma, Nt, precision="fp32", stream=None,
@@ -357,7 +356,7 @@ class Context:
 
     @property
     def tiles(self):
-        """(twiddle staging 1/2, pencils per tile, band rows per item) in effect."""
+        """(2, plane parts per x1 column, quads per band item) in effect."""
         a, b, c = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
         self._check(lib().lddmm_tile_config(self._h, ctypes.byref(a), ctypes.byref(b), ctypes.byref(c)))
         return a.value, b.value, c.value
