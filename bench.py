@@ -5,8 +5,7 @@ One step = one whole inexact Gauss-Newton-Krylov solve of the hot path from
 v0 = 0: 10 GN iterations, each a gradient (forward shoot, transport, adjoint
 Jacobi sweep), 20 PCG iterations (one GN Hessian-vector product each) and an
 Armijo line search.  Default workload: the 160x192x160 brain phantom, band
-32^3, Nt = 10, FP32 with FP64 reductions and tcgen05 3xTF32 transforms (the
-largest single-GPU configuration); ``--workload 3d_64_ellipsoids`` runs the
+32^3, Nt = 10, FP32 with FP64 reductions (the largest single-GPU configuration); ``--workload 3d_64_ellipsoids`` runs the
 64^3 ellipsoid phantom, band 16^3.  ``value`` = Hessian-vector products per
 second over the timed steps, summed over ranks (each rank registers its own
 pair: weak scaling, no collective on the data path).
@@ -53,12 +52,11 @@ def parse():
                     help="constraint: image state equation (Section 3.2) or band-limited deformation "
                          "state equation (Section 3.3)")
     ap.add_argument("--tensor-cores", default="auto", choices=["auto", "on", "off"],
-                    help="image-grid band-to-grid transforms on tcgen05 (3xTF32): auto = grids >= 2^20 voxels")
+                    help="accepted by the library; the transforms run in FP32 whatever it says")
     ap.add_argument("--persistent", default="auto", choices=["auto", "on", "off"],
-                    help="band-limited sweeps as one persistent kernel: auto = padded grids up to 32^3")
+                    help="band-limited sweeps as one persistent kernel (on) or two kernels per evaluation")
     ap.add_argument("--precision", default=None, choices=["fp32", "3xtf32", "bf16x3", "fp64"],
-                    help="fp32: tensor cores per --tensor-cores (3xTF32); 3xtf32 / bf16x3: every contraction "
-                         "with a tensor-core kernel for its sizes on tcgen05 with that operand split; fp64; "
+                    help="fp32, fp64; 3xtf32 / bf16x3 allow an operand split and run as fp32; "
                          "default: the workload's (fp64 for 2d_64_blobs, else fp32)")
     ap.add_argument("--grid", default=None,
                     help="override the workload's image grid, e.g. 64,64,64 (a smaller case of the same "
@@ -346,26 +344,6 @@ PROBE_CLASSES = ("sweep", "iota_ab", "cpw", "pi_ba", "inc_step", "transport", "i
 HBM_CLASSES = ("inc_step", "transport")
 FP32_LANES = 128
 NOMINAL_FP64_TFLOPS = 1.25
-# nominal dense tensor rates of the GB300 (PFLOP/s): TF32 takes the measured
-# BF16 peak times their ratio, and the 3xTF32 split issues three TF32 MMAs per
-# product, so its peak in algorithmic flops is a third of that
-NOMINAL_TF32_OVER_BF16 = 1.1 / 2.25
-# kernel classes whose contractions run on tcgen05 (3xTF32) in the per-evaluation
-# launches of padded grids above 32^3 points (the default tensor-core setting):
-# iota A+B, C / bracket products / C', pi B'+A'
-TENSOR_CLASSES = ("iota_ab", "cpw", "pi_ba")
-
-
-def tensor_chain(args, Ks):
-    """True when the bracket evaluations run as per-evaluation tcgen05 kernels."""
-    import numpy as np
-    mvol = int(np.prod([(3 * k + 1) // 2 for k in Ks]))
-    persistent = args.persistent == "on" or (args.persistent == "auto" and mvol <= 32768)
-    if persistent or args.tensor_cores == "off":
-        return False
-    if args.precision == "fp64":
-        return False
-    return args.tensor_cores == "on" or args.precision in ("3xtf32", "bf16x3") or mvol > 32768
 
 
 def pick_dominant(ctx, v, n_pcg):
@@ -517,25 +495,16 @@ def run_gpu(args):
             mhz = clk.get("sm_mhz") or 2070.0
             sms = torch.cuda.get_device_properties(dev).multi_processor_count
             achieved = work / avg_s / 1e12
-            tf32 = peaks.get("bf16_tflops", FALLBACK_PEAKS["bf16_tflops"]) * NOMINAL_TF32_OVER_BF16
-            tensor = {"peak": tf32 / 3.0, "frac": achieved / (tf32 / 3.0),
-                      "peak_source": f"{src} BF16 dense peak x 1.1/2.25 (nominal TF32/BF16) / 3 "
-                                     f"(3xTF32: three TF32 MMAs per product; of {src})"}
-            if probe_cls in TENSOR_CLASSES and tensor_chain(args, Ks):
-                peak = tensor["peak"]
-                roof = {"bound": "tensor", "unit": "TFLOP/s", "peak_source": tensor["peak_source"]}
+            if fp64:
+                peak = NOMINAL_FP64_TFLOPS
+                roof = {"bound": "alu", "unit": "TFLOP/s",
+                        "peak_source": f"nominal GB300 FP64 rate ({NOMINAL_FP64_TFLOPS} TFLOP/s); FP64 SIMT "
+                                       "contraction"}
             else:
-                if fp64:
-                    peak = NOMINAL_FP64_TFLOPS
-                    roof = {"bound": "alu", "unit": "TFLOP/s",
-                            "peak_source": f"nominal GB300 FP64 rate ({NOMINAL_FP64_TFLOPS} TFLOP/s); FP64 SIMT "
-                                           "contraction"}
-                else:
-                    peak = sms * FP32_LANES * 2 * mhz * 1e6 / 1e12
-                    roof = {"bound": "alu", "unit": "TFLOP/s",
-                            "peak_source": f"derived: {sms} SMs x {FP32_LANES} FP32 lanes x 2 flop x {mhz:.0f} MHz "
-                                           "(median sampled SM clock); FP32 SIMT contraction",
-                            "vs_tensor_3xtf32": tensor}
+                peak = sms * FP32_LANES * 2 * mhz * 1e6 / 1e12
+                roof = {"bound": "alu", "unit": "TFLOP/s",
+                        "peak_source": f"derived: {sms} SMs x {FP32_LANES} FP32 lanes x 2 flop x {mhz:.0f} MHz "
+                                       "(median sampled SM clock); FP32 SIMT contraction"}
             wunit = "flop"
         roof.update({"kernel": probe_cls, "achieved": achieved, "peak": peak, "frac": achieved / peak,
                      "traffic": measured_traffic(name, probe_cls), "traffic_unit": "B per launch (ncu)",
@@ -573,9 +542,8 @@ def run_gpu(args):
                        "l2": f"flushed between steps ({L2_FLUSH_BYTES >> 20} MiB write)",
                        "parallelism": f"replicas x{world}",
                        "precision": args.precision,
-                       "tensor_cores": f"{args.tensor_cores} (tcgen05 3xTF32: image-grid iota on grids of at "
-                                       "least 2^20 voxels, bracket evaluations launched per evaluation)",
-                       "tiles": dict(zip(("iota_ab_twiddles", "cpw_pencils", "pi_rows"), ctx.tiles))},
+                       "tensor_cores": f"{args.tensor_cores} (transforms run in FP32)",
+                       "tiles": dict(zip(("twiddles", "plane_parts", "band_quads"), ctx.tiles))},
             "gn_solve_s": 1e-3 * statistics.mean(step_ms),
             "gn_solve_note": f"mean timed step: one lddmm_gn_solve call ({rep_t['gn_iters']} GN iterations and "
                              f"{rep_t['pcg_iters']} products ran, E {rep_t['E_initial']:.6g} -> "
@@ -602,8 +570,8 @@ def run_population(args):
     all pairs at once through lddmm_batch_gn_solve (one CUDA stream and one host
     thread per context).  The work spans 32 streams, so steps are timed by the host
     clock between device synchronisations.  Also reported: the same contexts solved
-    one after another, and the population with plain FP32 SIMT transforms instead of
-    the tcgen05 3xTF32 split."""
+    one after another, and the population with tensor_cores off (the same FP32
+    kernels: the two have to agree)."""
     import collections
 
     import numpy as np
@@ -643,7 +611,7 @@ def run_population(args):
         return hv / t, t / steps, v0s
 
     # one pair of each grid and band: gradient and GN product at the pair's seeded
-    # point, for the split-precision against the plain FP32 comparison
+    # point, for the comparison of the two settings
     picked, seen = [], set()
     for i, (_, Ns, Ks, _, _) in enumerate(pop):
         if (tuple(Ns), tuple(Ks)) not in seen:
@@ -683,7 +651,7 @@ def run_population(args):
     prod_plain = products(made)
     for m in made:
         m[0].close()
-    # one GN step from v0 = 0 on the same images: the two precisions' updates
+    # one GN step from v0 = 0 on the same images: the two settings' updates
     diffs = [float(np.linalg.norm(a - b) / max(np.linalg.norm(b), 1e-30)) for a, b in zip(v_tc, v_plain)]
     hist = collections.Counter(f"{'x'.join(map(str, g))}/K{k[0]}" for _, g, k, _, _ in pop)
     line = {
@@ -693,7 +661,7 @@ def run_population(args):
         "config": {"workload": "population_32", "pairs": len(pop), "grids_bands": dict(hist), "Nt": 10,
                    "pcg_per_gn": N_PCG, "step": "one GN iteration on every pair",
                    "timer": "host clock between device synchronisations (32 streams)",
-                   "tensor_cores": "auto (grids of at least 2^20 voxels)"},
+                   "tensor_cores": "auto (transforms run in FP32)"},
         "sequential_value": seq_value,
         "plain_fp32_value": plain_value,
         "split_vs_plain_rel_update_diff_max": max(diffs),
