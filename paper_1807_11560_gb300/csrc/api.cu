@@ -350,7 +350,7 @@ int lddmm_tile_config(const lddmm_ctx* ctx, int* tws, int* tp, int* kc) {
   if (!ctx || !ctx->impl || !tws || !tp || !kc) return LDDMM_EINVAL;
   auto read = [&](const auto& p) {
     *tws = 2;
-    *tp = p.geom[lddmm::PW_GT].ppc;
+    *tp = p.geom[lddmm::PW_GT].nparts;
     *kc = 1 << p.geom[lddmm::PW_GT].tqs;
   };
   if (ctx->precision == LDDMM_FP64) read(static_cast<const Impl<double>*>(ctx->impl)->pad);
