@@ -147,6 +147,7 @@ struct Impl {
   // ---------------------------------------------------------------- utils
   void cuda(cudaError_t e, const char* what) {
     if (e != cudaSuccess) {
+      cudaGetLastError();   // reported here: not again by the next check_launch of this thread
       *err = std::string(what) + ": " + cudaGetErrorString(e);
       throw Fail{LDDMM_ECUDA};
     }
