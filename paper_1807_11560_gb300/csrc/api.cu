@@ -70,9 +70,13 @@ int dispatch(lddmm_ctx* ctx, Fn&& fn) {
     ctx->err = "cannot make the context's device current";
     return LDDMM_ECUDA;
   }
+  auto call = [&](auto& im) {
+    im.pending = false;   // the deferred epilogue of a call that failed part way
+    fn(im);
+  };
   if (ctx->precision == LDDMM_FP64)
-    return guarded(ctx, [&] { fn(*static_cast<Impl<double>*>(ctx->impl)); });
-  return guarded(ctx, [&] { fn(*static_cast<Impl<float>*>(ctx->impl)); });
+    return guarded(ctx, [&] { call(*static_cast<Impl<double>*>(ctx->impl)); });
+  return guarded(ctx, [&] { call(*static_cast<Impl<float>*>(ctx->impl)); });
 }
 
 bool bad_ptr(lddmm_ctx* ctx, const void* p, const char* name) {

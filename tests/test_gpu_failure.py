@@ -79,3 +79,18 @@ def test_the_call_after_a_refused_one_works(context):
     errors = _refused_then(ctx, v, torch.empty_like(v), lambda: ctx.hessvec(p, out))
     assert errors[1] is None
     np.testing.assert_array_equal(out.cpu().numpy(), ref.cpu().numpy())
+
+
+def test_the_call_after_a_refused_one_launches_its_own_kernels_only(context):
+    import torch
+    ctx, v, p, ref, kernels = context
+    counts = []
+
+    def then():
+        counts.append(ctx.kernel_count)
+        ctx.hessvec(p, torch.empty_like(p))
+        counts.append(ctx.kernel_count)
+
+    errors = _refused_then(ctx, v, torch.empty_like(v), then)
+    assert errors[1] is None
+    assert counts[1] - counts[0] == kernels
