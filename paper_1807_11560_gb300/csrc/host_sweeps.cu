@@ -19,10 +19,10 @@ void Impl<T>::eval(PwMode mode, T* slot, const C* srcA, const C* srcB, const PiE
   if (proj) link(pend_epi, srcA, srcB);
   pb(PR_PI_BA);
   cuda(band_phase<T>(pad, mode, proj ? &pend_epi : nullptr, P1, srcA, srcB, T1, Lhat, st), "band phase");
-  pe(PR_PI_BA, 2.0 * K.vol() * M.n1 * (mode_in(mode) + (proj ? mode_out(pend_mode) : 0)) * 0.5);
+  pe(PR_PI_BA, band_flops(eval_in(mode) + (proj ? eval_out(pend_mode) : 0)));
   pb(PR_CPW);
   cuda(plane_phase<T>(pad, mode, T1, slot, slot2, P1, st), "plane phase");
-  pe(PR_CPW, eval_flops(mode) - (double)K.vol() * M.n1 * (mode_in(mode) + mode_out(mode)));
+  pe(PR_CPW, plane_flops(mode));
   launches += kEvalLaunches;
   pending = true;
   pend_mode = mode;
@@ -36,7 +36,7 @@ void Impl<T>::flush() {
   if (pend_epi.nout == 0) return;
   pb(PR_PI_BA);
   cuda(band_phase<T>(pad, pend_mode, &pend_epi, P1, nullptr, nullptr, T1, Lhat, st), "band phase");
-  pe(PR_PI_BA, (double)K.vol() * M.n1 * mode_out(pend_mode));
+  pe(PR_PI_BA, band_flops(eval_out(pend_mode)));
   ++launches;
 }
 
@@ -46,7 +46,7 @@ void Impl<T>::run_sweep(PwMode mode, const EvalDesc<T>* ev, int nev) {
   pb(PR_SWEEP);
   cuda(sweep_launch<T>(pad, mode, ev, nev, Lhat, T1, P1, bar, dres + 7, st, opts.debug_stall),
        "persistent sweep");
-  pe(PR_SWEEP, eval_flops(mode) * nev);
+  pe(PR_SWEEP, (band_flops(eval_in(mode) + eval_out(mode)) + plane_flops(mode)) * nev);
   ++launches;
 }
 

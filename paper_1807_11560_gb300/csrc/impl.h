@@ -274,15 +274,21 @@ struct Impl {
   }
 
   // operations of the transforms of nf scalar fields between the band and grid g
-  // (folded cosine/sine sums: K/2 products per point and axis)
+  // (folded cosine/sine sums: K/2 products per point and axis; 2D has no third axis)
   double grid_flops(const Dims& g, int nf) const {
     const double k1 = K.k1, k2 = K.k2, k3 = K.k3, n1 = g.n1;
-    return nf * (k1 * n1 * k2 * k3 + n1 * k2 * g.n2 * k3 + n1 * (double)g.n2 * k3 * g.n3);
+    return nf * (k1 * n1 * k2 * k3 + n1 * k2 * g.n2 * k3 + (pad.flat ? 0.0 : n1 * (double)g.n2 * k3 * g.n3));
   }
-  // operations of one evaluation: its transforms and, roughly, the point products
-  double eval_flops(PwMode mode) const {
-    const double per_point[PW_MODES] = {30, 60, 60, 90, 21, 39, 18};
-    return grid_flops(M, mode_in(mode) + mode_out(mode)) + per_point[mode] * (double)Mvol;
+  // fields that an evaluation transforms, in and out
+  int eval_in(PwMode mode) const { return fields_in(mode, pad.flat); }
+  int eval_out(PwMode mode) const { return fields_out(mode, pad.flat); }
+  // operations of n fields of an evaluation in the band phase, and of its plane phase
+  // (with, roughly, the point products)
+  double band_flops(int n) const { return n * (double)Kuser * M.n1; }
+  double plane_flops(PwMode mode) const {
+    const double per_point[2][PW_MODES] = {{30, 60, 60, 90, 21, 39, 18}, {10, 22, 23, 34, 8, 16, 8}};
+    const int n = eval_in(mode) + eval_out(mode);
+    return grid_flops(M, n) - band_flops(n) + per_point[pad.flat][mode] * (double)Mvol;
   }
 
   // One evaluation of a pseudo-spectral expression (PwMode) with sources srcA,

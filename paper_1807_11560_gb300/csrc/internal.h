@@ -100,6 +100,18 @@ enum PwMode : int { PW_F = 0, PW_T, PW_TC, PW_GT, PW_D0, PW_D1, PW_D2, PW_MODES 
 __host__ __device__ constexpr int mode_in(int m) { return m == PW_T ? 10 : (m >= PW_D0 ? 12 : 18); }
 __host__ __device__ constexpr int mode_out(int m) { return m == PW_GT ? 11 : (m >= PW_D0 ? 3 : 4); }
 __host__ __device__ constexpr int mode_nper(int m) { return m == PW_GT ? 3 : 1; }
+// 2D problems (one point and one frequency on axis 3, "flat") have no third
+// component: their evaluations keep only the fields without one, in the order
+//   PW_F, PW_TC, PW_GT  A_1, A_2, d_1 A_1, d_2 A_1, d_1 A_2, d_2 A_2, m_1, m_2, (curl m)_3
+//   PW_T                A_1, A_2, div A, m_1, m_2, (curl m)_3
+//   deformation         d_1 A_1, d_2 A_1, d_1 A_2, d_2 A_2, B_1, B_2
+// and the sine columns of axis 3 are zero and skipped.
+__host__ __device__ constexpr int fields_in(int m, bool flat) {
+  return !flat ? mode_in(m) : (m == PW_T || m >= PW_D0 ? 6 : 9);
+}
+__host__ __device__ constexpr int fields_out(int m, bool flat) {
+  return !flat ? mode_out(m) : (m == PW_GT ? 8 : (m >= PW_D0 ? 2 : 3));
+}
 constexpr int kSlotFields = 18, kDefFields = 12, kMaxOutFields = 11, kMaxInFields = 18;
 
 // How an evaluation mode is cut into work items: the plane phase handles

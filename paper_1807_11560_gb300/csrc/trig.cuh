@@ -134,19 +134,6 @@ __device__ __forceinline__ void copy2(V2<T>* dst, const Pair<T>* src, int n) {
   for (int i = threadIdx.x; i < n; i += NT) dst[i] = s[i];
 }
 
-// 2D problems (one point and one frequency on axis 3, "flat") have no third
-// component: their evaluations keep only the fields without one, in the order
-//   PW_F, PW_TC, PW_GT  A_1, A_2, d_1 A_1, d_2 A_1, d_1 A_2, d_2 A_2, m_1, m_2, (curl m)_3
-//   PW_T                A_1, A_2, div A, m_1, m_2, (curl m)_3
-//   deformation         d_1 A_1, d_2 A_1, d_1 A_2, d_2 A_2, B_1, B_2
-// and the sine columns of axis 3 are zero and skipped.
-__host__ __device__ constexpr int fields_in(int m, bool flat) {
-  return !flat ? mode_in(m) : (m == PW_T || m >= PW_D0 ? 6 : 9);
-}
-__host__ __device__ constexpr int fields_out(int m, bool flat) {
-  return !flat ? mode_out(m) : (m == PW_GT ? 8 : (m >= PW_D0 ? 2 : 3));
-}
-
 // x / n for the kernels' index splits (exact while x * n < 2^32)
 __device__ __forceinline__ int fdiv(int x, FastDiv d) { return d.m ? (int)__umulhi((unsigned)x, d.m) : x; }
 

@@ -2,9 +2,9 @@
 
 import pytest
 
-from paper_1807_11560_gb300 import Context
+from paper_1807_11560_gb300 import Context, inputs
 
-from helpers import ALPHA, S, SIGMA
+from helpers import ALPHA, S, SIGMA, torch_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -15,3 +15,33 @@ pytestmark = pytest.mark.gpu
 def test_tiles_are_parts_and_quads(Ks, parts, quads):
     with Context(Ks, Ks, ALPHA, S, SIGMA, 1, precision="fp32") as ctx:
         assert ctx.tiles == (2, parts, quads)
+
+
+def _probed(ctx, kernel_class, call):
+    """(ms, launches, work) of one kernel class during call()."""
+    ctx.probe(kernel_class)
+    call()
+    got = ctx.probe_read()
+    ctx.probe(None)
+    return got
+
+
+@pytest.mark.parametrize("persistent", [False, True])
+def test_probe_counts_the_operations_of_2d_evaluations(persistent):
+    """A 2D shoot evaluation transforms 9 fields in and 3 out over two axes (K/2 products
+    of two sums a point and axis) and takes 10 operations a point for the products."""
+    import torch
+    (K1, K2), Nt = (14, 10), 3
+    M1, M2 = 21, 15
+    band, plane = 12 * K1 * M1 * K2, 12 * M1 * K2 * M2 + 10 * M1 * M2
+    v = torch_dev(inputs.random_bl((K1, K2), 2, 3, 1.0, (K1, K2)), "fp32")
+    with Context((K1, K2), (K1, K2), ALPHA, S, SIGMA, Nt, precision="fp32", persistent=persistent) as ctx:
+        shoot = lambda: ctx.shoot(v, torch.empty_like(v))
+        if persistent:
+            expect = {"sweep": (1, 2 * Nt * (band + plane))}
+        else:
+            expect = {"pi_ba": (2 * Nt + 1, 2 * Nt * band), "cpw": (2 * Nt, 2 * Nt * plane)}
+        for kernel_class, (launches, work) in expect.items():
+            ms, n, w = _probed(ctx, kernel_class, shoot)
+            assert n == launches and ms > 0
+            assert w == pytest.approx(work, rel=1e-12)
