@@ -338,8 +338,11 @@ int lddmm_last_dm1(lddmm_ctx* ctx, void* dm1_out);
  *                product grid (Eqs. 48-49): the plane phase (x2-x3 transforms
  *                and the bracket products) and the band phase (x1 transforms,
  *                spectral multipliers, time-step updates); work = flops of
- *                their contractions and products ("iota_ab" and "deform" name
- *                classes without launches of their own);
+ *                their contractions and products ("iota_ab" names a class
+ *                without launches of its own);
+ *   "deform"     one evaluation of the deformation products (Section 3.3), both its
+ *                kernels together, and the projection that ends a sweep of them;
+ *                work = flops;
  *   "iota_full", "pi_full"  transforms on the image grid; work = flops;
  *   "sweep"      one persistent band-limited sweep kernel; work = flops;
  * NULL or "" switches the probe off.  Changing the class rebuilds the graph

@@ -17,12 +17,17 @@ void Impl<T>::eval(PwMode mode, T* slot, const C* srcA, const C* srcB, const PiE
   if (pending && pend_mode != mode) flush();
   const bool proj = pending && pend_epi.nout > 0;
   if (proj) link(pend_epi, srcA, srcB);
-  pb(PR_PI_BA);
+  // the probe takes a deformation evaluation whole, a bracket by its two kernels
+  const bool whole = mode >= PW_D0;
+  const double in_band = band_flops(eval_in(mode) + (proj ? eval_out(pend_mode) : 0));
+  pb(whole ? PR_DEFORM : PR_PI_BA);
   cuda(band_phase<T>(pad, mode, proj ? &pend_epi : nullptr, P1, srcA, srcB, T1, Lhat, st), "band phase");
-  pe(PR_PI_BA, band_flops(eval_in(mode) + (proj ? eval_out(pend_mode) : 0)));
-  pb(PR_CPW);
+  if (!whole) {
+    pe(PR_PI_BA, in_band);
+    pb(PR_CPW);
+  }
   cuda(plane_phase<T>(pad, mode, T1, slot, slot2, P1, st), "plane phase");
-  pe(PR_CPW, plane_flops(mode));
+  pe(whole ? PR_DEFORM : PR_CPW, plane_flops(mode) + (whole ? in_band : 0.0));
   launches += kEvalLaunches;
   pending = true;
   pend_mode = mode;
@@ -34,9 +39,10 @@ void Impl<T>::flush() {
   if (rec || !pending) return;
   pending = false;
   if (pend_epi.nout == 0) return;
-  pb(PR_PI_BA);
+  const int cls = pend_mode >= PW_D0 ? PR_DEFORM : PR_PI_BA;
+  pb(cls);
   cuda(band_phase<T>(pad, pend_mode, &pend_epi, P1, nullptr, nullptr, T1, Lhat, st), "band phase");
-  pe(PR_PI_BA, band_flops(eval_out(pend_mode)));
+  pe(cls, band_flops(eval_out(pend_mode)));
   ++launches;
 }
 

@@ -45,3 +45,21 @@ def test_probe_counts_the_operations_of_2d_evaluations(persistent):
             ms, n, w = _probed(ctx, kernel_class, shoot)
             assert n == launches and ms > 0
             assert w == pytest.approx(work, rel=1e-12)
+
+
+def test_probe_times_deformation_evaluations():
+    """A deformation gradient: 2 Nt evaluations of the sweep and one of the terminal
+    product, each sweep ended by a projection; 12 fields in and 3 out of each."""
+    import torch
+    Ns, (K1, K2, K3), Nt = (12, 12, 12), (8, 6, 4), 3
+    M1, M2, M3 = 12, 9, 6
+    v = torch_dev(inputs.random_bl((K1, K2, K3), 3, 3, 1.0, Ns), "fp32")
+    I0, I1 = inputs.make_pair("ellipsoids", Ns, 5, max_disp=1.0)
+    with Context(Ns, (K1, K2, K3), ALPHA, S, SIGMA, Nt, precision="fp32", state="deformation") as ctx:
+        ctx.set_images(torch_dev(I0, "fp32"), torch_dev(I1, "fp32"))
+        ms, n, work = _probed(ctx, "deform", lambda: ctx.gradient(v, torch.empty_like(v)))
+        assert n == (2 * Nt + 1) + (1 + 1) and ms > 0
+        transforms = 15 * (K1 * M1 * K2 * K3 + M1 * K2 * M2 * K3 + M1 * M2 * K3 * M3)
+        assert work == pytest.approx((2 * Nt + 1) * transforms + (2 * Nt * 21 + 18) * M1 * M2 * M3, rel=1e-12)
+        # the classes of the bracket kernels leave them out
+        assert _probed(ctx, "cpw", lambda: ctx.gradient(v, torch.empty_like(v)))[1] == 2 * (2 * Nt)
