@@ -73,7 +73,9 @@ template <typename T, int MODE, bool FLAT, int MINB>
 __global__ void __launch_bounds__(kPhaseThreads, MINB)
 k_band(const __grid_constant__ BandArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  pdl_trigger();
+  // 2D bands of more items than SMs (one to an SM) let the plane phase start as they end:
+  // before, its small items would fill the SMs of the first wave and leave the rest idle
+  if (!FLAT || gridDim.x <= kSMs) pdl_trigger();
   band_item<T, MODE, kPhaseThreads, FLAT>(a.p, a.tqs, a.prev ? &a.e : nullptr, a.nparts, a.P1, a.A, a.B, a.T1, a.Lhat,
                                          blockIdx.x, reinterpret_cast<V2<T>*>(smraw));
 }
@@ -95,10 +97,11 @@ k_plane(const __grid_constant__ Plan<T> p, int ppc, int nparts, const T* T1, T* 
 // half-spectrum sums).
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kPhaseThreads)
-k_plane_flat(const __grid_constant__ Plan<T> p, const T* T1, T* slot, T* slot2, T* P1) {
+k_plane_flat(const __grid_constant__ Plan<T> p, int ppc, int nparts, const T* T1, T* slot, T* slot2, T* P1) {
   extern __shared__ __align__(16) unsigned char smraw[];
   pdl_trigger();
-  plane_item_flat<T, MODE, kPhaseThreads>(p, T1, slot, slot2, P1, blockIdx.x, reinterpret_cast<V2<T>*>(smraw));
+  plane_item_flat<T, MODE, kPhaseThreads>(p, ppc, nparts, T1, slot, slot2, P1, blockIdx.x,
+                                          reinterpret_cast<V2<T>*>(smraw));
 }
 
 // ---- image grid ----------------------------------------------------------------
@@ -364,7 +367,9 @@ k_pi_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ PiField<T>
   band_from_rows<T, kImgThreads, 1, 2>(p, Z, ppi, np, sm + s.off_2b, out);
 }
 
-// the two plane steps of a 2D image: one output per thread
+// the two plane steps of a 2D image: one output per thread.  k_pi_plane_flat takes part of
+// one plane and forms its folded points once, in shared memory: a thread that formed them
+// for itself was bound by that (FP64 terminal fields of 300 x 4096, band 64^2: 2.2 ms; 0.42).
 template <typename T>
 __global__ void __launch_bounds__(kImgThreads)
 k_iota_plane_flat(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList<T> d, const T* T1) {
@@ -386,23 +391,33 @@ k_iota_plane_flat(const __grid_constant__ Plan<T> p, const __grid_constant__ Iot
 }
 template <typename T, int KIND>
 __global__ void __launch_bounds__(kImgThreads)
-k_pi_plane_flat(const __grid_constant__ Plan<T> p, const __grid_constant__ PiField<T> src, T* __restrict__ P1) {
-  const int K2h = p.k.K2h, K2p = up8(K2h), G2 = p.g.n2, a = blockIdx.x * kImgThreads + threadIdx.x, f = blockIdx.y,
-            x1 = blockIdx.z;
+k_pi_plane_flat(const __grid_constant__ Plan<T> p, const __grid_constant__ PiField<T> src, int ppi,
+                T* __restrict__ P1) {
+  const int K2h = p.k.K2h, K2p = up8(K2h), G2 = p.g.n2, f = blockIdx.y, x1 = blockIdx.z;
+  const int t0 = blockIdx.x * ppi, t1 = min(t0 + ppi, p.NT2);
   pdl_trigger();
   pdl_wait();
-  if (a >= K2h) return;
   const T* fld = src.f[f];
-  const V2<T>* w = reinterpret_cast<const V2<T>*>(p.e2b) + a;
+  __shared__ V2<T> sZ[kImgThreads];                        // folded points, each formed once
+  const int a = threadIdx.x;                               // K_2 <= 512: a frequency per thread
   V2<T> acc = zero2<T>();
-#pragma unroll 4
-  for (int t = 0; t < p.NT2; ++t) {
-    const bool two = t > 0 && 2 * t != G2;
-    const T u = pi_source<T, KIND>(fld, src, p.g, f, x1, t, 0);
-    const T v = two ? pi_source<T, KIND>(fld, src, p.g, f, x1, G2 - t, 0) : T(0);
-    acc = fma2(two ? mk2(u + v, u - v) : mk2(u, T(0)), w[(long long)t * K2p], acc);
+  for (int c0 = t0; c0 < t1; c0 += kImgThreads) {
+    const int n = min(kImgThreads, t1 - c0), t = c0 + a;
+    if (c0 > t0) __syncthreads();
+    if (a < n) {
+      const bool two = t > 0 && 2 * t != G2;
+      const T u = pi_source<T, KIND>(fld, src, p.g, f, x1, t, 0);
+      const T v = two ? pi_source<T, KIND>(fld, src, p.g, f, x1, G2 - t, 0) : T(0);
+      sZ[a] = two ? mk2(u + v, u - v) : mk2(u, T(0));
+    }
+    __syncthreads();
+    if (a < K2h) {
+      const V2<T>* w = reinterpret_cast<const V2<T>*>(p.e2b) + (long long)c0 * K2p + a;
+      sum_flat<T>(n, acc, [&](int i) { return sZ[i]; }, [&](int i) { return w[(long long)i * K2p]; });
+    }
   }
-  stq(P1 + (((long long)x1 * gridDim.y + f) * K2h + a) * 4, Quad<T>{acc, zero2<T>()});
+  if (a < K2h)
+    stq(P1 + ((((long long)x1 * gridDim.x + blockIdx.x) * gridDim.y + f) * K2h + a) * 4, Quad<T>{acc, zero2<T>()});
 }
 
 // x1 -> k1 of the nf projected planes of image-grid fields and their scaling:
@@ -560,7 +575,12 @@ int iota_pairs(const Plan<T>& p) {
 }
 template <typename T>
 int pi_pairs(const Plan<T>& p) {
-  if (p.flat) return p.NT2;
+  if (p.flat) {
+    // a thread sums the points of an item in turn: parts of 64 row pairs while a wave has
+    // room (a pi call of a 64 x 1024 image, band 8 x 512: 88 us whole, 57 in parts)
+    const int parts = std::max(1, std::min((p.NT2 + 63) / 64, 4 * kSMs / p.g.n1));
+    return (p.NT2 + parts - 1) / parts;
+  }
   int most = std::max(1, 2 * kImgThreads / p.K3e);
   while (most > 1 && plane_shape(p, 0, 1, most, 1).smem > (size_t)96 * 1024) --most;
   return even_pairs(p.NT2, most, 1);
@@ -576,12 +596,13 @@ cudaError_t launch_plane_pt(const Plan<T>& p, const T* T1, T* slot, T* slot2, T*
 }
 template <typename T, int MODE>
 cudaError_t launch_plane(const Plan<T>& p, const T* T1, T* slot, T* slot2, T* P1, cudaStream_t st) {
-  const int pt = plane_pt(p.geom[MODE].ppc);
+  const EvalGeom g = p.geom[MODE];
+  const int pt = plane_pt(g.ppc);
   if (p.flat) {
     cudaError_t e = allow_smem<k_plane_flat<T, MODE>>();
     if (e != cudaSuccess) return e;
-    return launch_chain(k_plane_flat<T, MODE>, dim3((unsigned)p.g.n1), kPhaseThreads, plane_flat_smem(p, MODE), st, p,
-                        T1, slot, slot2, P1);
+    return launch_chain(k_plane_flat<T, MODE>, dim3((unsigned)(p.g.n1 * g.nparts)), kPhaseThreads,
+                        plane_flat_smem<T>(MODE, g.ppc), st, p, g.ppc, g.nparts, T1, slot, slot2, P1);
   }
   if (pt == 3) return launch_plane_pt<T, MODE, 3>(p, T1, slot, slot2, P1, st);
   if (pt == 5) return launch_plane_pt<T, MODE, 5>(p, T1, slot, slot2, P1, st);
@@ -647,11 +668,10 @@ cudaError_t launch_iota_plane_even(const Plan<T>& p, const IotaList<T>& d, const
 
 template <typename T, int KIND>
 cudaError_t launch_pi_plane(const Plan<T>& p, const PiField<T>& s, int nf, T* P1, cudaStream_t st) {
-  if (p.flat)
-    return launch_chain(k_pi_plane_flat<T, KIND>,
-                        dim3((unsigned)((p.k.K2h + kImgThreads - 1) / kImgThreads), (unsigned)nf, (unsigned)p.g.n1),
-                        kImgThreads, 0, st, p, s, P1);
   const int ppi = pi_pairs(p);
+  if (p.flat)
+    return launch_chain(k_pi_plane_flat<T, KIND>, dim3((unsigned)((p.NT2 + ppi - 1) / ppi), (unsigned)nf, (unsigned)p.g.n1),
+                        kImgThreads, 0, st, p, s, ppi, P1);
   cudaError_t e = allow_smem<k_pi_plane<T, KIND>>();
   if (e != cudaSuccess) return e;
   return launch_chain(k_pi_plane<T, KIND>, dim3((unsigned)((p.NT2 + ppi - 1) / ppi), (unsigned)nf, (unsigned)p.g.n1),
@@ -667,9 +687,16 @@ template <typename T>
 EvalGeom eval_geom(const Plan<T>& p, PwMode mode) {
   EvalGeom g{1, p.NT2, 0};
   if (p.flat) {
-    g.ppc = p.NT2;                                         // one item per plane
-    g.nparts = 1;
-    g.tqs = 0;
+    // Half a thread block of k2 -> x2 sums per item, while the items fit the SMs two to
+    // one.  Band 8 x 512 has 12 planes of 385 row pairs: 28 of an item's rounds of sums on
+    // 12 SMs took 490 us per evaluation of a product, 25 parts take 54.  Items of one sum
+    // per thread leave the way back longer (band 2 x 300: 46 us; 34).  At 64 x 512 in FP64,
+    // 96 planes: 1.3 ms whole, 0.75 in 3 parts.
+    const int most = std::max(1, 2 * kSMs / p.g.n1);
+    const int want = kPhaseThreads / (2 * fields_in(mode, true));
+    const int parts = std::min((p.NT2 + want - 1) / want, most);
+    g.ppc = (p.NT2 + parts - 1) / parts;
+    g.nparts = (p.NT2 + g.ppc - 1) / g.ppc;
     return g;
   }
   double best = 1e300;

@@ -99,7 +99,7 @@ k_sweep(const __grid_constant__ SweepArgs<T> a) {
     // (the test hook makes the very first barrier wait for arrivals that never come)
     if (!grid_barrier(a.bar, target, a.flag, a.spin_limit, ev == 0 ? a.stall : 0u)) return;
     for (int i = blockIdx.x; i < n_plane; i += gridDim.x) {
-      if constexpr (PT == 0) plane_item_flat<T, MODE, NT>(p, a.T1, cur->slot, cur->slot2, a.P1, i, sm);
+      if constexpr (PT == 0) plane_item_flat<T, MODE, NT>(p, a.g.ppc, a.g.nparts, a.T1, cur->slot, cur->slot2, a.P1, i, sm);
       else plane_item<T, MODE, NT, PT>(p, a.g.ppc, a.g.nparts, a.T1, cur->slot, cur->slot2, a.P1, i, sm);
       __syncthreads();
     }
@@ -160,7 +160,7 @@ cudaError_t sweep_launch(const Plan<T>& p, PwMode mode, const EvalDesc<T>* ev, i
   const bool flat = p.flat;
   const size_t smem =
       std::max(band_shape(p, 1 << a.g.tqs, fields_out(mode, flat), fields_in(mode, flat)).smem,
-               flat ? plane_flat_smem(p, mode)
+               flat ? plane_flat_smem<T>(mode, a.g.ppc)
                     : plane_shape(p, mode_in(mode), mode_out(mode), a.g.ppc, a.g.ppc <= 3 ? 3 : (a.g.ppc <= 5 ? 5 : 9)).smem);
   const int max_ctas = std::max((p.k.Kq() + (1 << a.g.tqs) - 1) >> a.g.tqs, p.g.n1 * a.g.nparts);
   cudaError_t e = cudaMemsetAsync(bar, 0, kSweepBarWords * sizeof(unsigned), st);

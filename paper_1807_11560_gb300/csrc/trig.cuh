@@ -1022,38 +1022,61 @@ __device__ __forceinline__ void products_flat(const T* x, const T* c, T* o) {
 __host__ __device__ constexpr int flat_cached(int m) { return m >= PW_D0 ? 6 : 9; }   // of a slot
 
 template <typename T>
-__host__ __device__ inline size_t plane_flat_smem(const Plan<T>& p, int mode) {
+__host__ __device__ inline size_t plane_flat_smem(int mode, int ppc) {
   const int NF = fields_in(mode, true), NO = fields_out(mode, true);
-  return (size_t)NO * p.NT2 * sizeof(V2<T>) + (size_t)(NF + NO) * p.g.n2 * sizeof(T);
+  return (size_t)NO * ppc * sizeof(V2<T>) + (size_t)(NF + NO) * 2 * ppc * sizeof(T);
 }
 
-// one plane of a 2D evaluation: x2 transforms only, one sum per thread
+// acc += sum of a(i) b(i), i < n, eight loads of each in flight
+template <typename T, typename A, typename B>
+__device__ __forceinline__ void sum_flat(int n, V2<T>& acc, A&& a, B&& b) {
+  int i = 0;
+  for (; i + 8 <= n; i += 8) {
+    V2<T> u[8], w[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      u[k] = a(i + k);
+      w[k] = b(i + k);
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc = fma2(u[k], w[k], acc);
+  }
+#pragma unroll 4
+  for (; i < n; ++i) acc = fma2(a(i), b(i), acc);
+}
+
+// one plane item of a 2D evaluation: x2 transforms of the row pairs [part ppc, ...) of
+// plane x1, one sum per thread.  Rows i and np + i are x2 = t and G2 - t.
 template <typename T, int MODE, int NT>
-__device__ __forceinline__ void plane_item_flat(const Plan<T>& p, const T* T1, T* slot, T* slot2, T* P1, int x1,
-                                                V2<T>* sm) {
+__device__ __forceinline__ void plane_item_flat(const Plan<T>& p, int ppc, int nparts, const T* T1, T* slot, T* slot2,
+                                                T* P1, int item, V2<T>* sm) {
   constexpr int NF = fields_in(MODE, true), NO = fields_out(MODE, true), NS = flat_cached(MODE);
   const int K2h = p.k.K2h, NT2 = p.NT2, G2 = p.g.n2, K2p = up8(K2h);
-  const V2<T>*tF = reinterpret_cast<const V2<T>*>(p.e2f), *tB = reinterpret_cast<const V2<T>*>(p.e2b);
-  V2<T>* sE = sm;                                          // folded products [o][t]
-  T *sX = reinterpret_cast<T*>(sE + NO * NT2), *sO = sX + NF * G2;
+  const int x1 = item / nparts, t0 = (item - x1 * nparts) * ppc, np = min(ppc, NT2 - t0), R = 2 * np;
+  const V2<T>*tF = reinterpret_cast<const V2<T>*>(p.e2f) + t0,
+             *tB = reinterpret_cast<const V2<T>*>(p.e2b) + (long long)t0 * K2p;
+  V2<T>* sE = sm;                                          // folded products [o][i]
+  T *sX = reinterpret_cast<T*>(sE + NO * np), *sO = sX + NF * R;
+  auto single = [&](int t) { return t == 0 || 2 * t == G2; };
   pdl_wait();
-  for (int it = threadIdx.x; it < NF * NT2; it += NT) {
-    const int f = it / NT2, t = it - f * NT2;
+  for (int it = threadIdx.x; it < NF * np; it += NT) {
+    const int f = it / np, i = it - f * np;
     const T* v = T1 + ((long long)x1 * NF + f) * K2h * 4;
     V2<T> acc = zero2<T>();
-#pragma unroll 8
-    for (int a = 0; a < K2h; ++a) acc = fma2(ldq(v + 4 * a).c, tF[a * NT2 + t], acc);
+    sum_flat<T>(K2h, acc, [&](int a) { return ldq(v + 4 * a).c; }, [&](int a) { return tF[a * NT2 + i]; });
     T E, O;
     un2(acc, E, O);
-    sX[f * G2 + t] = E + O;
-    if (t > 0 && 2 * t != G2) sX[f * G2 + G2 - t] = E - O;
+    sX[f * R + i] = E + O;
+    sX[f * R + np + i] = E - O;
   }
   __syncthreads();
-  for (int x2 = threadIdx.x; x2 < G2; x2 += NT) {
-    const long long at = (long long)x1 * G2 + x2;
+  for (int r = threadIdx.x; r < R; r += NT) {
+    const int u = t0 + (r < np ? r : r - np);
+    if (r >= np && single(u)) continue;
+    const long long at = (long long)x1 * G2 + (r < np ? u : G2 - u);
     T x[NF], c[NS], o[NO];
 #pragma unroll
-    for (int f = 0; f < NF; ++f) x[f] = sX[f * G2 + x2];
+    for (int f = 0; f < NF; ++f) x[f] = sX[f * R + r];
 #pragma unroll
     for (int i = 0; i < NS; ++i)
       c[i] = MODE == PW_T || MODE == PW_TC || MODE == PW_GT || MODE == PW_D1 ? slot[NS * at + i] : T(0);
@@ -1065,23 +1088,22 @@ __device__ __forceinline__ void plane_item_flat(const Plan<T>& p, const T* T1, T
     }
     products_flat<T, MODE>(x, c, o);
 #pragma unroll
-    for (int i = 0; i < NO; ++i) sO[i * G2 + x2] = o[i];
+    for (int i = 0; i < NO; ++i) sO[i * R + r] = o[i];
   }
   __syncthreads();
-  for (int it = threadIdx.x; it < NO * NT2; it += NT) {
-    const int o = it / NT2, t = it - o * NT2;
-    const T u = sO[o * G2 + t];
-    const bool two = t > 0 && 2 * t != G2;
-    const T v = two ? sO[o * G2 + G2 - t] : T(0);
+  for (int it = threadIdx.x; it < NO * np; it += NT) {
+    const int o = it / np, i = it - o * np;
+    const T u = sO[o * R + i];
+    const bool two = !single(t0 + i);
+    const T v = two ? sO[o * R + np + i] : T(0);
     sE[it] = two ? mk2(u + v, u - v) : mk2(u, T(0));
   }
   __syncthreads();
   for (int it = threadIdx.x; it < NO * K2h; it += NT) {
     const int o = it / K2h, a = it - o * K2h;
     V2<T> acc = zero2<T>();
-#pragma unroll 4
-    for (int t = 0; t < NT2; ++t) acc = fma2(sE[o * NT2 + t], tB[(long long)t * K2p + a], acc);
-    stq(P1 + (((long long)x1 * NO + o) * K2h + a) * 4, Quad<T>{acc, zero2<T>()});
+    sum_flat<T>(np, acc, [&](int i) { return sE[o * np + i]; }, [&](int i) { return tB[(long long)i * K2p + a]; });
+    stq(P1 + (((long long)item * NO + o) * K2h + a) * 4, Quad<T>{acc, zero2<T>()});
   }
 }
 
