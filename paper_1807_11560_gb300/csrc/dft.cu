@@ -420,13 +420,51 @@ k_pi_plane_flat(const __grid_constant__ Plan<T> p, const __grid_constant__ PiFie
     stq(P1 + ((((long long)x1 * gridDim.x + blockIdx.x) * gridDim.y + f) * K2h + a) * 4, Quad<T>{acc, zero2<T>()});
 }
 
+// The Hermitian array at the signs neg of the frequencies f from the coefficients
+// v(s1, s2, s3): the sum of prod_j w_j v, w = 1 for a zero frequency, else 1/2 (cosine) or
+// -i sigma / 2 (sine)
+template <typename T, typename V>
+__device__ __forceinline__ cplx<T> hermitian_value(const int* f, const bool* neg, V&& v) {
+  cplx<T> z{T(0), T(0)};
+#pragma unroll
+  for (int m = 0; m < 8; ++m) {
+    const int sn[3] = {m & 1, (m >> 1) & 1, (m >> 2) & 1};
+    T w = T(1);
+    int turns = 0;                                         // factors -i
+    bool skip = false;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      if (f[j] == 0) {
+        if (sn[j]) skip = true;
+        continue;
+      }
+      w *= T(0.5);
+      if (sn[j]) {
+        ++turns;
+        if (neg[j]) w = -w;
+      }
+    }
+    if (skip) continue;
+    const T u = w * v(sn[0], sn[1], sn[2]);
+    if (turns == 0) z.x += u;
+    else if (turns == 1) z.y -= u;
+    else if (turns == 2) z.x -= u;
+    else z.y += u;
+  }
+  return z;
+}
+
 // x1 -> k1 of the nf projected planes of image-grid fields and their scaling:
 // (14 us for 160 planes of three fields, band 32^3: latency and L2 reads)
-// out_c = coef * (applyK ? 1/L^ : 1) * the sums (twice per axis of nonzero frequency)
-template <typename T>
+// coef * (applyK ? 1/L^ : 1) * the sums (twice per axis of nonzero frequency), as band
+// vectors out, or with HERM as the Hermitian arrays herm.  A quad holds every sign of its
+// frequencies (the Nyquist slots stand where the negative of a zero would), so an item
+// writes them without the launch and the round trip of k_band_store (a call on host
+// arrays, 2D 64^2 / 16^2: 60 us with it, 50; on device arrays at 64^3 / 16^3: 40, 36).
+template <typename T, bool HERM>
 __global__ void __launch_bounds__(kImgThreads)
 k_pi_band(const __grid_constant__ Plan<T> p, const T* P1, int nf, int nparts, int tqs, T coef, int applyK,
-          const T* __restrict__ Lhat, T* __restrict__ out) {
+          const T* __restrict__ Lhat, T* __restrict__ out, cplx<T>* __restrict__ herm) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int PC = 4 << tqs, H1 = p.k.H1, q0 = blockIdx.x << tqs, nq = min(1 << tqs, p.k.Kq() - q0), H1p = up4(H1);
   V2<T>* sW = reinterpret_cast<V2<T>*>(smraw);             // [kChunk][H1p]
@@ -444,17 +482,45 @@ k_pi_band(const __grid_constant__ Plan<T> p, const T* P1, int nf, int nparts, in
     contract_k1<T, kImgThreads, false>(p, nf, nt, tqs, H1p, sE, sW, t0 > 0, sY);
   }
   __syncthreads();
+  auto scale = [&](int q, int h, int a, int b, int sc) {
+    const T l = applyK ? T(1) / Lhat[2 * (((long long)q * H1 + h) * 4 + sc)] : T(1);
+    return coef * l * (h ? T(2) : T(1)) * (a ? T(2) : T(1)) * (b ? T(2) : T(1));
+  };
+  if constexpr (HERM) {
+    for (int it = threadIdx.x; it < nf * H1 * PC * 2; it += kImgThreads) {   // (c, h, quad, signs)
+      const int m = it & 7, ql = (it >> 3) & ((1 << tqs) - 1), r = it >> (tqs + 3);
+      const int c = r / H1, h = r - c * H1, q = q0 + ql;
+      if (ql >= nq) continue;
+      const int a = fdiv(q, p.dK3h), f[3] = {h, a, q - a * p.k.K3h}, n[3] = {p.b.k1, p.b.k2, p.b.k3};
+      const bool neg[3] = {(m & 1) != 0, (m & 2) != 0, (m & 4) != 0};
+      if (neg[2] && n[2] == 1) continue;
+      int pos[3];
+      bool nyq = false;
+      for (int j = 0; j < 3; ++j) {
+        if (neg[j] && f[j] == 0) nyq = true;
+        pos[j] = !neg[j] ? f[j] : (f[j] == 0 ? n[j] / 2 : n[j] - f[j]);
+      }
+      const V2<T>* y = sY + (c * H1 + h) * PC + 4 * ql;
+      const cplx<T> z = hermitian_value<T>(f, neg, [&](int s1, int s2, int s3) {
+        const int sc = 2 * s3 + s2;
+        T x, u;
+        un2(y[sc], x, u);
+        return scale(q, h, a, f[2], sc) * (s1 ? u : x);
+      });
+      herm[(long long)c * p.b.vol() + ((long long)pos[0] * n[1] + pos[1]) * n[2] + pos[2]] = nyq ? cplx<T>{T(0), T(0)} : z;
+    }
+    return;
+  }
   for (int it = threadIdx.x; it < nf * H1 * PC; it += kImgThreads) {
     const int col = it & (PC - 1), r = it >> (tqs + 2);
     const int c = r / H1, h = r - c * H1, q = q0 + (col >> 2), sc = col & 3;
     if (col >= 4 * nq) continue;
     const int a = fdiv(q, p.dK3h), b = q - a * p.k.K3h;
-    const long long at = ((long long)q * H1 + h) * 4 + sc;
     const bool dead = (a == 0 && (sc & 1)) || (b == 0 && (sc & 2));
-    const T f = coef * (applyK ? T(1) / Lhat[2 * at] : T(1)) * (h ? T(2) : T(1)) * (a ? T(2) : T(1)) * (b ? T(2) : T(1));
+    const T f = scale(q, h, a, b, sc);
     T x, y;
     un2(sY[it], x, y);
-    reinterpret_cast<V2<T>*>(out)[(long long)c * p.k.Kq() * H1 * 4 + at] =
+    reinterpret_cast<V2<T>*>(out)[(long long)c * p.k.Kq() * H1 * 4 + ((long long)q * H1 + h) * 4 + sc] =
         dead ? zero2<T>() : mk2(f * x, h ? f * y : T(0));
   }
 }
@@ -496,8 +562,7 @@ __global__ void k_band_load(const cplx<T>* __restrict__ in, T* __restrict__ out,
   out[idx] = v;
 }
 
-// out(sigma k) = sum over (s1, s2, s3) of prod_j w_j V, w = 1 for a zero frequency,
-// else 1/2 (cosine) or -i sigma / 2 (sine); Nyquist slots are zero
+// out(sigma k) = hermitian_value of the slot's quad; Nyquist slots are zero
 template <typename T>
 __global__ void k_band_store(const T* __restrict__ in, cplx<T>* __restrict__ out, int ncomp, Band bd) {
   const Trig k = trig_of(bd);
@@ -516,29 +581,7 @@ __global__ void k_band_store(const T* __restrict__ in, cplx<T>* __restrict__ out
   cplx<T> z{T(0), T(0)};
   if (!nyq) {
     const T* v = in + (long long)c * k.vol() + ((long long)(f[1] * k.K3h + f[2]) * k.H1 + f[0]) * 8;
-    for (int m = 0; m < 8; ++m) {
-      const int sn[3] = {m & 1, (m >> 1) & 1, (m >> 2) & 1};
-      T w = T(1);
-      int turns = 0;                                       // factors -i
-      bool skip = false;
-      for (int j = 0; j < 3; ++j) {
-        if (f[j] == 0) {
-          if (sn[j]) skip = true;
-          continue;
-        }
-        w *= T(0.5);
-        if (sn[j]) {
-          ++turns;
-          if (neg[j]) w = -w;
-        }
-      }
-      if (skip) continue;
-      const T u = w * v[(2 * sn[2] + sn[1]) * 2 + sn[0]];
-      if (turns == 0) z.x += u;
-      else if (turns == 1) z.y -= u;
-      else if (turns == 2) z.x -= u;
-      else z.y += u;
-    }
+    z = hermitian_value<T>(f, neg, [&](int s1, int s2, int s3) { return v[(2 * s3 + s2) * 2 + s1]; });
   }
   out[idx] = z;
 }
@@ -793,7 +836,7 @@ long long pi_P1_elems(const Plan<T>& p) {
 }
 template <typename T>
 cudaError_t pi_fields(const Plan<T>& p, PiKind kind, const PiField<T>& s, const PiEpi<T>& e, const T* Lhat, T* P1,
-                      cudaStream_t st) {
+                      cudaStream_t st, cplx<T>* herm) {
   const int nf = e.ncomp, ppi = pi_pairs(p), nparts = (p.NT2 + ppi - 1) / ppi;
   cudaError_t rc;
   switch (kind) {
@@ -805,9 +848,17 @@ cudaError_t pi_fields(const Plan<T>& p, PiKind kind, const PiField<T>& s, const 
   if (rc != cudaSuccess) return rc;
   const int tqs = p.k.Kq() >= 2 * kSMs ? 1 : 0, PC = 4 << tqs, H1 = p.k.H1;
   const size_t smem = (size_t)(kChunk * up4(H1) + 3 * kChunk * PC + 3 * H1 * PC) * sizeof(V2<T>);
-  if ((rc = allow_smem<k_pi_band<T>>()) != cudaSuccess) return rc;
-  return launch_chain(k_pi_band<T>, dim3((unsigned)((p.k.Kq() + (1 << tqs) - 1) >> tqs)), kImgThreads, smem, st, p,
-                      (const T*)P1, nf, nparts, tqs, e.coef[0], e.applyK[0], Lhat, e.dst[0]);
+  const dim3 grid((unsigned)((p.k.Kq() + (1 << tqs) - 1) >> tqs));
+  auto launch = [&](auto kern) {
+    return launch_chain(kern, grid, kImgThreads, smem, st, p, (const T*)P1, nf, nparts, tqs, e.coef[0], e.applyK[0],
+                        Lhat, e.dst[0], herm);
+  };
+  if (herm != nullptr) {
+    if ((rc = allow_smem<k_pi_band<T, true>>()) != cudaSuccess) return rc;
+    return launch(k_pi_band<T, true>);
+  }
+  if ((rc = allow_smem<k_pi_band<T, false>>()) != cudaSuccess) return rc;
+  return launch(k_pi_band<T, false>);
 }
 
 template <typename T>
@@ -870,7 +921,7 @@ bool sizes_accepted(const Dims& g, const Band& b, int nper, bool brackets) {
   template cudaError_t iota_fields<T>(const Plan<T>&, const IotaList<T>&, T*, cudaStream_t);                       \
   template long long pi_P1_elems<T>(const Plan<T>&);                                                               \
   template cudaError_t pi_fields<T>(const Plan<T>&, PiKind, const PiField<T>&, const PiEpi<T>&, const T*, T*,      \
-                                    cudaStream_t);                                                                 \
+                                    cudaStream_t, cplx<T>*);                                                       \
   template void band_load<T>(const cplx<T>*, T*, int, const Band&, cudaStream_t);                                  \
   template void band_store<T>(const T*, cplx<T>*, int, const Band&, cudaStream_t);                                 \
   template bool sizes_accepted<T>(const Dims&, const Band&, int, bool);

@@ -47,12 +47,10 @@ void Impl<T>::pi_call(const void* f, int ncomp, void* out) {
     e.grp[0] = 0;
     e.coef[0] = (T)(1.0 / (double)Nvol);
     e.applyK[0] = 0;
-    add_out(e, vout, 0, 1.0, {});
-    cuda(pi_fields<T>(full, PI_FIELD, src, e, Lhat, P1, st), "pi");
     Z* dst = (Z*)out + (long long)c0 * Kuser;
     const bool direct = in_place(dst, (size_t)nc * Kuser * sizeof(Z), sizeof(Z));
-    band_store<T>(vout, direct ? dst : zout, nc, K, st);
-    launches += kPiLaunches + 1;
+    cuda(pi_fields<T>(full, PI_FIELD, src, e, Lhat, P1, st, direct ? dst : zout), "pi");
+    launches += kPiLaunches;
     check_launch("pi");
     if (!direct)
       cuda(cudaMemcpyAsync(dst, zout, (size_t)nc * Kuser * sizeof(Z), cudaMemcpyDefault, st), "copy");

@@ -239,6 +239,7 @@ cudaError_t iota_fields(const Plan<T>& p, const IotaList<T>& d, T* T1, cudaStrea
 //   PI_INCREMENT  c y d_j m                         (its Gauss-Newton increment, y = dm(1))
 //   PI_NEWTON     c (dm d_j m + (m - y) d_j dm)     (the full-Newton increment)
 // d_j: periodic central difference along axis j, taken while the rows are read
+// The result goes to the epilogue's output, or to the Hermitian arrays herm if given.
 enum PiKind { PI_FIELD = 0, PI_RESIDUAL, PI_INCREMENT, PI_NEWTON };
 template <typename T>
 struct PiField {
@@ -248,7 +249,7 @@ struct PiField {
 };
 template <typename T>
 cudaError_t pi_fields(const Plan<T>& p, PiKind kind, const PiField<T>& s, const PiEpi<T>& e, const T* Lhat, T* P1,
-                      cudaStream_t st);
+                      cudaStream_t st, cplx<T>* herm = nullptr);
 // elements of the scratch: T1 of nf fields, P1 of three
 template <typename T>
 long long iota_T1_elems(const Plan<T>& p, int nf);

@@ -1,10 +1,12 @@
 """The reporting calls of the C interface: work split, probe and launch counter."""
 
+import numpy as np
 import pytest
 
+from oracle import bl
 from paper_1807_11560_gb300 import Context, inputs
 
-from helpers import ALPHA, S, SIGMA, torch_dev
+from helpers import ALPHA, S, SIGMA, rel_2, torch_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -63,3 +65,22 @@ def test_probe_times_deformation_evaluations():
         assert work == pytest.approx((2 * Nt + 1) * transforms + (2 * Nt * 21 + 18) * M1 * M2 * M3, rel=1e-12)
         # the classes of the bracket kernels leave them out
         assert _probed(ctx, "cpw", lambda: ctx.gradient(v, torch.empty_like(v)))[1] == 2 * (2 * Nt)
+
+
+@pytest.mark.parametrize("Ns,Ks", [((12, 10, 9), (8, 6, 4)), ((12, 10), (6, 2)), ((40, 40, 40), (4, 40, 36))])
+def test_pi_writes_the_hermitian_array_in_its_two_kernels(Ns, Ks):
+    """The projection's second kernel writes every slot of the caller's array, the zero
+    Nyquist slots among them, without a launch of its own for that."""
+    import torch
+    d = len(Ns)
+    f = np.random.default_rng(5).normal(size=(d,) + Ns).astype(np.float32)
+    with Context(Ns, Ks, ALPHA, S, SIGMA, 1, precision="fp32") as ctx:
+        for out in (np.full((d,) + Ks, np.nan, np.complex64),
+                    torch.full((d,) + Ks, float("nan"), dtype=torch.complex64, device="cuda")):
+            before = ctx.kernel_count
+            ctx.pi(f, d, out)
+            assert ctx.kernel_count - before == 2
+            got = np.asarray(out if isinstance(out, np.ndarray) else out.cpu())
+            assert rel_2(got.astype(np.complex128), bl.pi(f.astype(np.float64), Ks)) < 2e-6
+            for axis, k in enumerate(Ks):
+                assert not np.take(got, k // 2, axis + 1).any()
