@@ -331,23 +331,13 @@ __device__ __forceinline__ T pi_source(const T* __restrict__ fld, const PiField<
   return s.c * (s.dm[at] * dm + (s.m[at] - s.y[at]) * ((s.dm[up] - s.dm[dn]) * h));
 }
 
-// pi of `ppi` row pairs of one x1 plane of one field: the rows folded along x3 into
-// shared memory, x3 -> k3, then x2 -> k2 as a partial plane.  The row loads (six
-// neighbours a point for the terminal fields) and the packed FMAs bind it: 72-80 us for
-// three terminal fields of 160x192x160, band 32^3, where a pass that formed the fields
-// (25 us) and the transform's plane kernels (95 us) ran before.
+// the np row pairs from t0 of plane x1 of field f: folded along x3 into shared memory,
+// x3 -> k3, then x2 -> k2 into (add: onto) the partial plane out
 template <typename T, int KIND>
-__global__ void __launch_bounds__(kImgThreads)
-k_pi_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ PiField<T> src, int ppi, T* __restrict__ P1) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  V2<T>* sm = reinterpret_cast<V2<T>*>(smraw);
-  const int f = blockIdx.y, x1 = blockIdx.z, t0 = blockIdx.x * ppi, np = min(ppi, p.NT2 - t0);
-  const PlaneShape<T> s = plane_shape(p, 0, 1, ppi, 1);
+__device__ __forceinline__ void pi_plane_part(const Plan<T>& p, const PiField<T>& src, const PlaneShape<T>& s, int ppi,
+                                              int f, int x1, int t0, int np, V2<T>* sm, T* out, bool add) {
   const int NT3 = p.NT3, NT3e = p.NT3e, G2 = p.g.n2, G3 = p.g.n3;
   V2<T>*Z = sm + s.off_s, *sP = sm + s.off_p;
-  pdl_trigger();
-  plane_tables<T, kImgThreads, 1>(p, s, t0, np, false, true, sm);
-  pdl_wait();
   const T* fld = src.f[f];
 #pragma unroll 4
   for (int it = threadIdx.x; it < 2 * np * NT3; it += kImgThreads) {
@@ -363,8 +353,45 @@ k_pi_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ PiField<T>
   __syncthreads();
   rows_to_k3<T, kImgThreads, 1, 1>(p, sP, t0, ppi, np, sm + s.off_3b, Z);
   __syncthreads();
+  band_from_rows<T, kImgThreads, 1, 2>(p, Z, ppi, np, sm + s.off_2b, out, add);
+}
+
+// pi of `ppi` row pairs of one x1 plane of one field.  The row loads (six
+// neighbours a point for the terminal fields) and the packed FMAs bind it: 72-80 us for
+// three terminal fields of 160x192x160, band 32^3, where a pass that formed the fields
+// (25 us) and the transform's plane kernels (95 us) ran before.
+template <typename T, int KIND>
+__global__ void __launch_bounds__(kImgThreads)
+k_pi_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ PiField<T> src, int ppi, T* __restrict__ P1) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  V2<T>* sm = reinterpret_cast<V2<T>*>(smraw);
+  const int f = blockIdx.y, x1 = blockIdx.z, t0 = blockIdx.x * ppi, np = min(ppi, p.NT2 - t0);
+  const PlaneShape<T> s = plane_shape(p, 0, 1, ppi, 1);
+  pdl_trigger();
+  plane_tables<T, kImgThreads, 1>(p, s, t0, np, false, true, sm);
+  pdl_wait();
   T* out = P1 + (((long long)x1 * gridDim.x + blockIdx.x) * gridDim.y + f) * p.k.Kq() * 4;
-  band_from_rows<T, kImgThreads, 1, 2>(p, Z, ppi, np, sm + s.off_2b, out);
+  pi_plane_part<T, KIND>(p, src, s, ppi, f, x1, t0, np, sm, out, false);
+}
+// the same for `reps` times ppi row pairs one after another, where a partial plane of each
+// would take too much scratch (pi_split)
+template <typename T, int KIND>
+__global__ void __launch_bounds__(kImgThreads)
+k_pi_plane_seq(const __grid_constant__ Plan<T> p, const __grid_constant__ PiField<T> src, int ppi, int reps,
+               T* __restrict__ P1) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  V2<T>* sm = reinterpret_cast<V2<T>*>(smraw);
+  const int f = blockIdx.y, x1 = blockIdx.z, first = blockIdx.x * reps * ppi, end = min(first + reps * ppi, p.NT2);
+  const PlaneShape<T> s = plane_shape(p, 0, 1, ppi, 1);
+  T* out = P1 + (((long long)x1 * gridDim.x + blockIdx.x) * gridDim.y + f) * p.k.Kq() * 4;
+  pdl_trigger();
+  pdl_wait();
+  for (int t0 = first; t0 < end; t0 += ppi) {
+    const int np = min(ppi, end - t0);
+    if (t0 > first) __syncthreads();
+    plane_tables<T, kImgThreads, 1>(p, s, t0, np, false, true, sm);
+    pi_plane_part<T, KIND>(p, src, s, ppi, f, x1, t0, np, sm, out, t0 > first);
+  }
 }
 
 // the two plane steps of a 2D image: one output per thread.  k_pi_plane_flat takes part of
@@ -616,17 +643,36 @@ int iota_pairs(const Plan<T>& p) {
   while (most > kIotaPT && plane_shape(p, kIotaGroup, 0, most, kIotaPT).smem > (size_t)96 * 1024) most -= kIotaPT;
   return even_pairs(p.NT2, most, kIotaPT);
 }
+// Most elements of the image-grid scratch: what a transform that takes axis 1 last would
+// hold of 33 fields, or 2^24; at least one partial plane and one velocity.  The planes of
+// the kernels here grow with the first axis, so a long one with a thin band would take
+// many times that (19020 x 2965 x 21, band 2 x 416 x 18, one time step: 72 GB for 33 fields
+// at once and a partial plane per item, beside 165 GB of the rest; 1.7 GB so).
 template <typename T>
-int pi_pairs(const Plan<T>& p) {
+long long image_scratch(const Plan<T>& p) {
+  return std::max(33LL * p.b.k1 * p.g.n2 * p.g.n3, 1LL << 24);
+}
+struct PiSplit {
+  int ppi, reps, nparts;   // row pairs at once, times one after another, partial planes
+};
+template <typename T>
+PiSplit pi_split(const Plan<T>& p) {
+  PiSplit s{p.NT2, 1, 1};
   if (p.flat) {
     // a thread sums the points of an item in turn: parts of 64 row pairs while a wave has
     // room (a pi call of a 64 x 1024 image, band 8 x 512: 88 us whole, 57 in parts)
     const int parts = std::max(1, std::min((p.NT2 + 63) / 64, 4 * kSMs / p.g.n1));
-    return (p.NT2 + parts - 1) / parts;
+    s.ppi = (p.NT2 + parts - 1) / parts;
+  } else {
+    int most = std::max(1, 2 * kImgThreads / p.K3e);
+    while (most > 1 && plane_shape(p, 0, 1, most, 1).smem > (size_t)96 * 1024) --most;
+    s.ppi = even_pairs(p.NT2, most, 1);
+    const int parts = (p.NT2 + s.ppi - 1) / s.ppi;
+    const long long fit = std::max(1LL, image_scratch(p) / ((long long)p.g.n1 * 3 * p.k.Kq() * 4));
+    if (parts > fit) s.reps = (int)((parts + fit - 1) / fit);
   }
-  int most = std::max(1, 2 * kImgThreads / p.K3e);
-  while (most > 1 && plane_shape(p, 0, 1, most, 1).smem > (size_t)96 * 1024) --most;
-  return even_pairs(p.NT2, most, 1);
+  s.nparts = (p.NT2 + s.ppi * s.reps - 1) / (s.ppi * s.reps);
+  return s;
 }
 
 template <typename T, int MODE, int PT>
@@ -711,14 +757,17 @@ cudaError_t launch_iota_plane_even(const Plan<T>& p, const IotaList<T>& d, const
 
 template <typename T, int KIND>
 cudaError_t launch_pi_plane(const Plan<T>& p, const PiField<T>& s, int nf, T* P1, cudaStream_t st) {
-  const int ppi = pi_pairs(p);
-  if (p.flat)
-    return launch_chain(k_pi_plane_flat<T, KIND>, dim3((unsigned)((p.NT2 + ppi - 1) / ppi), (unsigned)nf, (unsigned)p.g.n1),
-                        kImgThreads, 0, st, p, s, ppi, P1);
-  cudaError_t e = allow_smem<k_pi_plane<T, KIND>>();
-  if (e != cudaSuccess) return e;
-  return launch_chain(k_pi_plane<T, KIND>, dim3((unsigned)((p.NT2 + ppi - 1) / ppi), (unsigned)nf, (unsigned)p.g.n1),
-                      kImgThreads, plane_shape(p, 0, 1, ppi, 1).smem, st, p, s, ppi, P1);
+  const PiSplit w = pi_split(p);
+  const dim3 grid((unsigned)w.nparts, (unsigned)nf, (unsigned)p.g.n1);
+  if (p.flat) return launch_chain(k_pi_plane_flat<T, KIND>, grid, kImgThreads, 0, st, p, s, w.ppi, P1);
+  const size_t smem = plane_shape(p, 0, 1, w.ppi, 1).smem;
+  cudaError_t e;
+  if (w.reps > 1) {
+    if ((e = allow_smem<k_pi_plane_seq<T, KIND>>()) != cudaSuccess) return e;
+    return launch_chain(k_pi_plane_seq<T, KIND>, grid, kImgThreads, smem, st, p, s, w.ppi, w.reps, P1);
+  }
+  if ((e = allow_smem<k_pi_plane<T, KIND>>()) != cudaSuccess) return e;
+  return launch_chain(k_pi_plane<T, KIND>, grid, kImgThreads, smem, st, p, s, w.ppi, P1);
 }
 
 }  // namespace
@@ -803,6 +852,12 @@ long long iota_T1_elems(const Plan<T>& p, int nf) {
   return (long long)p.g.n1 * nf * p.k.Kq() * 4;
 }
 template <typename T>
+int iota_fields_at_once(const Plan<T>& p, int most) {
+  int nf = std::min(most, 33);
+  while (nf > 3 && iota_T1_elems(p, nf) > image_scratch(p)) nf -= 3;
+  return nf;
+}
+template <typename T>
 cudaError_t iota_fields(const Plan<T>& p, const IotaList<T>& d, T* T1, cudaStream_t st) {
   const int tqs = p.k.Kq() >= 4 ? 2 : 0;
   const size_t smem = (size_t)(up2(kIotaBandGroup * p.k.H1 * (4 << tqs)) + p.k.H1 * kChunk) * sizeof(V2<T>);
@@ -831,13 +886,12 @@ cudaError_t iota_fields(const Plan<T>& p, const IotaList<T>& d, T* T1, cudaStrea
 
 template <typename T>
 long long pi_P1_elems(const Plan<T>& p) {
-  const int ppi = pi_pairs(p);
-  return (long long)p.g.n1 * ((p.NT2 + ppi - 1) / ppi) * 3 * p.k.Kq() * 4;
+  return (long long)p.g.n1 * pi_split(p).nparts * 3 * p.k.Kq() * 4;
 }
 template <typename T>
 cudaError_t pi_fields(const Plan<T>& p, PiKind kind, const PiField<T>& s, const PiEpi<T>& e, const T* Lhat, T* P1,
                       cudaStream_t st, cplx<T>* herm) {
-  const int nf = e.ncomp, ppi = pi_pairs(p), nparts = (p.NT2 + ppi - 1) / ppi;
+  const int nf = e.ncomp, nparts = pi_split(p).nparts;
   cudaError_t rc;
   switch (kind) {
     case PI_FIELD: rc = launch_pi_plane<T, PI_FIELD>(p, s, nf, P1, st); break;
@@ -918,6 +972,7 @@ bool sizes_accepted(const Dims& g, const Band& b, int nper, bool brackets) {
   template long long eval_T1_elems<T>(const Plan<T>&);                                                             \
   template long long eval_P1_elems<T>(const Plan<T>&);                                                             \
   template long long iota_T1_elems<T>(const Plan<T>&, int);                                                        \
+  template int iota_fields_at_once<T>(const Plan<T>&, int);                                                        \
   template cudaError_t iota_fields<T>(const Plan<T>&, const IotaList<T>&, T*, cudaStream_t);                       \
   template long long pi_P1_elems<T>(const Plan<T>&);                                                               \
   template cudaError_t pi_fields<T>(const Plan<T>&, PiKind, const PiField<T>&, const PiEpi<T>&, const T*, T*,      \

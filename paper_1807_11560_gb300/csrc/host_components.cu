@@ -49,7 +49,7 @@ void Impl<T>::pi_call(const void* f, int ncomp, void* out) {
     e.applyK[0] = 0;
     Z* dst = (Z*)out + (long long)c0 * Kuser;
     const bool direct = in_place(dst, (size_t)nc * Kuser * sizeof(Z), sizeof(Z));
-    cuda(pi_fields<T>(full, PI_FIELD, src, e, Lhat, P1, st, direct ? dst : zout), "pi");
+    cuda(pi_fields<T>(full, PI_FIELD, src, e, Lhat, T1, st, direct ? dst : zout), "pi");
     launches += kPiLaunches;
     check_launch("pi");
     if (!direct)

@@ -126,8 +126,9 @@ void Impl<T>::create(int nd, const int* grid, const int* band, double a, int s_,
 
   alloc(I0, (size_t)Nvol);
   alloc(I1, (size_t)Nvol);
-  alloc(T1, (size_t)std::max(iota_T1_elems<T>(full, 33), eval_T1_elems<T>(pad)));
-  alloc(P1, (size_t)std::max(pi_P1_elems<T>(full), eval_P1_elems<T>(pad)));
+  iota_nf = iota_fields_at_once<T>(full, opts.recompute || deform() ? 3 : 3 * (Nt + 1));
+  alloc(T1, (size_t)std::max({iota_T1_elems<T>(full, iota_nf), pi_P1_elems<T>(full), eval_T1_elems<T>(pad)}));
+  alloc(P1, (size_t)eval_P1_elems<T>(pad));
   alloc(zin, (size_t)3 * Kuser);
   alloc(zout, (size_t)3 * Kuser);
   for (C** b : {&k1, &aU, &aW, &Ut, &Wt, &U, &W, &vout, &gbuf, &px, &pr,

@@ -58,8 +58,9 @@ void Impl<T>::run_sweep(PwMode mode, const EvalDesc<T>* ev, int nev) {
 
 template <typename T>
 void Impl<T>::to_grid(const C* hist, int count, T* grid) {
-  for (int v0 = 0; v0 < count; v0 += 11) {
-    const int nv = std::min(11, count - v0);
+  const int group = iota_nf / 3;
+  for (int v0 = 0; v0 < count; v0 += group) {
+    const int nv = std::min(group, count - v0);
     IotaList<T> d{};
     d.nf = 3 * nv;
     for (int v = 0; v < nv; ++v)
@@ -83,7 +84,7 @@ void Impl<T>::project(PiKind kind, const PiField<T>& f, C* out, double coef, boo
   e.applyK[0] = applyK ? 1 : 0;
   add_out(e, out, 0, 1.0, {});
   pb(PR_PI_FULL);
-  cuda(pi_fields<T>(full, kind, f, e, Lhat, P1, st), "projection");
+  cuda(pi_fields<T>(full, kind, f, e, Lhat, T1, st), "projection");
   pe(PR_PI_FULL, grid_flops(N, 3));
   launches += kPiLaunches;
 }

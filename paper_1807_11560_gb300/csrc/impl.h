@@ -87,7 +87,9 @@ struct Impl {
   T *I0 = nullptr, *I1 = nullptr;
   State<T> lin, trial;
   bool have_images = false, have_lin = false, have_dm1 = false;
-  T *T1 = nullptr, *P1 = nullptr;     // transform scratch: plane fields, projected planes
+  T* T1 = nullptr;                    // transform scratch: plane fields; projected image planes
+  T* P1 = nullptr;                    // projected planes of an evaluation
+  int iota_nf = 33;                   // fields of one image-grid transform (T1 is sized for)
   Z *zin = nullptr, *zout = nullptr;  // [3][Kuser] staging of the caller's arrays
   C *k1 = nullptr, *aU = nullptr, *aW = nullptr, *Ut = nullptr, *Wt = nullptr, *U = nullptr,
     *W = nullptr, *vout = nullptr, *gbuf = nullptr;

@@ -253,6 +253,9 @@ cudaError_t pi_fields(const Plan<T>& p, PiKind kind, const PiField<T>& s, const 
 // elements of the scratch: T1 of nf fields, P1 of three
 template <typename T>
 long long iota_T1_elems(const Plan<T>& p, int nf);
+// fields of one iota_fields call (of at most `most`, in threes) that keep the scratch small
+template <typename T>
+int iota_fields_at_once(const Plan<T>& p, int most);
 template <typename T>
 long long pi_P1_elems(const Plan<T>& p);
 constexpr int kIotaLaunches = 2, kPiLaunches = 2, kEvalLaunches = 2;

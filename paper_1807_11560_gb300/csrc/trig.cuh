@@ -655,11 +655,11 @@ __device__ __forceinline__ void rows_from_band(const Plan<T>& p, const T* V, int
 }
 
 // x2 -> k2 of the folded rows Z [NO][ppc][K3e][2] (the pairs over s2 of s3 = 0 and
-// of s3 = 1) over np row pairs into the partial plane out [NO][Kq][4], AG
+// of s3 = 1) over np row pairs into (add: onto) the partial plane out [NO][Kq][4], AG
 // frequencies per thread
 template <typename T, int NT, int NO, int AG>
 __device__ __forceinline__ void band_from_rows(const Plan<T>& p, const V2<T>* Z, int ppc, int np, const V2<T>* tw2b,
-                                               T* out) {
+                                               T* out, bool add = false) {
   const int K2h = p.k.K2h, K2p = up8(K2h), K3h = p.k.K3h, K3e = p.K3e;
   const long long Kq = p.k.Kq();
   const int ng = (K2h + AG - 1) / AG;
@@ -690,7 +690,14 @@ __device__ __forceinline__ void band_from_rows(const Plan<T>& p, const V2<T>* Z,
     T* d = out + ((long long)o * Kq + (long long)(g * AG) * K3h + b) * 4;
 #pragma unroll
     for (int k = 0; k < AG; ++k)
-      if (g * AG + k < K2h) stq(d + k * K3h * 4, Quad<T>{c[k], s[k]});
+      if (g * AG + k < K2h) {
+        if (add) {                                         // onto this thread's own sums
+          const Quad<T> q = ldq(d + k * K3h * 4);
+          c[k] = sum2(q.c, c[k]);
+          s[k] = sum2(q.s, s[k]);
+        }
+        stq(d + k * K3h * 4, Quad<T>{c[k], s[k]});
+      }
   }
 }
 
