@@ -22,7 +22,6 @@ using namespace dev;
 constexpr int kImgThreads = 256;
 constexpr int kIotaGroup = 3;     // fields per image-plane item (one velocity)
 constexpr int kIotaBandGroup = 6; // fields per k1 -> x1 item
-constexpr int kSMs = 152;         // sizing only: fixed, so that sums never depend on the device
 
 // raises a kernel's dynamic shared memory limit once per device
 template <auto Kernel>
@@ -76,8 +75,9 @@ k_band(const __grid_constant__ BandArgs<T> a) {
   // 2D bands of more items than SMs (one to an SM) let the plane phase start as they end:
   // before, its small items would fill the SMs of the first wave and leave the rest idle
   if (!FLAT || gridDim.x <= kSMs) pdl_trigger();
-  band_item<T, MODE, kPhaseThreads, FLAT>(a.p, a.tqs, a.prev ? &a.e : nullptr, a.nparts, a.P1, a.A, a.B, a.T1, a.Lhat,
-                                         blockIdx.x, reinterpret_cast<V2<T>*>(smraw));
+  band_item<T, MODE, kPhaseThreads, FLAT, MINB == 1 ? kSplit<T> : 1>(
+      a.p, a.tqs, a.prev ? &a.e : nullptr, a.nparts, a.P1, a.A, a.B, a.T1, a.Lhat, blockIdx.x,
+      reinterpret_cast<V2<T>*>(smraw));
 }
 
 // Plane phase: bound by packed-FMA issue and shared-memory reads, about one pair read
@@ -351,9 +351,9 @@ __device__ __forceinline__ void pi_plane_part(const Plan<T>& p, const PiField<T>
     if (t == NT3 - 1 && NT3e > NT3) o[1] = zero2<T>();
   }
   __syncthreads();
-  rows_to_k3<T, kImgThreads, 1, 1>(p, sP, t0, ppi, np, sm + s.off_3b, Z);
+  rows_to_k3<T, kImgThreads, 1, 1, kSplit<T>>(p, sP, t0, ppi, np, sm + s.off_3b, Z);
   __syncthreads();
-  band_from_rows<T, kImgThreads, 1, 2>(p, Z, ppi, np, sm + s.off_2b, out, add);
+  band_from_rows<T, kImgThreads, 1, 2, kSplit<T>>(p, Z, ppi, np, sm + s.off_2b, out, add);
 }
 
 // pi of `ppi` row pairs of one x1 plane of one field.  The row loads (six
@@ -506,7 +506,7 @@ k_pi_band(const __grid_constant__ Plan<T> p, const T* P1, int nf, int nparts, in
     fold_planes<T, kImgThreads>(p, P1, nf, nparts, q0, nq, tqs, t0, nt, FastDiv{nt > 1 ? 0xffffffffu / nt + 1u : 0u},
                                 sE);
     __syncthreads();
-    contract_k1<T, kImgThreads, false>(p, nf, nt, tqs, H1p, sE, sW, t0 > 0, sY);
+    contract_k1<T, kImgThreads, false, sizeof(T) == 4 ? 4 : 1>(p, nf, nt, tqs, H1p, sE, sW, t0 > 0, sY);
   }
   __syncthreads();
   auto scale = [&](int q, int h, int a, int b, int sc) {
@@ -728,7 +728,7 @@ cudaError_t launch_band(const Plan<T>& p, const PiEpi<T>* prev, const T* P1, con
   // more items than SMs: two to an SM (band 64^3: 166 us per evaluation against 182
   // with one, band 40^3: 36.4 / 39.6); below that the registers are worth more (32^3:
   // 21.6 / 19.5)
-  if (sizeof(T) == 4 && (p.k.Kq() >> p.geom[MODE].tqs) > kSMs)
+  if (shared_sms(p, p.geom[MODE].tqs))
     return launch_band_as<T, MODE, false, sizeof(T) == 4 ? 2 : 1>(p, prev, P1, A, B, T1, Lhat, st);
   return launch_band_as<T, MODE, false, 1>(p, prev, P1, A, B, T1, Lhat, st);
 }

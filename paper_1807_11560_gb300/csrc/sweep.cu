@@ -61,7 +61,8 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned& target, 
   return __syncthreads_and(ok) != 0;
 }
 
-template <typename T, int MODE, int PT>
+// NS: the band phase's accumulators, as its kernel launched by itself has them
+template <typename T, int MODE, int PT, int NS>
 __global__ void __launch_bounds__(kPhaseThreads, 1)
 k_sweep(const __grid_constant__ SweepArgs<T> a) {
   constexpr int NT = kPhaseThreads;
@@ -90,8 +91,8 @@ k_sweep(const __grid_constant__ SweepArgs<T> a) {
     const PiEpi<T>* e = ev > 0 && prev->epi.nout > 0 ? &prev->epi : nullptr;
     if (more || e != nullptr) {
       for (int i = blockIdx.x; i < n_band; i += gridDim.x) {
-        band_item<T, MODE, NT, PT == 0>(p, a.g.tqs, e, a.g.nparts, a.P1, more ? cur->A : nullptr, more ? cur->B : nullptr, a.T1,
-                               a.Lhat, i, sm);
+        band_item<T, MODE, NT, PT == 0, NS>(p, a.g.tqs, e, a.g.nparts, a.P1, more ? cur->A : nullptr,
+                                             more ? cur->B : nullptr, a.T1, a.Lhat, i, sm);
         __syncthreads();
       }
     }
@@ -107,9 +108,9 @@ k_sweep(const __grid_constant__ SweepArgs<T> a) {
   }
 }
 
-template <typename T, int MODE, int PT>
-cudaError_t launch_pt(const SweepArgs<T>& a, size_t smem, cudaStream_t st, int max_ctas) {
-  auto kern = k_sweep<T, MODE, PT>;
+template <typename T, int MODE, int PT, int NS>
+cudaError_t launch_ns(const SweepArgs<T>& a, size_t smem, cudaStream_t st, int max_ctas) {
+  auto kern = k_sweep<T, MODE, PT, NS>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0, dev_id = 0, sms = 0;
@@ -130,6 +131,13 @@ cudaError_t launch_pt(const SweepArgs<T>& a, size_t smem, cudaStream_t st, int m
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+template <typename T, int MODE, int PT>
+cudaError_t launch_pt(const SweepArgs<T>& a, size_t smem, cudaStream_t st, int max_ctas) {
+  if constexpr (PT != 0 && kSplit<T> != 1)
+    if (shared_sms(a.p, a.g.tqs)) return launch_ns<T, MODE, PT, 1>(a, smem, st, max_ctas);
+  return launch_ns<T, MODE, PT, kSplit<T>>(a, smem, st, max_ctas);
 }
 
 template <typename T, int MODE>

@@ -35,6 +35,14 @@ namespace dev {
 
 constexpr double kTwoPi = 6.283185307179586476925286766559;
 constexpr int kMaxSmem = 224 * 1024;
+// FP32 sums back to the band are split over interleaved accumulators (four in k_pi_band): a
+// sum of like signs (an image, the lowest frequencies) loses about the square root of a
+// third of its length in roundings, and half of that in two halves.  Relative errors at
+// 64^3, band 16^3: projection of images 1.24e-7 to 7.7e-8, ad~^dagger 1.49e-7 to 1.40e-7
+// (complex half-spectrum sums: 7.4e-8 and 1.35e-7).  It costs no time, the chains being
+// shorter; sums in blocks of eight, added to a total, cost 1-2% of a product.
+template <typename T> constexpr int kSplit = sizeof(T) == 4 ? 2 : 1;
+constexpr int kSMs = 152;   // sizing only: fixed, so that sums never depend on the device
 // Threads of the two phases.  The contractions are bound by issue slots and by the
 // register write-back of shared-memory reads (one pair per lane costs two packed
 // FMAs), so a thread takes a register tile of several sums.
@@ -164,6 +172,19 @@ __host__ __device__ inline BandShape<T> band_shape(const Plan<T>& p, int tq, int
   s.off_y = s.off_e + (e > g ? e : g) * PC;
   s.smem = (size_t)up2(s.off_y + NO * H1 * PC) * sizeof(V2<T>);
   return s;
+}
+
+// N sums of NS accumulators each (acc [NS][N]) into the first
+template <typename T, int NS, int N>
+__device__ __forceinline__ void add_sums(V2<T>* acc) {
+  if constexpr (NS == 4) {
+#pragma unroll
+    for (int i = 0; i < 2 * N; ++i) acc[i] = sum2(acc[i], acc[2 * N + i]);
+  }
+  if constexpr (NS > 1) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) acc[i] = sum2(acc[i], acc[N + i]);
+  }
 }
 
 template <typename T>
@@ -319,8 +340,8 @@ __device__ __forceinline__ void fold_planes(const Plan<T>& p, const T* P1, int N
 }
 
 // x1 -> k1 of the folded inputs sE [NO][nt][PC] with the table sW [nt][H1p], into
-// (add: onto) sY [NO][H1][PC]
-template <typename T, int NT, bool FLAT>
+// (add: onto) sY [NO][H1][PC]; NS accumulators (kSplit)
+template <typename T, int NT, bool FLAT, int NS>
 __device__ __forceinline__ void contract_k1(const Plan<T>& p, int NO, int nt, int tqs, int H1p, const V2<T>* sE,
                                             const V2<T>* sW, bool add, V2<T>* sY) {
   constexpr int HG = BandTile<T>::HG, CP = BandTile<T>::CP;
@@ -333,13 +354,10 @@ __device__ __forceinline__ void contract_k1(const Plan<T>& p, int NO, int nt, in
     const int o = HG == 1 ? fdiv(r, p.dH1) : fdiv(r, p.dH1g), g = r - o * ng;
     const V2<T>* v = sE + o * nt * PC + col;
     const V2<T>* w = sW + g * HG;
-    V2<T> acc[HG][CP];
+    V2<T> acc[NS][HG][CP];
 #pragma unroll
-    for (int i = 0; i < HG; ++i)
-#pragma unroll
-      for (int c = 0; c < CP; ++c) acc[i][c] = zero2<T>();
-#pragma unroll 4
-    for (int t = 0; t < nt; ++t) {
+    for (int i = 0; i < NS * HG * CP; ++i) acc[i / (HG * CP)][i / CP % HG][i % CP] = zero2<T>();
+    auto term = [&](int t, V2<T>(&sum)[HG][CP]) {
       V2<T> u[2];
       if (CP == 2) ld2(v + t * PC, u[0], u[1]);
       else u[0] = v[t * PC];
@@ -350,18 +368,39 @@ __device__ __forceinline__ void contract_k1(const Plan<T>& p, int NO, int nt, in
         else w0 = w[t * H1p];
 #pragma unroll
         for (int c = 0; c < CP; ++c) {
-          acc[i][c] = fma2(u[c], w0, acc[i][c]);
-          if (HG > 1) acc[i + (HG > 1)][c] = fma2(u[c], w1, acc[i + (HG > 1)][c]);
+          sum[i][c] = fma2(u[c], w0, sum[i][c]);
+          if (HG > 1) sum[i + (HG > 1)][c] = fma2(u[c], w1, sum[i + (HG > 1)][c]);
         }
       }
+    };
+    if constexpr (NS == 1) {
+#pragma unroll 4
+      for (int t = 0; t < nt; ++t) term(t, acc[0]);
+    } else if constexpr (NS == 2) {
+      int t = 0;
+#pragma unroll 2
+      for (; t + 2 <= nt; t += 2) {
+        term(t, acc[0]);
+        term(t + 1, acc[1]);
+      }
+      if (t < nt) term(t, acc[0]);
+    } else {
+      int t = 0;
+#pragma unroll 1
+      for (; t + NS <= nt; t += NS)
+#pragma unroll
+        for (int k = 0; k < NS; ++k) term(t + k, acc[k]);
+#pragma unroll 1
+      for (; t < nt; ++t) term(t, acc[0]);
     }
+    add_sums<T, NS, HG * CP>(&acc[0][0][0]);
 #pragma unroll
     for (int i = 0; i < HG; ++i) {
       const int h = g * HG + i;
       if (h >= H1) break;
       V2<T>* y = sY + (o * H1 + h) * PC + col;
 #pragma unroll
-      for (int c = 0; c < CP; ++c) y[c] = add ? sum2(y[c], acc[i][c]) : acc[i][c];
+      for (int c = 0; c < CP; ++c) y[c] = add ? sum2(y[c], acc[0][i][c]) : acc[0][i][c];
     }
   }
 }
@@ -436,9 +475,16 @@ __device__ __forceinline__ void band_to_planes(const Plan<T>& p, const V2<T>* sG
   }
 }
 
+// whether band-phase items of 2^tqs quads share an SM (FP32: more items than SMs)
+// and then have the registers for one accumulator (two spill: band 64^3 0.7% slower)
+template <typename T>
+__host__ __device__ __forceinline__ bool shared_sms(const Plan<T>& p, int tqs) {
+  return sizeof(T) == 4 && !p.flat && (p.k.Kq() >> tqs) > kSMs;
+}
+
 // one band-phase item of mode MODE: e != nullptr, the previous evaluation's
 // projection and epilogue; A != nullptr, the fields of the next evaluation
-template <typename T, int MODE, int NT, bool FLAT>
+template <typename T, int MODE, int NT, bool FLAT, int NS>
 __device__ __forceinline__ void band_item(const Plan<T>& p, int tqs, const PiEpi<T>* e, int nparts, const T* P1,
                                           const T* A, const T* B, T* T1, const T* __restrict__ Lhat, int item,
                                           V2<T>* sm) {
@@ -480,7 +526,7 @@ __device__ __forceinline__ void band_item(const Plan<T>& p, int tqs, const PiEpi
     }
     fold_planes<T, NT>(p, P1, NO, nparts, q0, nq, tqs, 0, p.NT1, p.dNT1, sE);
     __syncthreads();
-    contract_k1<T, NT, FLAT>(p, NO, p.NT1, tqs, s.H1p, sE, sB, false, sY);
+    contract_k1<T, NT, FLAT, NS>(p, NO, p.NT1, tqs, s.H1p, sE, sB, false, sY);
     __syncthreads();
     const bool dead2 = (a == 0 && (sc & 1)) || (b == 0 && (sc & 2));
     const T fac = dead2 ? T(0) : (h ? T(2) : T(1)) * (a ? T(2) : T(1)) * (b ? T(2) : T(1));
@@ -657,7 +703,7 @@ __device__ __forceinline__ void rows_from_band(const Plan<T>& p, const T* V, int
 // x2 -> k2 of the folded rows Z [NO][ppc][K3e][2] (the pairs over s2 of s3 = 0 and
 // of s3 = 1) over np row pairs into (add: onto) the partial plane out [NO][Kq][4], AG
 // frequencies per thread
-template <typename T, int NT, int NO, int AG>
+template <typename T, int NT, int NO, int AG, int NS>
 __device__ __forceinline__ void band_from_rows(const Plan<T>& p, const V2<T>* Z, int ppc, int np, const V2<T>* tw2b,
                                                T* out, bool add = false) {
   const int K2h = p.k.K2h, K2p = up8(K2h), K3h = p.k.K3h, K3e = p.K3e;
@@ -671,8 +717,7 @@ __device__ __forceinline__ void band_from_rows(const Plan<T>& p, const V2<T>* Z,
     V2<T> c[AG], s[AG];
 #pragma unroll
     for (int i = 0; i < AG; ++i) c[i] = s[i] = zero2<T>();
-#pragma unroll 3
-    for (int i = 0; i < np; ++i) {
+    auto row = [&](V2<T>* c, V2<T>* s) {
       V2<T> qc, qs;
       ld2(z, qc, qs);
       z += 2 * K3e;
@@ -686,6 +731,25 @@ __device__ __forceinline__ void band_from_rows(const Plan<T>& p, const V2<T>* Z,
         s[k + 1] = fma2(qs, w1, s[k + 1]);
       }
       w += K2p;
+    };
+    if constexpr (NS == 1) {
+#pragma unroll 3
+      for (int i = 0; i < np; ++i) row(c, s);
+    } else {
+      V2<T> c2[AG], s2[AG];
+#pragma unroll
+      for (int k = 0; k < AG; ++k) c2[k] = s2[k] = zero2<T>();
+#pragma unroll 2
+      for (int i = 0; i < np / 2; ++i) {
+        row(c, s);
+        row(c2, s2);
+      }
+      if (np & 1) row(c, s);
+#pragma unroll
+      for (int k = 0; k < AG; ++k) {
+        c[k] = sum2(c[k], c2[k]);
+        s[k] = sum2(s[k], s2[k]);
+      }
     }
     T* d = out + ((long long)o * Kq + (long long)(g * AG) * K3h + b) * 4;
 #pragma unroll
@@ -704,7 +768,7 @@ __device__ __forceinline__ void band_from_rows(const Plan<T>& p, const V2<T>* Z,
 // x3 -> k3 of the folded points sP [NO][R][NT3e] (table tw3b [NT3e][K3e]), then the
 // fold of each row pair: Z [NO][ppc][K3e][2].  A thread takes both rows of a pair,
 // two frequencies and OG fields; a self-paired x2 has one row only.
-template <typename T, int NT, int NO, int OG>
+template <typename T, int NT, int NO, int OG, int NS>
 __device__ __forceinline__ void rows_to_k3(const Plan<T>& p, const V2<T>* sP, int t0, int ppc, int np,
                                            const V2<T>* tw3b, V2<T>* Z) {
   constexpr int NG = (NO + OG - 1) / OG;
@@ -716,9 +780,9 @@ __device__ __forceinline__ void rows_to_k3(const Plan<T>& p, const V2<T>* sP, in
     const V2<T>* v = sP + (g * OG * R + 2 * i) * NT3e;
     const V2<T>* w = tw3b + b;
     const int second = two ? NT3e : 0;                     // (a missing row repeats the first)
-    V2<T> acc[OG][2][2];
+    V2<T> acc[NS][OG][2][2];
 #pragma unroll
-    for (int o = 0; o < OG; ++o) acc[o][0][0] = acc[o][0][1] = acc[o][1][0] = acc[o][1][1] = zero2<T>();
+    for (int o = 0; o < NS * OG * 4; ++o) acc[o / (OG * 4)][o / 4 % OG][o / 2 % 2][o % 2] = zero2<T>();
     for (int t3 = 0; t3 < NT3e; t3 += 2) {
       V2<T> w00, w01, w10, w11;
       ld2(w, w00, w01);
@@ -731,11 +795,14 @@ __device__ __forceinline__ void rows_to_k3(const Plan<T>& p, const V2<T>* sP, in
         for (int k = 0; k < 2; ++k) {
           V2<T> a0, a1;
           ld2(v + o * R * NT3e + k * second + t3, a0, a1);
-          acc[o][k][0] = fma2(a1, w10, fma2(a0, w00, acc[o][k][0]));
-          acc[o][k][1] = fma2(a1, w11, fma2(a0, w01, acc[o][k][1]));
+          acc[0][o][k][0] = fma2(a0, w00, acc[0][o][k][0]);
+          acc[0][o][k][1] = fma2(a0, w01, acc[0][o][k][1]);
+          acc[NS - 1][o][k][0] = fma2(a1, w10, acc[NS - 1][o][k][0]);
+          acc[NS - 1][o][k][1] = fma2(a1, w11, acc[NS - 1][o][k][1]);
         }
       }
     }
+    add_sums<T, NS, OG * 4>(&acc[0][0][0][0]);
 #pragma unroll
     for (int o = 0; o < OG; ++o) {
       if (NO % OG != 0 && g * OG + o >= NO) break;
@@ -743,8 +810,8 @@ __device__ __forceinline__ void rows_to_k3(const Plan<T>& p, const V2<T>* sP, in
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         T c1, s1, c2, s2;
-        un2(acc[o][0][j], c1, s1);
-        un2(acc[o][1][j], c2, s2);
+        un2(acc[0][o][0][j], c1, s1);
+        un2(acc[0][o][1][j], c2, s2);
         z[2 * j] = two ? mk2(c1 + c2, c1 - c2) : mk2(c1, T(0));
         z[2 * j + 1] = two ? mk2(s1 + s2, s1 - s2) : mk2(s1, T(0));
       }
@@ -979,11 +1046,11 @@ __device__ __forceinline__ void plane_item(const Plan<T>& p, int ppc, int nparts
     }
   }
   __syncthreads();
-  rows_to_k3<T, NT, NO, k3_fields(NO, PT)>(p, sP, t0, ppc, np, sm + s.off_3b, S1);
+  rows_to_k3<T, NT, NO, k3_fields(NO, PT), k3_fields(NO, PT) == 1 ? kSplit<T> : 1>(p, sP, t0, ppc, np, sm + s.off_3b, S1);
   __syncthreads();
   T* out = P1 + ((long long)x1 * nparts + part) * NO * Kq * 4;
-  if (p.k.K2h >= 16) band_from_rows<T, NT, NO, 8>(p, S1, ppc, np, sm + s.off_2b, out);
-  else band_from_rows<T, NT, NO, 4>(p, S1, ppc, np, sm + s.off_2b, out);
+  if (p.k.K2h >= 16) band_from_rows<T, NT, NO, 8, 1>(p, S1, ppc, np, sm + s.off_2b, out);
+  else band_from_rows<T, NT, NO, 4, 1>(p, S1, ppc, np, sm + s.off_2b, out);
 }
 
 // ---- 2D problems ---------------------------------------------------------------
