@@ -195,3 +195,26 @@ def test_batch_of_deformation_contexts_equals_sequential_solves():
         assert r_b["E_final"] < r_b["E_initial"]
     for c in ctxs:
         c.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("case", CASES)
+def test_persistent_sweeps_of_the_deformation_form(case, precision):
+    """The shoot, its tangent and the backward sweep as persistent kernels beside the
+    launches of the deformation products: bit for bit the results of launches throughout."""
+    kind, Ns, Ks, seed, Nt = case
+    got = []
+    for persistent in (True, False):
+        ctx, D, v0, p = dproblem(kind, Ns, Ks, seed, Nt, precision, persistent=persistent)
+        g, Hp = _cplx(precision, v0.shape), _cplx(precision, v0.shape)
+        E = ctx.gradient(torch_dev(v0, precision), g)
+        for _ in range(2):                              # captured, then replayed
+            ctx.hessvec(torch_dev(p, precision), Hp)
+        got.append((E, host(g), host(Hp)))
+        ctx.close()
+    assert got[0][0] == got[1][0]
+    np.testing.assert_array_equal(got[0][1], got[1][1])
+    np.testing.assert_array_equal(got[0][2], got[1][2])
+    lin = D.gradient(v0)
+    assert rel_V(got[0][1], lin.g, Ks) < TOL[precision]["g"]
+    assert rel_V(got[0][2], D.hessvec(lin, p), Ks) < TOL[precision]["g"]

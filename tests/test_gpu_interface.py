@@ -84,3 +84,31 @@ def test_pi_writes_the_hermitian_array_in_its_two_kernels(Ns, Ks):
             assert rel_2(got.astype(np.complex128), bl.pi(f.astype(np.float64), Ks)) < 2e-6
             for axis, k in enumerate(Ks):
                 assert not np.take(got, k // 2, axis + 1).any()
+
+
+@pytest.mark.parametrize("state", ["image", "deformation"])
+def test_probe_changes_no_result(state):
+    """Gradient and product (captured and replayed) with every class probed and with none."""
+    import torch
+    Ns, Ks, Nt = (20, 18, 15), (8, 6, 4), 3
+    v = torch_dev(inputs.random_bl(Ks, 3, 3, 1.0, Ns), "fp32")
+    p = torch_dev(inputs.random_bl(Ks, 3, 4, 1.0, Ns), "fp32")
+    I0, I1 = (torch_dev(x, "fp32") for x in inputs.make_pair("ellipsoids", Ns, 5, max_disp=1.0))
+    with Context(Ns, Ks, ALPHA, S, SIGMA, Nt, precision="fp32", state=state) as ctx:
+        ctx.set_images(I0, I1)
+
+        def results():
+            g, h = torch.empty_like(v), torch.empty_like(v)
+            E = ctx.gradient(v, g)
+            for _ in range(2):
+                ctx.hessvec(p, h)
+            return E, g.cpu().numpy(), h.cpu().numpy()
+
+        ref = results()
+        for kernel_class in ("cpw", "pi_ba", "deform", "transport", "inc_step", "iota_full", "pi_full", "sweep"):
+            ctx.probe(kernel_class)
+            got = results()
+            ctx.probe_read()
+            assert got[0] == ref[0]
+            np.testing.assert_array_equal(got[1], ref[1])
+            np.testing.assert_array_equal(got[2], ref[2])
