@@ -570,8 +570,7 @@ def run_population(args):
     all pairs at once through lddmm_batch_gn_solve (one CUDA stream and one host
     thread per context).  The work spans 32 streams, so steps are timed by the host
     clock between device synchronisations.  Also reported: the same contexts solved
-    one after another, and the population with tensor_cores off (the same FP32
-    kernels: the two have to agree)."""
+    one after another."""
     import collections
 
     import numpy as np
@@ -583,13 +582,12 @@ def run_population(args):
         return
     pop = inputs.population()
 
-    def make(tc):
+    def make():
         made = []
         for kind, Ns, Ks, Nt, seed in pop:
             I0, I1 = inputs.make_pair(kind, Ns, seed)
             st = torch.cuda.Stream()
-            ctx = Context(Ns, Ks, ALPHA, S, SIGMA, Nt, precision="fp32", stream=st.cuda_stream,
-                          tensor_cores=tc, persistent=False)
+            ctx = Context(Ns, Ks, ALPHA, S, SIGMA, Nt, precision="fp32", stream=st.cuda_stream, persistent=False)
             I0d = torch.as_tensor(I0, dtype=torch.float32, device="cuda")
             I1d = torch.as_tensor(I1, dtype=torch.float32, device="cuda")
             torch.cuda.synchronize()
@@ -608,51 +606,17 @@ def run_population(args):
             torch.cuda.synchronize()
             t += time.perf_counter() - t0
             hv += sum(r["pcg_iters"] for r in reps)
-        return hv / t, t / steps, v0s
+        return hv / t, t / steps
 
-    # one pair of each grid and band: gradient and GN product at the pair's seeded
-    # point, for the comparison of the two settings
-    picked, seen = [], set()
-    for i, (_, Ns, Ks, _, _) in enumerate(pop):
-        if (tuple(Ns), tuple(Ks)) not in seen:
-            seen.add((tuple(Ns), tuple(Ks)))
-            picked.append(i)
-
-    def products(made):
-        out = {}
-        for i in picked:
-            _, Ns, Ks, _, seed = pop[i]
-            v0 = inputs.random_bl(Ks, 3, seed + 1, 2.0, Ns).astype(np.complex64)
-            pv = inputs.random_bl(Ks, 3, seed + 2, 1.0, Ns).astype(np.complex64)
-            g, Hp = np.empty_like(v0), np.empty_like(v0)
-            made[i][0].gradient(v0, g)
-            made[i][0].hessvec(pv, Hp)
-            out[i] = (g.astype(np.complex128), Hp.astype(np.complex128))
-        return out
-
-    def rel(a, b):
-        return float(max(np.linalg.norm((a - b).ravel()) / np.linalg.norm(b.ravel()),
-                         np.abs(a - b).max() / np.abs(b).max()))
-
-    made = make("auto")
+    made = make()
     timed(made, args.warmup, 0)
     clocks = Clocks()
-    value, step_s, v_tc = timed(made, args.steps, 0)
+    value, step_s = timed(made, args.steps, 0)
     clk = clocks.stop()
-    seq_value, _, _ = timed(made, 1, 1)
-    prod_tc = products(made)
+    seq_value, _ = timed(made, 1, 1)
     held = sum(m[0].device_bytes for m in made)
     for m in made:
         m[0].close()
-    del made
-    made = make(False)
-    timed(made, 1, 0)
-    plain_value, _, v_plain = timed(made, args.steps, 0)
-    prod_plain = products(made)
-    for m in made:
-        m[0].close()
-    # one GN step from v0 = 0 on the same images: the two settings' updates
-    diffs = [float(np.linalg.norm(a - b) / max(np.linalg.norm(b), 1e-30)) for a, b in zip(v_tc, v_plain)]
     hist = collections.Counter(f"{'x'.join(map(str, g))}/K{k[0]}" for _, g, k, _, _ in pop)
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": 1, "steps": args.steps,
@@ -660,15 +624,8 @@ def run_population(args):
         "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": "population_32", "pairs": len(pop), "grids_bands": dict(hist), "Nt": 10,
                    "pcg_per_gn": N_PCG, "step": "one GN iteration on every pair",
-                   "timer": "host clock between device synchronisations (32 streams)",
-                   "tensor_cores": "auto (transforms run in FP32)"},
+                   "timer": "host clock between device synchronisations (32 streams)"},
         "sequential_value": seq_value,
-        "plain_fp32_value": plain_value,
-        "split_vs_plain_rel_update_diff_max": max(diffs),
-        "split_vs_plain_product_rel_diff_max": {
-            "gradient": max(rel(prod_tc[i][0], prod_plain[i][0]) for i in picked),
-            "hessvec": max(rel(prod_tc[i][1], prod_plain[i][1]) for i in picked),
-            "pairs": len(picked), "measure": "larger of l2 and element-wise, one pair per grid and band"},
         "device_bytes_held": held,
         "clocks": clk,
     }
