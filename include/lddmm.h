@@ -152,16 +152,16 @@ void lddmm_default_opts(lddmm_opts* opts);
 /* Create a registration context (Section 3.2).
  *   ndim    2 or 3.
  *   grid    ndim image sizes N_j >= 2, N_1 N_2 N_3 < 2^31 (int array, host).
- *   K       ndim band sizes: even, 2 <= K_j <= N_j, K_1 <= 64 (int array, host).
+ *   K       ndim band sizes: even, 2 <= K_j <= N_j, K_1 <= 64, K_j <= 512 (int
+ *           array, host).
  *   alpha   > 0, s >= 1: L = (Id - alpha Lap)^s (Eq. 1).
  *   sigma   > 0: data weight 1/sigma^2 (Eq. 50).
  *   Nt      >= 1 time steps on [0,1].
  *   opts    NULL for defaults.
  * Allocates every device buffer the context needs (histories for Nt steps,
  * padded-grid caches, transform scratch).  Returns LDDMM_ENOMEM if the
- * device lacks memory, LDDMM_EINVAL for bad sizes (including N_3 > 1024 and
- * grids whose transform tiles exceed shared memory: N_3 above about 700 at
- * K = 32 in FP32, half that in FP64).  *out is NULL on failure. */
+ * device lacks memory, LDDMM_EINVAL for bad sizes (including N_3 > 512, K_3 > 112
+ * and sizes whose transform tiles exceed shared memory).  *out is NULL on failure. */
 int lddmm_create(lddmm_ctx** out, int ndim, const int* grid, const int* K,
                  double alpha, int s, double sigma, int Nt, const lddmm_opts* opts);
 

@@ -143,7 +143,8 @@ k_iota_band(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList<
 // k_iota_plane_even).  k3 -> x3 costs K3/2 products per point and dominates: a lane owns TL points t (and their
 // partners G3 - t) of RB rows, so a row's coefficients are read once per warp
 // (broadcast) and a twiddle once per RB rows.  Packed FMAs and shared reads bind it:
-// 306 us for 33 fields of 160x192x160 at band 32^3.
+// with k_iota_band 324 us for 33 fields of 160x192x161 at band 32^3 (247 for 160x192x160
+// in the even kernel).
 template <typename T, int TL, int RB>
 __global__ void __launch_bounds__(kImgThreads)
 k_iota_plane(const __grid_constant__ Plan<T> p, const __grid_constant__ IotaList<T> d, int ppi, const T* T1) {
@@ -928,8 +929,11 @@ void band_store(const T* in, cplx<T>* out, int ncomp, const Band& b, cudaStream_
 
 // ---- accepted sizes -----------------------------------------------------------
 // The interface takes the grids and bands whose complex half-spectrum tiles (two
-// slabs and a twiddle table per axis) fit 200 KB of shared memory, N_3 nper <= 512
-// and K_1 <= 64; every kernel above runs within that range in less.
+// slabs and a twiddle table per axis, in the item sizes below) fit 200 KB of shared
+// memory, N_3 nper <= 512 and K_1 <= 64, and lddmm_create K_j <= 512: a rule of the
+// interface, kept as it is so that the same sizes run.  Every kernel above fits kMaxSmem
+// within it (all accepted sizes evaluated: at most 224 KB in 3D, where eval_geom cuts the
+// items to fit; a whole 2D plane 75 KB, in FP64 150).
 template <typename T>
 bool sizes_accepted(const Dims& g, const Band& b, int nper, bool brackets) {
   constexpr size_t lim = 200 * 1024, C = 2 * sizeof(T);

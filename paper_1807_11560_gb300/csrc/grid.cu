@@ -3,10 +3,10 @@
 //     (Eqs. 52 and 31),
 //   * band-vector updates and deterministic FP64 reductions (Eq. 47, Eq. 50),
 //   * the deformation-state form (Section 3.3): terminal sampling of I0 at the
-//     inverse map, its force fields, and the padded-grid products of the
-//     band-limited deformation sweep.
-// One thread per grid point or band slot; the transport kernels are bound by
-// HBM traffic (coalesced streams plus an L1/L2-served 8-corner gather).
+//     inverse map and its force fields (its padded-grid products are evaluations:
+//     trig.cuh).
+// One thread per grid point or band slot; the transport kernels are bound by their
+// corner gathers (load issue and latency), beside coalesced streams.
 #include "internal.h"
 
 namespace lddmm {
@@ -136,9 +136,10 @@ k_transport(const T* __restrict__ m, const T* __restrict__ vn, const T* __restri
 // carried is the single grid q_n = dm_n - dt/2 s_n, s_n = grad m_n . dv_n:
 //   dm_{n+1} = q_n(X_n) - dt/2 s_{n+1},   q_{n+1} = q_n(X_n) - dt s_{n+1}
 // out = q(X) - c s: c = dt on the way, dt/2 for dm(1); q null: out = -c s (q_0).
-// HBM-bound with eight gathers in flight per voxel: 36 bytes are streamed (m and its
-// stencil, dv, the displacement, q read and written), 177 MB in 43 us at 160x192x160
-// (alone, cold); with dm and s carried apart, 16 gathers and 44 bytes, 50 us.
+// Bound by the eight gathers and the stencil of a voxel (load issue and latency): 36 bytes
+// are streamed (m and its stencil, dv, the displacement, q read and written), 177 MB in
+// 43 us at 160x192x160 (alone, cold), 61% of the copy rate; with dm and s carried apart,
+// 16 gathers and 44 bytes, 50 us.
 template <typename T, bool G3D>
 __global__ void __launch_bounds__(kThreads)
 k_inc_step(const T* __restrict__ q, const T* __restrict__ m, const T* __restrict__ dv, const T* __restrict__ off,

@@ -98,7 +98,7 @@ void Impl<T>::create(int nd, const int* grid, const int* band, double a, int s_,
   cuda(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "event");
 
   if (!sizes_accepted<T>(N, K, 1, false) || !sizes_accepted<T>(M, K, 3, true)) {
-    *err = "grid or band too large for the transform tiles (N_3 <= 1024, shared memory)";
+    *err = "grid or band too large for the transform tiles (N_3 <= 512, K_3 <= 112, shared memory)";
     throw Fail{LDDMM_EINVAL};
   }
   make_plan(full, N);
