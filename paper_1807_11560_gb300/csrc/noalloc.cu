@@ -32,6 +32,14 @@ struct CPlan {
   float2 *E3f, *E2f, *E1f;
 };
 
+// The kernels after the first are launched while their predecessor runs (programmatic
+// dependent launch) and wait here for its end; the first one follows the stream's earlier
+// work as usual.  What a predecessor wrote is read through plain pointers: loads through
+// const __restrict__ ones could be moved before the wait.
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 __device__ __forceinline__ bool nyq(int q, int K) { return (K % 2 == 0) && (2 * q == K); }
 __device__ __forceinline__ void cmac(float2& acc, const float2& a, const float2& e) {
   acc.x = fmaf(a.x, e.x, fmaf(-a.y, e.y, acc.x));
@@ -46,6 +54,7 @@ __host__ __device__ __forceinline__ int even_up(int n) { return n + (n & 1); }
 
 // (a(k) + conj a(-k)) / 2 with the Nyquist slots dropped
 __global__ void k_hermitianize(const float2* __restrict__ in, float2* __restrict__ out, int ncomp, Band b) {
+  chain_wait();
   const long long kvol = b.vol();
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= ncomp * kvol) return;
@@ -64,7 +73,7 @@ __global__ void k_hermitianize(const float2* __restrict__ in, float2* __restrict
 // stages A (k3 -> x3) and B (k2 -> x2) of one slab (field f, h), in 2 x 2 complex
 // register tiles; shared memory: S0 [K2][K3], S1 [K2][G3e], with TWS the twiddles
 template <bool TWS>
-__global__ void __launch_bounds__(kThr) k_slab(CPlan p, const float2* __restrict__ src0, float2* __restrict__ T2) {
+__global__ void __launch_bounds__(kThr) k_slab(CPlan p, const float2* src0, float2* T2) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int G2 = p.g.n2, G3 = p.g.n3, K2 = p.b.k2, K3 = p.b.k3, H1 = p.b.h1;
   const int G2e = even_up(G2), G3e = even_up(G3);
@@ -74,6 +83,7 @@ __global__ void __launch_bounds__(kThr) k_slab(CPlan p, const float2* __restrict
   float2* E3s = S1 + K2 * G3e;
   float2* E2s = E3s + K3 * G3e;
   const float2 zero = make_float2(0.f, 0.f);
+  chain_wait();
   if (TWS) {
     for (int i = tid; i < K3 * G3e; i += kThr) {
       const int r = i / G3e, x = i - r * G3e;
@@ -84,7 +94,7 @@ __global__ void __launch_bounds__(kThr) k_slab(CPlan p, const float2* __restrict
       E2s[i] = x < G2 ? p.E2f[r * G2 + x] : zero;
     }
   }
-  const float2* __restrict__ src = src0 + (long long)f * p.b.vol() + (long long)h * K2 * K3;
+  const float2* src = src0 + (long long)f * p.b.vol() + (long long)h * K2 * K3;
   for (int i = tid; i < K2 * K3; i += kThr) S0[i] = src[i];
   __syncthreads();
   const int n3p = G3e / 2, n2p = G2e / 2;
@@ -138,20 +148,21 @@ __global__ void __launch_bounds__(kThr) k_slab(CPlan p, const float2* __restrict
 // stage C: each thread holds the H1 coefficients of one (x2, x3) position and
 // walks all x1
 template <int HR>
-__global__ void __launch_bounds__(kThr) k_pencil(CPlan p, const float2* __restrict__ T2, float* __restrict__ f_out) {
+__global__ void __launch_bounds__(kThr) k_pencil(CPlan p, const float2* T2, float* __restrict__ f_out) {
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sE = reinterpret_cast<float2*>(smraw);           // [G1][H1]
   const int G1 = p.g.n1, H1 = p.b.h1;
   const long long inner = (long long)p.g.n2 * p.g.n3, nblk = (inner + kThr - 1) / kThr;
   const int f = (int)(blockIdx.x / nblk);
   const long long i = (blockIdx.x % nblk) * kThr + threadIdx.x;
+  chain_wait();
   for (int j = threadIdx.x; j < H1 * G1; j += kThr) {
     const int x = j / H1, h = j - x * H1;
     sE[j] = p.E1f[h * G1 + x];
   }
   float2 a[HR];
   const bool live = i < inner;
-  const float2* __restrict__ src = T2 + (long long)f * H1 * inner + i;
+  const float2* src = T2 + (long long)f * H1 * inner + i;
 #pragma unroll
   for (int h = 0; h < HR; ++h) a[h] = (live && h < H1) ? src[(long long)h * inner] : make_float2(0.f, 0.f);
   __syncthreads();
@@ -169,15 +180,20 @@ __global__ void __launch_bounds__(kThr) k_pencil(CPlan p, const float2* __restri
   }
 }
 
-template <typename K>
-void run(K kern, unsigned grid, size_t smem, cudaStream_t st, CPlan p, const float2* a, float2* T2) {
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-  kern<<<grid, kThr, smem, st>>>(p, a, T2);
-}
-template <typename K>
-void run(K kern, unsigned grid, size_t smem, cudaStream_t st, CPlan p, const float2* T2, float* out) {
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-  kern<<<grid, kThr, smem, st>>>(p, T2, out);
+template <typename... KArgs, typename... Args>
+cudaError_t run(void (*kern)(KArgs...), long long grid, size_t smem, cudaStream_t st, Args... args) {
+  // large items start as the predecessor ends: early ones would share the few SMs then free
+  const bool large = smem > 32 * 1024;
+  if (large) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kThr);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  cfg.attrs = at;
+  cfg.numAttrs = large ? 0 : chain_attrs(at);
+  return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
 }
 
 // Fixed scratch: every GPU that loads this library holds it until exit.
@@ -292,18 +308,20 @@ extern "C" int lddmm_iota_noalloc(int ndim, const int* grid, const int* K, const
   const long long ntw = (long long)b.k3 * N.n3 + (long long)b.k2 * N.n2 + (long long)b.h1 * N.n1;
   k_iota_twiddles<<<(unsigned)((ntw + 255) / 256), 256, 0, st>>>(p.E3f, p.E2f, p.E1f, b, N);
   const long long nb = (long long)ncomp * b.vol();
-  k_hermitianize<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(static_cast<const float2*>(a), herm, ncomp, b);
   if (cudaGetLastError() != cudaSuccess) return LDDMM_ECUDA;   // nothing further is enqueued
+  const float2* in = static_cast<const float2*>(a);
+  cudaError_t e = run(k_hermitianize, (nb + kThr - 1) / kThr, 0, st, in, herm, ncomp, b);
   const size_t G2e = even_up(N.n2), G3e = even_up(N.n3);
   const size_t s0 = ((size_t)even_up(b.k2 * b.k3) + b.k2 * G3e) * c8, tw = (b.k3 * G3e + b.k2 * G2e) * c8;
-  const unsigned slabs = (unsigned)(ncomp * b.h1);
-  if (s0 + tw <= (size_t)64 * 1024) run(k_slab<true>, slabs, s0 + tw, st, p, herm, T2);
-  else run(k_slab<false>, slabs, s0, st, p, herm, T2);
-  const unsigned pencils = (unsigned)(ncomp * (((long long)N.n2 * N.n3 + kThr - 1) / kThr));
+  const long long slabs = (long long)ncomp * b.h1, pencils = ncomp * (((long long)N.n2 * N.n3 + kThr - 1) / kThr);
+  if (e == cudaSuccess)
+    e = s0 + tw <= (size_t)64 * 1024 ? run(k_slab<true>, slabs, s0 + tw, st, p, herm, T2)
+                                     : run(k_slab<false>, slabs, s0, st, p, herm, T2);
   const size_t se = (size_t)b.h1 * N.n1 * c8;
   float* out = static_cast<float*>(f_out);
-  if (b.h1 <= 8) run(k_pencil<8>, pencils, se, st, p, T2, out);
-  else if (b.h1 <= 16) run(k_pencil<16>, pencils, se, st, p, T2, out);
-  else run(k_pencil<kMaxH1>, pencils, se, st, p, T2, out);
+  if (e == cudaSuccess)
+    e = b.h1 <= 8 ? run(k_pencil<8>, pencils, se, st, p, T2, out)
+                  : (b.h1 <= 16 ? run(k_pencil<16>, pencils, se, st, p, T2, out)
+                                : run(k_pencil<kMaxH1>, pencils, se, st, p, T2, out));
   return cudaGetLastError() == cudaSuccess ? LDDMM_OK : LDDMM_ECUDA;
 }

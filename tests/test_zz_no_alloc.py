@@ -100,3 +100,24 @@ def test_noalloc_binding_checks_extents():
         lddmm.iota_noalloc((16, 16, 16), (8, 8, 8), a, 3, out[:2])
     with pytest.raises(ValueError):
         lddmm.iota_noalloc((16, 16, 16), (8, 8), a, 3, out)
+
+
+@pytest.mark.parametrize("Ns,Ks", [((32, 32, 32), (8, 8, 8)), ((64, 64, 64), (32, 32, 32)), ((48, 48, 49), (16, 48, 48))])
+def test_noalloc_calls_in_a_row_keep_their_order(Ns, Ks):
+    """The kernels of a call overlap their predecessors' ends (small items and large
+    ones), and a call follows the one before on the same scratch without a
+    synchronisation: every result is its own input's."""
+    import torch
+    stream = torch.cuda.current_stream().cuda_stream
+    a = [torch.as_tensor(inputs.random_bl(Ks, 3, seed, 2.0, Ns), dtype=torch.complex64, device="cuda")
+         for seed in range(6)]
+    out = [torch.full((3,) + Ns, float("nan"), dtype=torch.float32, device="cuda") for _ in a]
+    torch.cuda.synchronize()
+    for x, y in zip(a, out):
+        assert lddmm.iota_noalloc(Ns, Ks, x, 3, y, stream) == 0
+    torch.cuda.synchronize()
+    with Context(Ns, Ks, ALPHA, S, SIGMA, 2, precision="fp32") as ctx:
+        ref = torch.empty((3,) + Ns, dtype=torch.float32, device="cuda")
+        for x, y in zip(a, out):
+            ctx.iota(x, 3, ref)
+            assert _rel(y.cpu().numpy(), ref.cpu().numpy()) < TOL
