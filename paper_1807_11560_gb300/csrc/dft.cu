@@ -93,7 +93,7 @@ k_plane(const __grid_constant__ Plan<T> p, int ppc, int nparts, const T* T1, T* 
 }
 
 // The plane phase of a 2D problem: latency, and in FP64 the double pipe (a product of
-// the 64^2 / 16^2 configuration, 40 evaluations: 1.02 ms; 2.5 ms with complex
+// the 64^2 / 16^2 configuration, 40 evaluations: 0.98 ms; 2.5 ms with complex
 // half-spectrum sums).
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kPhaseThreads)
@@ -358,7 +358,7 @@ __device__ __forceinline__ void pi_plane_part(const Plan<T>& p, const PiField<T>
 }
 
 // pi of `ppi` row pairs of one x1 plane of one field.  The row loads (six
-// neighbours a point for the terminal fields) and the packed FMAs bind it: 72-80 us for
+// neighbours a point for the terminal fields) and the packed FMAs bind it: 63-79 us for
 // three terminal fields of 160x192x160, band 32^3, where a pass that formed the fields
 // (25 us) and the transform's plane kernels (95 us) ran before.
 template <typename T, int KIND>
@@ -483,7 +483,7 @@ __device__ __forceinline__ cplx<T> hermitian_value(const int* f, const bool* neg
 }
 
 // x1 -> k1 of the nf projected planes of image-grid fields and their scaling:
-// (14 us for 160 planes of three fields, band 32^3: latency and L2 reads)
+// (13 us for 160 planes of three fields, band 32^3: latency and L2 reads)
 // coef * (applyK ? 1/L^ : 1) * the sums (twice per axis of nonzero frequency), as band
 // vectors out, or with HERM as the Hermitian arrays herm.  A quad holds every sign of its
 // frequencies (the Nyquist slots stand where the negative of a zero would), so an item
